@@ -174,12 +174,21 @@ size_t col_elems(const cip_plan* p, int planes) {
 }
 size_t real_elems(const cip_plan* p, int maps) { return (size_t)maps * p->N * p->N; }
 
+// orthonormal 8-point DCT-II, computed once per process: every prior-pass launch carries a copy, and
+// 64 cosines per launch cost the host more than the launch of a small plan's kernel
 template <typename T> void fill_dct(T* d) {
-  for (int k = 0; k < 8; ++k)
-    for (int n = 0; n < 8; ++n) {
-      const double a = k == 0 ? std::sqrt(1.0 / 8.0) : std::sqrt(2.0 / 8.0);
-      d[k * 8 + n] = (T)(a * std::cos(M_PI * (2 * n + 1) * k / 16.0));
+  struct Table {
+    T v[64];
+    Table() {
+      for (int k = 0; k < 8; ++k)
+        for (int n = 0; n < 8; ++n) {
+          const double a = k == 0 ? std::sqrt(1.0 / 8.0) : std::sqrt(2.0 / 8.0);
+          v[k * 8 + n] = (T)(a * std::cos(M_PI * (2 * n + 1) * k / 16.0));
+        }
     }
+  };
+  static const Table t;
+  std::memcpy(d, t.v, sizeof(t.v));
 }
 
 // exp(-2 pi i k / 2048) with the angle reduced exactly through octant symmetry
@@ -715,8 +724,9 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
 }
 
 std::mutex g_tune_mu;
-// (N, M, dtype, prior) -> (column-pass form, fused tile width, prior-pass variant)
-using TuneKey = std::tuple<int, int, int, int>;
+// (N, M, dtype, prior, forced prior-pass variant or -1) -> (column-pass form, fused tile width,
+// prior-pass variant)
+using TuneKey = std::tuple<int, int, int, int, int>;
 using TuneVal = std::tuple<int, int, int>;
 std::map<TuneKey, TuneVal> g_tune;
 bool g_tune_loaded = false;
@@ -731,11 +741,11 @@ void tune_cache_load() {
   if (!path || !*path) return;
   std::ifstream in(path);
   int n, m, dt, pr, mode, cc, av;
-  while (in >> n >> m >> dt >> pr >> mode >> cc >> av) g_tune[std::make_tuple(n, m, dt, pr)] = {mode, cc, av};
+  while (in >> n >> m >> dt >> pr >> mode >> cc >> av) g_tune[std::make_tuple(n, m, dt, pr, -1)] = {mode, cc, av};
 }
 void tune_cache_store(const TuneKey& key, const TuneVal& v) {
   const char* path = std::getenv("CIP_TUNE_CACHE");
-  if (!path || !*path) return;
+  if (!path || !*path || std::get<4>(key) >= 0) return;  // the file holds unforced decisions only
   std::ofstream out(path, std::ios::app);
   out << std::get<0>(key) << ' ' << std::get<1>(key) << ' ' << std::get<2>(key) << ' ' << std::get<3>(key) << ' '
       << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << '\n';
@@ -767,19 +777,22 @@ template <typename T> void set_colmode(cip_plan* p, int mode, int cc) {
 // Autotuner: times whole iterations (column pass, then prior pass, launched back to back as in
 // cip_iterate) for every column-pass form (fused kernel; split FFT / solve / FFT) and both
 // prior-pass FFT widths where a variant exists, on this plan's buffers, and keeps the fastest,
-// cached per (N, M, dtype, prior) for the process.  The prior pass reads u[cur] and writes the
+// cached per (N, M, dtype, prior, forced width) for the process: plans with one width (wavelet
+// prior, complex128, N < 256, N = 2048) and plans with a forced one time their candidates once as
+// well, not at every cip_set_measurements (14 to 28 iterations and the event waits between them:
+// 2.5 ms of the 8.6 ms of a 40-iteration 512 x 512 x 10 wavelet reconstruction).  The prior pass reads u[cur] and writes the
 // other u buffer and q-hat without moving cur, so repeating an iteration keeps its inputs; the
 // state is reset afterwards (cip_set_measurements).
 template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   using C = typename CT<T>::type;
-  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior);
+  const int fav = forced_avar(p);
+  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, prior_has_variant(p) ? fav : -1);
   if (low_fix(p)) {  // the low-column correction of large TV plans is part of the split form
     set_colmode<T>(p, 2, p->cc);
     if (!p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));
     return CIP_OK;
   }
-  const int fav = forced_avar(p);
-  if (fav < 0) {
+  {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_cache_load();
     auto it = g_tune.find(key);
@@ -834,7 +847,6 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   cudaEventDestroy(e1);
   set_colmode<T>(p, std::get<0>(pick), std::get<1>(pick));
   p->avar = std::get<2>(pick);
-  if (fav >= 0) return CIP_OK;  // a forced width is not the autotuner's decision: not cached
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune[key] = pick;
   tune_cache_store(key, pick);
