@@ -8,7 +8,7 @@
 //     packed triangle of each bin in shared memory.  Bins where g(w) = 0 (the
 //     DC bin of TV, singular when the PSFs have unit sum) or where the
 //     factorisation fails get the min-norm pseudo-inverse from a cyclic Jacobi
-//     eigendecomposition of the real 2M x 2M embedding of Psi in FP64
+//     eigendecomposition of the Hermitian Psi in FP64
 //     (eigenvalues below 1e-10 of the largest dropped).  Results are scaled by
 //     1/N^2 (the inverse-DFT normalisation) and rounded once to the plan's
 //     precision, packed as the upper triangle row by row; a setup-precision
@@ -347,86 +347,146 @@ __global__ void __launch_bounds__(32 * kFacWarps) factor_warp_kernel(const Setup
   }
 }
 
-// Min-norm pseudo-inverse at the listed bins (one thread per bin).
+// Min-norm pseudo-inverse at the listed bins, one warp per bin: cyclic Jacobi on the complex
+// Hermitian Psi in FP64, in shared memory.  The rounds of a sweep follow the round-robin schedule,
+// so the up to M/2 rotations of a round touch disjoint index pairs: lanes 0 .. M/2 - 1 form them,
+// then all lanes apply them to the columns of A and V and to the rows of A.
+// Usually a single bin is listed (DC of TV), so this is one serial chain that nothing overlaps and
+// its latency adds to every factor formation.  The first form (one thread, the real 2M x 2M
+// embedding in local memory) took 82 / 270 / 908 us at M = 3 / 5 / 10 before every change of rho;
+// this one 21 / 29 / 92 us (unit-sum PSFs).
 template <typename Tout>
-__global__ void factor_pinv_kernel(const SetupC<Tout>* __restrict__ lam, const double* __restrict__ gs, int use_g,
-                                   int K, int M, int N, double rho, double beta,
-                                   typename CT<Tout>::type* __restrict__ pinv, SetupC<Tout>* __restrict__ pinv64,
-                                   const int* list, int cap) {
+__global__ void __launch_bounds__(32) factor_pinv_kernel(const SetupC<Tout>* __restrict__ lam,
+                                                         const double* __restrict__ gs, int use_g, int K, int M,
+                                                         int N, double rho, double beta,
+                                                         typename CT<Tout>::type* __restrict__ pinv,
+                                                         SetupC<Tout>* __restrict__ pinv64, const int* list, int cap) {
   using C = typename CT<Tout>::type;
+  __shared__ double2 A[kMaxM][kMaxM + 1], V[kMaxM][kMaxM + 1];
+  __shared__ double rc[kMaxM / 2], rs[kMaxM / 2];  // rotation of each pair: cosine, sine
+  __shared__ double2 rp[kMaxM / 2];                // and exp(-i arg A_pq)
   const int n = min(list[0], cap);
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
+  if ((int)blockIdx.x >= n) return;
+  const int lane = threadIdx.x;
   const int H = N / 2 + 1, P = half_pitch(N);
-  const int bin = list[1 + t];
+  const int bin = list[1 + blockIdx.x];
   const int k1 = bin / H, k2 = bin - k1 * H;
   const size_t off = (size_t)k1 * P + k2, mplane = (size_t)N * P;
   const double g = bin_g(gs, use_g, k1, k2);
-  const int D = 2 * M;
-  double A[2 * kMaxM][2 * kMaxM], V[2 * kMaxM][2 * kMaxM];
-  for (int i = 0; i < M; ++i) {
-    for (int j = 0; j <= i; ++j) {
-      const double2 p = psi_entry(lam, off, mplane, K, M, i, j, rho * g, beta);
-      // Psi_ij = p (i >= j), Psi_ji = conj(p); embedding [[B, -C], [C, B]]
-      A[i][j] = p.x; A[M + i][M + j] = p.x; A[M + i][j] = p.y; A[i][M + j] = -p.y;
-      A[j][i] = p.x; A[M + j][M + i] = p.x; A[M + j][i] = -p.y; A[j][M + i] = p.y;
-    }
+  const int MM = M * M;
+  for (int e = lane; e < MM; e += 32) {
+    const int i = e / M, j = e - i * M;
+    V[i][j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
+    if (j > i) continue;
+    const double2 p = psi_entry(lam, off, mplane, K, M, i, j, rho * g, beta);
+    A[i][j] = p;
+    if (i != j) A[j][i] = make_double2(p.x, -p.y);
   }
-  for (int i = 0; i < D; ++i)
-    for (int j = 0; j < D; ++j) V[i][j] = (i == j) ? 1.0 : 0.0;
-  double fro = 0.0;
-  for (int i = 0; i < D; ++i)
-    for (int j = 0; j < D; ++j) fro += A[i][j] * A[i][j];
+  __syncwarp();
+  auto sum_sq = [&](bool off_only) {
+    double t = 0.0;
+    for (int e = lane; e < MM; e += 32) {
+      const int i = e / M, j = e - i * M;
+      if (!off_only || i != j) t += A[i][j].x * A[i][j].x + A[i][j].y * A[i][j].y;
+    }
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+  };
+  const double fro = sum_sq(false);
+  const int Me = M + (M & 1), rounds = Me - 1, npair = Me / 2;  // odd M: one index sits out a round
+  // round-robin: index Me - 1 stays, the others rotate; pair 0 is (Me - 1, r)
+  auto pair_of = [&](int r, int i, int& p, int& q) {
+    const int a = i == 0 ? Me - 1 : (r + i) % (Me - 1), b = i == 0 ? r : (r + Me - 1 - i) % (Me - 1);
+    p = a < b ? a : b;
+    q = a < b ? b : a;
+  };
   for (int sweep = 0; sweep < 60; ++sweep) {
-    double off2 = 0.0;
-    for (int p = 0; p < D; ++p)
-      for (int q = p + 1; q < D; ++q) off2 += A[p][q] * A[p][q];
-    if (off2 <= 1e-32 * fro || off2 == 0.0) break;
-    for (int p = 0; p < D; ++p) {
-      for (int q = p + 1; q < D; ++q) {
-        const double apq = A[p][q];
-        if (apq == 0.0) continue;
-        const double theta = (A[q][q] - A[p][p]) / (2.0 * apq);
-        const double tt = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-        const double c = 1.0 / sqrt(tt * tt + 1.0), s = tt * c;
-        for (int k = 0; k < D; ++k) {
-          const double akp = A[k][p], akq = A[k][q];
-          A[k][p] = c * akp - s * akq;
-          A[k][q] = s * akp + c * akq;
+    const double off2 = sum_sq(true);
+    if (off2 <= 1e-32 * fro) break;
+    for (int r = 0; r < rounds; ++r) {
+      if (lane < npair) {
+        int p, q;
+        pair_of(r, lane, p, q);
+        double c = 1.0, s = 0.0;
+        double2 ph = make_double2(1.0, 0.0);
+        if (q < M) {
+          const double2 apq = A[p][q];
+          const double n2 = apq.x * apq.x + apq.y * apq.y;
+          if (n2 > 0.0) {
+            const double ri = rsqrt(n2);  // 1 / |A_pq|
+            const double theta = 0.5 * (A[q][q].x - A[p][p].x) * ri;
+            const double tt = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+            c = rsqrt(tt * tt + 1.0);
+            s = tt * c;
+            ph = make_double2(apq.x * ri, -apq.y * ri);
+          }
         }
-        for (int k = 0; k < D; ++k) {
-          const double apk = A[p][k], aqk = A[q][k];
-          A[p][k] = c * apk - s * aqk;
-          A[q][k] = s * apk + c * aqk;
-        }
-        for (int k = 0; k < D; ++k) {
-          const double vkp = V[k][p], vkq = V[k][q];
-          V[k][p] = c * vkp - s * vkq;
-          V[k][q] = s * vkp + c * vkq;
-        }
+        rc[lane] = c;
+        rs[lane] = s;
+        rp[lane] = ph;
       }
+      __syncwarp();
+      // columns p, q of A (x < M) and of V (x >= M)
+      for (int e = lane; e < 2 * M * npair; e += 32) {
+        const int i = e / (2 * M), x = e - i * 2 * M;
+        int p, q;
+        pair_of(r, i, p, q);
+        if (q >= M || rs[i] == 0.0) continue;
+        double2* row = x < M ? A[x] : V[x - M];
+        const double c = rc[i], s = rs[i];
+        const double2 u = row[p], v = cmul(rp[i], row[q]);
+        row[p] = make_double2(c * u.x - s * v.x, c * u.y - s * v.y);
+        row[q] = make_double2(s * u.x + c * v.x, s * u.y + c * v.y);
+      }
+      __syncwarp();
+      // rows p, q of A; the annihilated entries and the imaginary parts of the diagonal are exact zeros
+      for (int e = lane; e < M * npair; e += 32) {
+        const int i = e / M, x = e - i * M;
+        int p, q;
+        pair_of(r, i, p, q);
+        if (q >= M || rs[i] == 0.0) continue;
+        const double c = rc[i], s = rs[i];
+        const double2 u = A[p][x], v = cmulc(rp[i], A[q][x]);
+        double2 a = make_double2(c * u.x - s * v.x, c * u.y - s * v.y);
+        double2 b = make_double2(s * u.x + c * v.x, s * u.y + c * v.y);
+        if (x == p) {
+          a.y = 0.0;
+          b = make_double2(0.0, 0.0);
+        } else if (x == q) {
+          b.y = 0.0;
+          a = make_double2(0.0, 0.0);
+        }
+        A[p][x] = a;
+        A[q][x] = b;
+      }
+      __syncwarp();
     }
   }
   double emax = 0.0;
-  for (int i = 0; i < D; ++i) emax = fmax(emax, A[i][i]);
+  for (int i = 0; i < M; ++i) emax = fmax(emax, A[i][i].x);
   const double cut = 1e-10 * emax;
   const double sc = 1.0 / ((double)N * (double)N);
-  int pk = 0;
-  for (int i = 0; i < M; ++i) {
-    for (int j = i; j < M; ++j) {
-      double re = 0.0, im = 0.0;
-      for (int e = 0; e < D; ++e) {
-        const double d = A[e][e];
-        if (d > cut) {
-          re += V[i][e] * V[j][e] / d;
-          im += V[M + i][e] * V[j][e] / d;
-        }
-      }
-      if (i == j) im = 0.0;
-      pinv[binp(k2, pk, k1, M * (M + 1) / 2, N)] = mk<C>(re * sc, im * sc);
-      if (pinv64) pinv64[(size_t)pk * mplane + off] = cconv<SetupC<Tout>>(make_double2(re * sc, im * sc));
-      ++pk;
+  // Psi^+ = sum_e V_e V_e^H / d_e over the kept eigenvalues, packed upper row by row
+  const int npk = M * (M + 1) / 2;
+  for (int pk = lane; pk < npk; pk += 32) {
+    int i = 0, rem = pk;
+    while (rem >= M - i) {
+      rem -= M - i;
+      ++i;
     }
+    const int j = i + rem;
+    double re = 0.0, im = 0.0;
+    for (int e = 0; e < M; ++e) {
+      const double d = A[e][e].x;
+      if (d > cut) {
+        const double2 a = V[i][e], b = V[j][e];
+        re += (a.x * b.x + a.y * b.y) / d;
+        im += (a.y * b.x - a.x * b.y) / d;
+      }
+    }
+    if (i == j) im = 0.0;
+    pinv[binp(k2, pk, k1, npk, N)] = mk<C>(re * sc, im * sc);
+    if (pinv64) pinv64[(size_t)pk * mplane + off] = cconv<SetupC<Tout>>(make_double2(re * sc, im * sc));
   }
 }
 
@@ -558,7 +618,7 @@ cudaError_t launch_factor_pinv(const SetupC<Tout>* lam, const double* gs, int us
                                double beta, typename CT<Tout>::type* pinv, SetupC<Tout>* pinv64, const int* pinv_list,
                                int list_cap, cudaStream_t s) {
   if (M > kMaxM) return cudaErrorInvalidValue;
-  factor_pinv_kernel<Tout><<<(list_cap + 31) / 32, 32, 0, s>>>(lam, gs, use_g, K, M, N, rho, beta, pinv, pinv64,
+  factor_pinv_kernel<Tout><<<list_cap, 32, 0, s>>>(lam, gs, use_g, K, M, N, rho, beta, pinv, pinv64,
                                                                pinv_list, list_cap);
   return cudaGetLastError();
 }
