@@ -15,6 +15,8 @@
 //      the row half-spectra that pass B turns into the full 2D DFT.
 // Optionally it stores t (for the next iteration's dual residual) and writes
 // per-CTA partial sums of the residual norms (Eq. paramS quantities).
+#include <type_traits>
+
 #include "fft.cuh"
 #include "kernels.h"
 
@@ -24,6 +26,9 @@ namespace {
 
 #ifndef PASSA_RT32
 #define PASSA_RT32 48
+#endif
+#ifndef PASSA_TV_RT32
+#define PASSA_TV_RT32 64
 #endif
 
 template <typename T>
@@ -73,16 +78,24 @@ template <typename T> constexpr bool has_variant(int N, int prior) {
 constexpr int zs_of(int N) { return spad(N) + (N >= 256 ? 4 : 0); }
 
 // rows per tile
-template <typename T> constexpr int rows_for(int N, int prior) {
-  if (!prior_is_tv(prior)) return 8;
-  using C = typename CT<T>::type;
-  for (int R = 8; R >= 2; R /= 2) {
-    size_t zs = (size_t)zs_of(N);
-    size_t sm = (size_t)((R + 2) / 2) * zs * sizeof(C) + (size_t)(2 * R + 1) * N * sizeof(T);
-    if (sm <= 200 * 1024) return R;
-  }
-  return 2;
-}
+template <typename T> constexpr int rows_for(int N, int prior) { return 8; }
+
+// TV work split of the shrinkage phase.  A thread works on two adjacent columns and walks down
+// rows, keeping the row above in registers, so the tile needs no shared-memory copy of the
+// components of t - u: the phase costs 3 shared-memory loads per row pair and column pair, and the
+// CTA's shared memory is the FFT buffers alone.  a_h of the column to the left comes from the next
+// lane down; the values that cross a warp's 64 columns are formed once, ahead of the walk.
+//   N <= 512: row groups of tv_rows() rows side by side, one column pair per thread; q stays in
+//     registers until every thread has read the x tile (it is written in place).  A group recomputes
+//     a_v of the row above it, so groups are as tall as they can be with most threads busy.
+//   N >= 1024: every thread walks down all rows of its column pairs; q of a row pair is written over
+//     the x rows that no later row needs, one barrier per row pair.
+// Bound by the latency of its phases (long-scoreboard and barrier stalls; FFT shared-memory traffic
+// 45-50% of the LSU pipe).  The prior pass alone, before (components of t - u in shared memory, 2 to
+// 8-row tiles, u read where it is used) and now: 64^2 x 3 10.3 -> 8.0 us, 256^2 x 3 14.3 -> 9.8,
+// 512^2 x 5 22.1 -> 17.5, 512^2 x 10 37.3 -> 26.5, 1024^2 x 10 125 -> 99, 2048^2 x 3 286 -> 168 us;
+// isotropic 512^2 x 10 39.2 -> 30.2, 2048^2 x 3 302 -> 191 us.
+constexpr int tv_rows(int N) { return N >= 512 ? 8 : (N >= 256 ? 4 : 2); }
 
 // DCT and l1 tiles stage their R rows of u in shared memory with one TMA bulk
 // copy issued before the grid dependency (u does not depend on the preceding
@@ -93,27 +106,35 @@ template <typename T> constexpr bool u_staged(int N, int prior, int R) {
          (size_t)(R / 2) * zs_of(N) * sizeof(C) + (size_t)R * N * sizeof(T) <= 100 * 1024;
 }
 
+// TV tiles up to N = 512 stage theirs too: R + 1 rows (the row above included) of both components,
+// so that the u reads, which every thread needs in one burst, cost no global latency after the FFTs
+template <typename T> constexpr bool tv_staged(int N, int prior) {
+  return sizeof(T) == 4 && prior_is_tv(prior) && N <= 512;
+}
+
 template <typename T> constexpr size_t smem_for(int N, int prior, int R) {
   using C = typename CT<T>::type;
   const int halo = prior_is_tv(prior) ? 1 : 0;
   size_t sm = (size_t)((R + 2 * halo) / 2) * zs_of(N) * sizeof(C);
-  if (prior_is_tv(prior)) sm += (size_t)(2 * R + 1) * N * sizeof(T);
   if (u_staged<T>(N, prior, R)) sm += (size_t)R * N * sizeof(T);
+  if (tv_staged<T>(N, prior)) sm += 2 * (size_t)(R + 1) * N * sizeof(T);
   return sm;
 }
 
+// The TV CTAs of small images get threads beyond the FFT teams for the other phases (a row group's
+// threads are then whole warps).
 template <typename T> constexpr int threads_for(int N, int prior, int R, int V = 0) {
   const int npin = (R + (prior_is_tv(prior) ? 2 : 0)) / 2;
-  const int n = npin * (N / elems_a<T>(N, prior, V));
-  return ((n + 31) / 32) * 32;
+  const int n = ((npin * (N / elems_a<T>(N, prior, V)) + 31) / 32) * 32;
+  return prior_is_tv(prior) && n < 256 ? 256 : n;
 }
 
 // CTAs per SM the register budget is cut for: as many as shared memory and the
 // thread limit allow, at <= ~48 registers per thread for complex64 (so that a
 // 10-channel 512 x 512 prior pass runs as one wave) and <= ~168 for complex128
 // (whose 16-element FFT registers would otherwise spill).
-template <typename T> constexpr int minblocks_for(int nth, size_t smem) {
-  const int by_regs = 65536 / (nth * (sizeof(T) == 4 ? PASSA_RT32 : 168));
+template <typename T> constexpr int minblocks_for(int nth, size_t smem, bool tv) {
+  const int by_regs = 65536 / (nth * (sizeof(T) == 4 ? (tv ? PASSA_TV_RT32 : PASSA_RT32) : 168));
   const int by_smem = (int)((227 * 1024) / (smem + 1024));
   const int by_thr = 2048 / nth;
   int b = by_regs < by_smem ? by_regs : by_smem;
@@ -206,10 +227,33 @@ __device__ __forceinline__ void acc_resid(T (&part)[kNPart], T w, T t, T un, con
   }
 }
 
+// sums of 16 values per lane over the warp by recursive halving: at xor distance 16, 8, 4, 2 a lane
+// keeps one half of its values (the upper half when that bit of the lane is set) and adds its
+// partner's; then v[0] of lane l is the warp's sum of value l >> 1
+template <typename T> __device__ __forceinline__ void reduce_scatter16(T* v, int lane) {
+#pragma unroll
+  for (int live = 16, o = 16; live > 1; live /= 2, o /= 2) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < live / 2; ++i) {
+      const T keep = up ? v[i + live / 2] : v[i], send = up ? v[i] : v[i + live / 2];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// products and differences that the compiler must not contract: the isotropic shrinkage spells its
+// roundings out, so that every place that forms a pixel's components gets the same bits
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+
 template <typename T, int LOGN, int PRIOR, int R, int V>
 __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
                                   minblocks_for<T>(threads_for<T>(1 << LOGN, PRIOR, R, V),
-                                                   smem_for<T>(1 << LOGN, PRIOR, R)))
+                                                   smem_for<T>(1 << LOGN, PRIOR, R), prior_is_tv(PRIOR)))
     passA_kernel(const PassAArgs<T> a) {
   using C = typename CT<T>::type;
   constexpr int N = 1 << LOGN;
@@ -223,13 +267,18 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
   constexpr int E = elems_a<T>(N, PRIOR, V);
   constexpr int TEAM = N / E;
   constexpr int NCOMP = prior_is_tv(PRIOR) ? 2 : 1;
+  constexpr int NT = threads_for<T>(N, PRIOR, R, V);
+  static_assert(kLowK == 2, "the TV walk forms k2 = 0 and 1");
+  __shared__ T edge[R][prior_is_tv(PRIOR) ? N / 64 : 1];
+  __shared__ T lows[2][prior_is_tv(PRIOR) && LOGN == 11 ? NT / 32 : 1][12];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* zb = reinterpret_cast<C*>(smem_raw);
-  T* ah = reinterpret_cast<T*>(zb + NPIN * ZS);  // TV only: [R][N], a_h at tile rows 1..R
-  T* av = ah + R * N;                             // TV only: [R+1][N], a_v at tile rows 0..R
   constexpr bool USTAGE = u_staged<T>(N, PRIOR, R);
   static_assert(!USTAGE || (NPIN * ZS * sizeof(C)) % 16 == 0, "the TMA destination must be 16-byte aligned");
-  T* us = reinterpret_cast<T*>(zb + NPIN * ZS);   // DCT / l1 with USTAGE: [R][N] rows r0.. of u_in
+  constexpr bool TVSTAGE = tv_staged<T>(N, PRIOR);
+  static_assert(!TVSTAGE || (NPIN * ZS * sizeof(C)) % 16 == 0, "the TMA destination must be 16-byte aligned");
+  // USTAGE: [R][N] rows r0 .. of u_in; TVSTAGE: [2][R + 1][N] rows r0 - 1 .. of both components
+  T* us = reinterpret_cast<T*>(zb + NPIN * ZS);
   __shared__ unsigned long long ubar;
 
   const int tid = threadIdx.x;
@@ -254,6 +303,14 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
 
   auto grow = [&](int j) { return (r0 - HALO + j) & (N - 1); };
 
+  auto stage_tv = [&]() {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      T* dst = us + c * (R + 1) * N;
+      bulk_copy_g2s(dst, u_in + c * plane + (size_t)grow(0) * N, (unsigned)(N * sizeof(T)), &ubar);
+      bulk_copy_g2s(dst + N, u_in + c * plane + (size_t)r0 * N, (unsigned)(R * N * sizeof(T)), &ubar);
+    }
+  };
   if constexpr (USTAGE) {
     // u rows r0 .. r0+R-1 of this channel: one contiguous block (16-byte aligned: r0 is a
     // multiple of 8 and N >= 64), fetched by the TMA unit while the previous kernel drains
@@ -267,13 +324,22 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
       } else {
         mbar_init(&ubar, 1);
         mbar_arrive_expect_tx(&ubar, bytes);
-        bulk_copy_g2s(us, u_in + (size_t)r0 * N, bytes, &ubar);
+        if (!import_mode) bulk_copy_g2s(us, u_in + (size_t)r0 * N, bytes, &ubar);
       }
     }
     __syncthreads();  // the barrier is initialised before anyone waits on it
   }
+  if constexpr (TVSTAGE) {
+    // per component the row above the tile (wraps to the last row) and the tile's R rows
+    if (tid == 0) {
+      mbar_init(&ubar, 1);
+      mbar_arrive_expect_tx(&ubar, (unsigned)(2 * (R + 1) * N * sizeof(T)));
+      if (!import_mode) stage_tv();
+    }
+    __syncthreads();  // the barrier is initialised before anyone waits on it
+  }
   // L2 prefetch of the u rows (and t_prev rows) read after the inverse FFT
-  if (!ROWXF && tid < 2 * NCOMP && !(USTAGE && (tid & 1) == 0)) {
+  if (!ROWXF && tid < 2 * NCOMP && !((USTAGE || TVSTAGE) && (tid & 1) == 0)) {
     const T* src = (tid & 1) ? tprev_rd : u_in;
     if (src) {
       const size_t comp = (size_t)(tid >> 1) * plane;
@@ -284,26 +350,46 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
 
   grid_dep_wait();  // x (and u, t) of the previous kernels are complete from here on
   grid_dep_launch();
+  // an import follows whatever wrote u (a copy or the rescaling of u), so its rows are fetched only now
+  if (import_mode && tid == 0) {
+    if constexpr (USTAGE) {
+      if (a.test_fault != 1) bulk_copy_g2s(us, u_in + (size_t)r0 * N, (unsigned)(R * N * sizeof(T)), &ubar);
+    }
+    if constexpr (TVSTAGE) stage_tv();
+  }
   if (!import_mode) {
     // 1. gather the row half-spectra of the tile (two rows per complex FFT) from the column
     //    layout and invert the row DFT; thread = (pair p, column k) with p fastest, so that a warp
     //    reads the contiguous row segments of a few columns
     const C* xh = a.xh + (size_t)m * CP;
     const size_t kstride = (size_t)a.M * CP;
-    for (int idx = tid; idx < NPIN * H; idx += nth) {
-      const int p = idx % NPIN, k = idx / NPIN;
-      const C* col = xh + (size_t)k * kstride;
-      C xa, xb;
-      if constexpr (sizeof(C) == 8 && !HALO) {
-        // rows r0 + 2p, r0 + 2p + 1: adjacent, 16-byte aligned (r0 even, CP even)
-        const float4 v = *reinterpret_cast<const float4*>(col + r0 + 2 * p);
-        xa = mk<C>(v.x, v.y);
-        xb = mk<C>(v.z, v.w);
-      } else {
-        xa = col[grow(2 * p)];
-        xb = col[grow(2 * p + 1)];
+    // (kGather loads in flight per thread before the first use)
+    constexpr int ITEMS = NPIN * H, kGather = sizeof(T) == 4 ? 4 : 2;
+    for (int base = tid; base < ITEMS; base += kGather * NT) {
+      C xa[kGather], xb[kGather];
+#pragma unroll
+      for (int i = 0; i < kGather; ++i) {
+        const int idx = base + i * NT;
+        if (idx >= ITEMS) continue;
+        const int p = idx % NPIN, k = idx / NPIN;
+        const C* col = xh + (size_t)k * kstride;
+        if constexpr (sizeof(C) == 8 && !HALO) {
+          // rows r0 + 2p, r0 + 2p + 1: adjacent, 16-byte aligned (r0 even, CP even)
+          const float4 v = *reinterpret_cast<const float4*>(col + r0 + 2 * p);
+          xa[i] = mk<C>(v.x, v.y);
+          xb[i] = mk<C>(v.z, v.w);
+        } else {
+          xa[i] = col[grow(2 * p)];
+          xb[i] = col[grow(2 * p + 1)];
+        }
       }
-      pair_spectrum_put(zb + p * ZS, N, k, xa, xb);
+#pragma unroll
+      for (int i = 0; i < kGather; ++i) {
+        const int idx = base + i * NT;
+        if (idx >= ITEMS) continue;
+        const int p = idx % NPIN, k = idx / NPIN;
+        pair_spectrum_put(zb + p * ZS, N, k, xa[i], xb[i]);
+      }
     }
     __syncthreads();
     {
@@ -327,106 +413,271 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
 
   // 2. analysis operator, shrinkage, dual update; 3. q = qscale T^T (t - u')
   if constexpr (prior_is_tv(PRIOR)) {
-    // a_v at tile rows 0..R, a_h at tile rows 1..R; thread = (row pair p, column c)
-    for (int idx = tid; idx < NPIN * N; idx += nth) {
-      const int p = idx / N, c = idx - p * N;
-      C z0 = mk<C>(0.0, 0.0), zr = z0, zd = z0;
-      if (!import_mode) {
-        z0 = zb[p * ZS + spad(c)];
-        zr = zb[p * ZS + spad((c + 1) & (N - 1))];
-        if (p + 1 < NPIN) zd = zb[(p + 1) * ZS + spad(c)];
-      }
-      const T x0[2] = {z0.x, z0.y};
-      const T wv[2] = {z0.y - z0.x, zd.x - z0.y};
-      const T wh[2] = {zr.x - z0.x, zr.y - z0.y};
-#pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        const int j = 2 * p + s;
-        if (j > R) continue;  // row R+1: neither component needed
+    constexpr bool WALK = N >= 1024, LOW = LOGN == 11;
+    // MODE 0: plain; 1: with residual sums and / or t stored; 2: import (t given, x unused)
+    // u of component `comp` at tile row j, columns c0, c0 + 1
+    auto ldu = [&](int comp, int j, int c0) -> C {
+      if constexpr (TVSTAGE) return *reinterpret_cast<const C*>(us + (comp * (R + 1) + j) * N + c0);
+      else return __ldg(reinterpret_cast<const C*>(u_in + comp * plane + (size_t)grow(j) * N + c0));
+    };
+    auto ldu1 = [&](int comp, int j, int c) -> T {
+      if constexpr (TVSTAGE) return us[(comp * (R + 1) + j) * N + c];
+      else return __ldg(u_in + comp * plane + (size_t)grow(j) * N + c);
+    };
+    constexpr bool ISO = PRIOR == PRIOR_TV_ISO;
+    const C czero = mk<C>(0.0, 0.0);
+    if constexpr (TVSTAGE) mbar_wait_bounded(&ubar, 0, a.err);  // a failure is flagged: the iterate is then invalid
+    // isotropic TV: the pixel's two components shrink together (group soft threshold)
+    auto group = [&](T wh, T uh, T wv, T uv, T& th, T& uhn, T& ah, T& tv, T& uvn, T& av) {
+      const T vh = wh + uh, vv = wv + uv;
+      const T nrm = sqrt(fma(vh, vh, mul_rn(vv, vv)));
+      const T f = nrm > tau ? T(1) - tau / nrm : T(0);
+      th = mul_rn(vh, f);
+      tv = mul_rn(vv, f);
+      uhn = sub_rn(vh, th);
+      uvn = sub_rn(vv, tv);
+      ah = sub_rn(th, uhn);
+      av = sub_rn(tv, uvn);
+    };
+    // a_h of the output rows at the columns 64 b - 1, one thread each: what lane 0 of the warp that
+    // works on the columns 64 b .. 64 b + 63 needs
+    auto edges = [&](auto mode) {
+      constexpr int MODE = decltype(mode)::value, NB = N / 64;
+      if (tid < R * NB) {
+        const int j = 1 + tid / NB, b = tid & (NB - 1), c = (64 * b - 1) & (N - 1), cr = 64 * b;
         const size_t g = (size_t)grow(j) * N + c;
-        T tv, uvn, th = T(0), uhn = T(0);
-        if (import_mode) {
-          tv = timp[plane + g];
-          uvn = u_in[plane + g];
-          if (j >= 1) {
-            th = timp[g];
-            uhn = u_in[g];
-          }
-        } else if constexpr (PRIOR == PRIOR_TV_ISO) {
-          // isotropic TV: the pixel's two components shrink together (group soft threshold);
-          // the halo row needs its horizontal component too, for the vertical one
-          const T vh = wh[s] + u_in[g], vv = wv[s] + u_in[plane + g];
-          const T nrm = sqrt(vh * vh + vv * vv);
-          const T f = nrm > tau ? T(1) - tau / nrm : T(0);
-          th = vh * f;
-          tv = vv * f;
-          uhn = vh - th;
-          uvn = vv - tv;
+        T t = T(0), un = T(0), ah;
+        if constexpr (MODE == 2) {
+          ah = timp[g] - u_in[g];
         } else {
-          shrink(wv[s], u_in[plane + g], tau, tv, uvn);
-          if (j >= 1) shrink(wh[s], u_in[g], tau, th, uhn);
-        }
-        av[j * N + c] = tv - uvn;
-        if (j >= 1) {
-          u_out[plane + g] = uvn;
-          ah[(j - 1) * N + c] = th - uhn;
-          u_out[g] = uhn;
-          if (resid) {
-            acc_resid(part, wh[s], th, uhn, tprev_rd, g);
-            acc_resid(part, wv[s], tv, uvn, tprev_rd ? tprev_rd + plane : nullptr, g);
-          }
-          if (store_t) {
-            tprev[g] = th;
-            tprev[plane + g] = tv;
+          auto X = [&](int jj, int cc) {
+            const C z = zb[(jj >> 1) * ZS + spad(cc)];
+            return (jj & 1) ? z.y : z.x;
+          };
+          const T x = X(j, c);
+          if constexpr (PRIOR == PRIOR_TV_ISO) {
+            T t2, un2, av2;
+            group(X(j, cr) - x, ldu1(0, j, c), X(j + 1, c) - x, ldu1(1, j, c), t, un, ah, t2, un2, av2);
+          } else {
+            shrink(X(j, cr) - x, ldu1(0, j, c), tau, t, un);
+            ah = t - un;
           }
         }
-        (void)x0;
+        edge[tid / NB][b] = ah;
       }
-    }
-    __syncthreads();
-    // q at output rows jj = 0..R-1 (tile rows jj+1), written as row pairs
-    for (int idx = tid; idx < NPOUT * N; idx += nth) {
-      const int p = idx / N, c = idx - p * N;
-      const int cm = (c - 1) & (N - 1);
-      T q[2];
+      __syncthreads();
+    };
+    // One tile row j at the columns c0, c0 + 1: x of the row at c0 .. c0 + 2 and of the next row at
+    // c0, c0 + 1, a_v of the row above in avp (replaced by this row's).  FULL: the row is one of the
+    // tile's output rows (u, t and the residual sums are its own, q is formed).
+    auto row = [&](auto mode, auto full, int j, int c0, const T(&x)[3], const T(&xn)[3], C uh, C uv, T(&avp)[2],
+                   T(&q)[2], T(&ah)[2]) {
+      constexpr int MODE = decltype(mode)::value;
+      constexpr bool FULL = decltype(full)::value;
+      const size_t g = (size_t)grow(j) * N + c0;
+      T tv[2], uvn[2], th[2], uhn[2], av[2], wh[2] = {T(0), T(0)}, wv[2] = {T(0), T(0)};
+      if constexpr (MODE == 2) {
 #pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        const int jj = 2 * p + s;
-        q[s] = (ah[jj * N + cm] - ah[jj * N + c] + av[jj * N + c] - av[(jj + 1) * N + c]) * a.qscale;
-      }
-      zb[p * ZS + spad(c)] = mk<C>(q[0], q[1]);
-    }
-    // Row frequencies k2 = 0 and 1 (kLowK = 2) of the two components of a = t - u' on the output
-    // rows, as direct sums with the exact table twiddle exp(-2 pi i c / N), for the low-column
-    // correction of the x-update (launch_passB_split): near DC the FP32 transforms of q = D^T a
-    // carry a uniform rounding error that Psi^{-1} amplifies by ~1/g, while transforms of a itself
-    // do not.  One warp per (row, component), lanes over the columns; layout [comp][k2][map][CP].
-    static_assert(kLowK == 2, "the sums below form k2 = 0 and 1");
-    if (a.lowbuf) {
-      const int nw = nth >> 5, wid = tid >> 5, lane = tid & 31;
-      for (int o = wid; o < R * 2; o += nw) {
-        const int jj = o >> 1, comp = o & 1;
-        const T* src = comp == 0 ? ah + jj * N : av + (jj + 1) * N;
-        T s0 = T(0), re = T(0), im = T(0);
-        for (int c = lane; c < N; c += 32) {
-          const T v = src[c];
-          const C w = ldg_tw(&a.tw[c * (kTwN / N)]);
-          s0 += v;
-          re = fma(v, (T)w.x, re);
-          im = fma(v, (T)w.y, im);
+        for (int e = 0; e < 2; ++e) {
+          tv[e] = timp[plane + g + e];
+          uvn[e] = u_in[plane + g + e];
+          if constexpr (FULL) {
+            th[e] = timp[g + e];
+            uhn[e] = u_in[g + e];
+          }
         }
+      } else {
+        wv[0] = xn[0] - x[0];
+        wv[1] = xn[1] - x[1];
+        if constexpr (PRIOR == PRIOR_TV_ISO) {
+          wh[0] = x[1] - x[0];
+          wh[1] = x[2] - x[1];
+          group(wh[0], uh.x, wv[0], uv.x, th[0], uhn[0], ah[0], tv[0], uvn[0], av[0]);
+          group(wh[1], uh.y, wv[1], uv.y, th[1], uhn[1], ah[1], tv[1], uvn[1], av[1]);
+        } else {
+          shrink(wv[0], uv.x, tau, tv[0], uvn[0]);
+          shrink(wv[1], uv.y, tau, tv[1], uvn[1]);
+          if constexpr (FULL) {
+            wh[0] = x[1] - x[0];
+            wh[1] = x[2] - x[1];
+            shrink(wh[0], uh.x, tau, th[0], uhn[0]);
+            shrink(wh[1], uh.y, tau, th[1], uhn[1]);
+          }
+        }
+      }
+      if constexpr (PRIOR != PRIOR_TV_ISO || MODE == 2) {
+        av[0] = tv[0] - uvn[0];
+        av[1] = tv[1] - uvn[1];
+        if constexpr (FULL) {
+          ah[0] = th[0] - uhn[0];
+          ah[1] = th[1] - uhn[1];
+        }
+      }
+      if constexpr (FULL) {
+        T ahm = __shfl_up_sync(0xffffffffu, ah[1], 1);
+        if ((tid & 31) == 0) ahm = edge[j - 1][c0 / 64];
+        *reinterpret_cast<C*>(u_out + plane + g) = cpack<C>(uvn[0], uvn[1]);
+        *reinterpret_cast<C*>(u_out + g) = cpack<C>(uhn[0], uhn[1]);
+        if constexpr (MODE == 1) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          s0 += __shfl_down_sync(0xffffffffu, s0, off);
-          re += __shfl_down_sync(0xffffffffu, re, off);
-          im += __shfl_down_sync(0xffffffffu, im, off);
+          for (int e = 0; e < 2; ++e) {
+            if (resid) {
+              acc_resid(part, wh[e], th[e], uhn[e], tprev_rd, g + e);
+              acc_resid(part, wv[e], tv[e], uvn[e], tprev_rd ? tprev_rd + plane : nullptr, g + e);
+            }
+            if (store_t) {
+              tprev[g + e] = th[e];
+              tprev[plane + g + e] = tv[e];
+            }
+          }
         }
-        if (lane == 0) {
-          a.lowbuf[((size_t)(comp * kLowK + 0) * a.M + m) * CP + r0 + jj] = mk<C>(s0, 0.0);
-          a.lowbuf[((size_t)(comp * kLowK + 1) * a.M + m) * CP + r0 + jj] = mk<C>(re, im);
+        q[0] = (ahm - ah[0] + avp[0] - av[0]) * a.qscale;
+        q[1] = (ah[0] - ah[1] + avp[1] - av[1]) * a.qscale;
+      }
+      avp[0] = av[0];
+      avp[1] = av[1];
+    };
+    // x of tile rows 2p, 2p + 1 at the columns c0 .. c0 + 2
+    auto load_pair = [&](auto mode, int p, int c0, T(&xa)[3], T(&xb)[3]) {
+      if constexpr (decltype(mode)::value != 2) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const C z = zb[p * ZS + spad((c0 + e) & (N - 1))];
+          xa[e] = z.x;
+          xb[e] = z.y;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) xa[e] = xb[e] = T(0);
+      }
+    };
+    constexpr std::true_type full{};
+    constexpr std::false_type halo{};
+    auto phase = [&](auto mode) {
+      edges(mode);
+      if constexpr (!WALK) {
+        constexpr int RG = tv_rows(N), NG = R / RG, TG = NT / NG;
+        static_assert(TG >= N / 2 && TG % 32 == 0, "one column pair per thread, whole warps per row group");
+        const int rg = tid / TG, cp = tid - rg * TG, c0 = 2 * cp;
+        const bool on = rg < NG && cp < N / 2;
+        const int p0 = rg * (RG / 2);  // output rows: tile rows 2 p0 + 1 .. 2 p0 + RG
+        T qv[RG][2];
+        if (on) {
+          T xa[3], xb[3], avp[2], ah[2];
+          load_pair(mode, p0, c0, xa, xb);
+          row(mode, halo, 2 * p0, c0, xa, xb, ISO ? ldu(0, 2 * p0, c0) : czero, ldu(1, 2 * p0, c0), avp, qv[0], ah);
+#pragma unroll
+          for (int i = 0; i < RG / 2; ++i) {
+            T ya[3], yb[3];
+            load_pair(mode, p0 + i + 1, c0, ya, yb);
+            const int j = 2 * (p0 + i) + 1;
+            row(mode, full, j, c0, xb, ya, ldu(0, j, c0), ldu(1, j, c0), avp, qv[2 * i], ah);
+            row(mode, full, j + 1, c0, ya, yb, ldu(0, j + 1, c0), ldu(1, j + 1, c0), avp, qv[2 * i + 1], ah);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) xb[e] = yb[e];
+          }
+        }
+        __syncthreads();  // every thread has read the x tile: q takes its place, as row pairs
+        if (on) {
+#pragma unroll
+          for (int i = 0; i < RG / 2; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) zb[(p0 + i) * ZS + spad(c0 + e)] = cpack<C>(qv[2 * i][e], qv[2 * i + 1][e]);
+        }
+      } else {
+        constexpr int NIT = (N / 2 + NT - 1) / NT;
+        T xb[NIT][3], avp[NIT][2], q[NIT][2][2];
+        C un[NIT][2][2];  // u of the next two rows, [row][component], loaded one row pair ahead
+#pragma unroll
+        for (int it = 0; it < NIT; ++it) {
+          const int cp = tid + it * NT;
+          if (cp < N / 2) {
+            T xa[3], ah[2];
+            load_pair(mode, 0, 2 * cp, xa, xb[it]);
+            row(mode, halo, 0, 2 * cp, xa, xb[it], ISO ? ldu(0, 0, 2 * cp) : czero, ldu(1, 0, 2 * cp), avp[it],
+                q[it][0], ah);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) un[it][e >> 1][e & 1] = ldu(e & 1, 1 + (e >> 1), 2 * cp);
+          }
+        }
+#pragma unroll 1
+        for (int i = 0; i < R / 2; ++i) {
+          // Row frequencies k2 = 0 and 1 (kLowK = 2) of the two components of a = t - u' on the
+          // output rows, as direct sums with the exact table twiddle exp(-2 pi i c / N), for the
+          // low-column correction of the x-update (launch_passB_split): near DC the FP32 transforms
+          // of q = D^T a carry a uniform rounding error that Psi^{-1} amplifies by ~1/g, while
+          // transforms of a itself do not.  Value 6 r + 3 comp + {0, 1, 2}: row r of the pair, sum a,
+          // Re and Im of sum a exp(-2 pi i c / N)
+          T low[LOW ? 16 : 1];
+#pragma unroll
+          for (int e = 0; e < (LOW ? 16 : 1); ++e) low[e] = T(0);
+#pragma unroll
+          for (int it = 0; it < NIT; ++it) {
+            const int cp = tid + it * NT, c0 = 2 * cp;
+            if (cp < N / 2) {
+              T ya[3], yb[3], ah[2];
+              load_pair(mode, i + 1, c0, ya, yb);
+              auto add_low = [&](int r) {
+                if constexpr (LOW) {
+                  const C w0 = ldg_tw(&a.tw[c0 * (kTwN / N)]), w1 = ldg_tw(&a.tw[(c0 + 1) * (kTwN / N)]);
+#pragma unroll
+                  for (int s = 0; s < 2; ++s) {
+                    const T v0 = s ? avp[it][0] : ah[0], v1 = s ? avp[it][1] : ah[1];
+                    T* l = &low[6 * r + 3 * s];
+                    l[0] += v0 + v1;
+                    l[1] = fma(v1, (T)w1.x, fma(v0, (T)w0.x, l[1]));
+                    l[2] = fma(v1, (T)w1.y, fma(v0, (T)w0.y, l[2]));
+                  }
+                }
+              };
+              C uc[2][2];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                uc[e >> 1][e & 1] = un[it][e >> 1][e & 1];
+                if (i + 1 < R / 2) un[it][e >> 1][e & 1] = ldu(e & 1, 2 * i + 3 + (e >> 1), c0);
+              }
+              row(mode, full, 2 * i + 1, c0, xb[it], ya, uc[0][0], uc[0][1], avp[it], q[it][0], ah);
+              add_low(0);
+              row(mode, full, 2 * i + 2, c0, ya, yb, uc[1][0], uc[1][1], avp[it], q[it][1], ah);
+              add_low(1);
+#pragma unroll
+              for (int e = 0; e < 3; ++e) xb[it][e] = yb[e];
+            }
+          }
+          if constexpr (LOW) {
+            // warp sums of the 12 values by recursive halving: lane l ends with value l >> 1
+            reduce_scatter16(low, tid & 31);
+            if ((tid & 1) == 0 && (tid & 31) < 24) lows[i & 1][tid >> 5][(tid & 31) >> 1] = low[0];
+          }
+          __syncthreads();  // every thread has read x rows 2i, 2i + 1: q rows 2i, 2i + 1 take their place
+#pragma unroll
+          for (int it = 0; it < NIT; ++it) {
+            const int cp = tid + it * NT;
+            if (cp < N / 2) {
+#pragma unroll
+              for (int e = 0; e < 2; ++e) zb[i * ZS + spad(2 * cp + e)] = cpack<C>(q[it][0][e], q[it][1][e]);
+            }
+          }
+          if constexpr (LOW) {
+            if (a.lowbuf && tid < 12) {  // value tid of rows 2i, 2i + 1: the warps' sums in order
+              T s = T(0);
+              for (int wp = 0; wp < NT / 32; ++wp) s += lows[i & 1][wp][tid];
+              const int r = tid / 6, comp = (tid / 3) & 1, e = tid % 3;
+              T* dst = reinterpret_cast<T*>(a.lowbuf + ((size_t)(comp * kLowK + (e > 0)) * a.M + m) * CP + r0 + 2 * i + r);
+              if (e == 0) {
+                dst[0] = s;
+                dst[1] = T(0);
+              } else {
+                dst[e - 1] = s;
+              }
+            }
+          }
         }
       }
-    }
+    };
+    if (import_mode) phase(std::integral_constant<int, 2>{});
+    else if (resid || store_t) phase(std::integral_constant<int, 1>{});
+    else phase(std::integral_constant<int, 0>{});
   } else if constexpr (PRIOR == PRIOR_DCT8) {
     if (!import_mode) {
       // row DCT of every 8-sample segment of both rows of a pair, in place
@@ -546,6 +797,9 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     }
   }
   if (resid) block_reduce_store<T>(part, a.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kNPart);
+  if constexpr (TVSTAGE) {
+    if (tid == 0) mbar_wait_bounded(&ubar, 0, a.err);  // as below, for a wait that gave up
+  }
   if constexpr (USTAGE) {
     // a copy that was only late must not write this CTA's shared memory after the CTA ends
     if (tid == 0 && !u_ok && a.test_fault == 0) mbar_wait_bounded(&ubar, 0, a.err);
