@@ -675,35 +675,39 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
     // dictionary: column DFT of rho (t - u) over the L*M coefficient maps, the per-(bin, channel)
     // x- and z-update, inverse column DFT of v
     const int S = smaps(p);
-    CIP_LAUNCH(p, launch_cols_fft<T>(static_cast<const C*>(p->qh), static_cast<C*>(p->colbuf),
-                                     static_cast<const C*>(p->tw), p->N, S, -1, s));
+    const bool fused = p->Q == 0 && cd_fused_fits<T>(p->N, p->L);
+    if (!fused)
+      CIP_LAUNCH(p, launch_cols_fft<T>(static_cast<const C*>(p->qh), static_cast<C*>(p->colbuf),
+                                       static_cast<const C*>(p->tw), p->N, S, -1, s));
     if (p->Q > 0) {
       CD3Args<T> a = cd3_args<T>(p);
       CIP_LAUNCH(p, launch_cd3_solve<T>(a, s));
+    } else {
+      CDArgs<T> a;
+      a.colbuf = !fused || p->dl_sigma > 0 ? static_cast<C*>(p->colbuf) : nullptr;
+      a.qh = static_cast<const C*>(p->qh);
+      a.xh = static_cast<C*>(p->xh);
+      a.tw = static_cast<const C*>(p->tw);
+      a.theta = static_cast<const C*>(theta_of(p));
+      a.th_planes = theta_planes(p);
+      a.p_in = static_cast<const C*>(p->pbuf[p->pcur]);
+      a.p_out = static_cast<C*>(p->pbuf[p->pcur ^ 1]);
+      a.xb = static_cast<const C*>(p->bhat);
+      a.pinv = static_cast<const C*>(p->pinv);
+      a.xcol = static_cast<C*>(p->xcol);
+      a.N = p->N;
+      a.M = p->M;
+      a.L = p->L;
+      a.gs = p->gs;
+      a.rho = (T)p->rho;
+      a.mu = (T)p->mu;
+      a.n2 = (T)((double)p->N * p->N);
+      if (fused) CIP_LAUNCH(p, launch_cd_fused<T>(a, s));
+      else CIP_LAUNCH(p, launch_cd_solve<T>(a, s));
+    }
+    if (!fused)
       CIP_LAUNCH(p, launch_cols_fft<T>(static_cast<const C*>(p->colbuf), static_cast<C*>(p->xh),
                                        static_cast<const C*>(p->tw), p->N, S, +1, s));
-      p->pcur ^= 1;
-      return CIP_OK;
-    }
-    CDArgs<T> a;
-    a.colbuf = static_cast<C*>(p->colbuf);
-    a.theta = static_cast<const C*>(theta_of(p));
-    a.th_planes = theta_planes(p);
-    a.p_in = static_cast<const C*>(p->pbuf[p->pcur]);
-    a.p_out = static_cast<C*>(p->pbuf[p->pcur ^ 1]);
-    a.xb = static_cast<const C*>(p->bhat);
-    a.pinv = static_cast<const C*>(p->pinv);
-    a.xcol = static_cast<C*>(p->xcol);
-    a.N = p->N;
-    a.M = p->M;
-    a.L = p->L;
-    a.gs = p->gs;
-    a.rho = (T)p->rho;
-    a.mu = (T)p->mu;
-    a.n2 = (T)((double)p->N * p->N);
-    CIP_LAUNCH(p, launch_cd_solve<T>(a, s));
-    CIP_LAUNCH(p, launch_cols_fft<T>(static_cast<const C*>(p->colbuf), static_cast<C*>(p->xh),
-                                     static_cast<const C*>(p->tw), p->N, S, +1, s));
     p->pcur ^= 1;
     return CIP_OK;
   }

@@ -91,6 +91,126 @@ __global__ void __launch_bounds__(128) cd_solve_kernel(CDArgs<T> a) {
   a.p_out[((size_t)k2 * M + m) * CP + k1] = pn;
 }
 
+// The whole column pass of one (column k2, channel m) in one CTA: the forward column DFTs of the
+// channel's L maps of G into a shared-memory tile, the x-update and the Sherman-Morrison z-update
+// per bin on the tile, and the inverse column DFTs of v out of it.  The L maps are all a bin's
+// z-update needs, so the code spectra are read once and written once (the three-kernel form, column
+// DFT / cd_solve_kernel / column DFT, moves them six times).
+// What bounds it: shared-memory traffic of the FFT stages (16 passes over the tile, ~20 us at 256^2 x 5
+// with 32 filters); HBM needs 12 us for the two passes over the spectra.  Column pass there 95.7 ->
+// 46.1 us, 128^2 x 3 with 8 filters 16.9 -> 10.0, 512^2 x 3 with 16 filters 100 -> 54 us.
+constexpr int kFuseThreads = 256;
+template <typename T> constexpr int fuse_elems(int N) {  // FFT elements per thread: teams stay inside a warp
+  if (sizeof(T) == 4) return N <= 256 ? 8 : (N == 512 ? 16 : 32);
+  return N <= 128 ? 8 : 16;
+}
+template <typename T> constexpr int fuse_slot(int N) { return spad(N); }
+
+template <typename T, int LOGN>
+__global__ void __launch_bounds__(kFuseThreads) cd_fused_kernel(const CDArgs<T> a) {
+  using C = typename CT<T>::type;
+  constexpr int N = 1 << LOGN, E = fuse_elems<T>(N), TT = N / E, TEAMS = kFuseThreads / TT;
+  constexpr int CP = col_pitch(N), ZS = fuse_slot<T>(N);
+  static_assert(TT <= 32, "a team's barriers are warp barriers");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tile = reinterpret_cast<C*>(smem_raw);  // [L][ZS]
+  const int M = a.M, L = a.L;
+  const int m = blockIdx.x, k2 = blockIdx.y, tid = threadIdx.x, team = tid / TT, tt = tid % TT;
+  const unsigned mask = TT == 32 ? 0xffffffffu : (((1u << TT) - 1u) << ((team * TT) & 31));
+  auto sync = [&]() { __syncwarp(mask); };
+  const size_t map0 = ((size_t)k2 * M * L + (size_t)m * L) * CP;
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int l = team; l < L; l += TEAMS) {
+    const C* src = a.qh + map0 + (size_t)l * CP;
+    C* buf = tile + (size_t)l * ZS;
+    auto in0 = [&](int i0, int off) { return src[i0 + off]; };
+    auto outL = [&](int i0, int off, C v) { buf[spad(i0) + off + (off >> 4)] = v; };
+    fft_team_io<C, LOGN, E, -1, true>(buf, tt, a.tw, sync, in0, outL);
+  }
+  __syncthreads();
+  const int npk = M * (M + 1) / 2;
+  const C* th0 = a.theta + (size_t)k2 * a.th_planes * CP;
+  for (int k1 = tid; k1 < N; k1 += kFuseThreads) {
+    // x_m = xb_m + N^2 sum_j (Psi^{-1} / N^2)(m, j) p_j, as in cd_solve_kernel
+    const C* pin = a.p_in + (size_t)k2 * M * CP + k1;
+    const C* pcol = a.pinv + binp(k2, 0, k1, npk, N);
+    C acc = mk<C>(0.0, 0.0);
+    for (int j = 0; j < M; ++j) {
+      const int i0 = min(m, j), j0 = max(m, j);
+      const C pij = pcol[(size_t)(i0 * M - (i0 * (i0 - 1)) / 2 + (j0 - i0)) * kBinBlock];
+      const C pj = pin[(size_t)j * CP];
+      if (m <= j) cfma(acc, pij, pj);
+      else cfmac(acc, pij, pj);
+    }
+    C x = a.xb[binp(k2, m, k1, M, N)];
+    x.x += a.n2 * acc.x;
+    x.y += a.n2 * acc.y;
+    a.xcol[((size_t)k2 * M + m) * CP + k1] = x;
+    // c_l = conj(theta_l) x + G_l (formed again in the second loop: one shared-memory load and four
+    // multiply-adds instead of 2 L registers), s = theta^T c, nrm = ||theta||^2
+    const C* th = th0 + k1;
+    C* g = tile + spad(k1);
+    C s = mk<C>(0.0, 0.0);
+    T nrm = T(0);
+#pragma unroll 8
+    for (int l = 0; l < L; ++l) {
+      const C t = __ldg(th + (size_t)l * CP);
+      C cl = g[(size_t)l * ZS];
+      cfmac(cl, t, x);
+      cfma(s, t, cl);
+      nrm += t.x * t.x + t.y * t.y;
+    }
+    const T rho_w = a.mu == T(0) ? a.rho : a.rho + a.mu * (T)(a.gs[k1] + a.gs[k2]);
+    const T inv_rho = T(1) / rho_w;
+    const T den = T(1) / (rho_w + nrm);
+    const C coef = mk<C>(s.x * den, s.y * den);
+    C pn = mk<C>(0.0, 0.0);
+#pragma unroll 8
+    for (int l = 0; l < L; ++l) {
+      const C t = __ldg(th + (size_t)l * CP);
+      C v = g[(size_t)l * ZS];
+      cfmac(v, t, x);
+      v.x -= t.x * coef.x + t.y * coef.y;
+      v.y -= t.x * coef.y - t.y * coef.x;
+      v.x *= inv_rho;
+      v.y *= inv_rho;
+      g[(size_t)l * ZS] = v;
+      if (a.colbuf) a.colbuf[map0 + (size_t)l * CP + k1] = v;  // kept for the dictionary update
+      cfma(pn, t, v);
+    }
+    a.p_out[((size_t)k2 * M + m) * CP + k1] = pn;
+  }
+  __syncthreads();
+  for (int l = team; l < L; l += TEAMS) {
+    C* buf = tile + (size_t)l * ZS;
+    C* dst = a.xh + map0 + (size_t)l * CP;
+    auto in0 = [&](int i0, int off) { return buf[spad(i0) + off + (off >> 4)]; };
+    auto outL = [&](int i0, int off, C v) { dst[i0 + off] = v; };
+    fft_team_io<C, LOGN, E, +1, false>(buf, tt, a.tw, sync, in0, outL);
+  }
+}
+
+// shared memory of the fused column pass; 0 where it does not run (a team wider than a warp, or a
+// tile beyond one CTA's shared memory): the three-kernel form is used there
+template <typename T> size_t fuse_smem(int N, int L) {
+  if (N / fuse_elems<T>(N) > 32) return 0;
+  const size_t sm = (size_t)L * fuse_slot<T>(N) * sizeof(typename CT<T>::type);
+  return sm <= 224 * 1024 ? sm : 0;
+}
+
+template <typename T, int LOGN> cudaError_t launch_fused(const CDArgs<T>& a, cudaStream_t s) {
+  if constexpr ((1 << LOGN) / fuse_elems<T>(1 << LOGN) > 32) {
+    return cudaErrorInvalidValue;
+  } else {
+    auto k = cd_fused_kernel<T, LOGN>;
+    static PerDeviceOnce once;
+    cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024); });
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k, dim3(a.M, a.N / 2 + 1), dim3(kFuseThreads), fuse_smem<T>(a.N, a.L), s, 0, a);
+  }
+}
+
 // filters d[L][P][P] (centre P/2) placed on the N x N torus with the centre at (0,0)
 template <typename Tin>
 __global__ void embed_kernel(const Tin* __restrict__ d, double* __restrict__ out, int L, int P, int N) {
@@ -631,6 +751,23 @@ template <typename T> cudaError_t launch_cd_solve(const CDArgs<T>& a, cudaStream
   }
   return cudaGetLastError();
 }
+
+template <typename T> bool cd_fused_fits(int N, int L) { return fuse_smem<T>(N, L) > 0; }
+template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s) {
+  if (a.L < 1 || a.L > 32 || !cd_fused_fits<T>(a.N, a.L)) return cudaErrorInvalidValue;
+  switch (a.N) {
+    case 64: return launch_fused<T, 6>(a, s);
+    case 128: return launch_fused<T, 7>(a, s);
+    case 256: return launch_fused<T, 8>(a, s);
+    case 512: return launch_fused<T, 9>(a, s);
+    case 1024: return launch_fused<T, 10>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+template bool cd_fused_fits<float>(int, int);
+template bool cd_fused_fits<double>(int, int);
+template cudaError_t launch_cd_fused<float>(const CDArgs<float>&, cudaStream_t);
+template cudaError_t launch_cd_fused<double>(const CDArgs<double>&, cudaStream_t);
 
 template <typename Tin>
 cudaError_t launch_embed_filters(const Tin* d, double* out, int L, int P, int N, cudaStream_t s) {

@@ -75,7 +75,11 @@ cudaError_t launch_rhs_fp32(const cdf* lam, const cdf* yhat, int K, int M, int N
 // thread per (frequency, channel).  Column layout [k2][plane][col_pitch(N)].
 template <typename T> struct CDArgs {
   using C = typename CT<T>::type;
-  C* colbuf;       // [H][M*L]: in G = col-DFT of rho (t - u) / N^2, out v (channel-major, m*L + l)
+  C* colbuf;       // [H][M*L]: in G = col-DFT of rho (t - u) / N^2, out v (channel-major, m*L + l);
+                   // fused column pass: out v where non-null (the dictionary update reads it)
+  const C* qh;     // fused column pass: [H][M*L] row spectra of rho (t - u) / N^2
+  C* xh;           // fused column pass: [H][M*L] row spectra of v
+  const C* tw;
   const C* theta;  // [H][th_planes]: DFT of the embedded filters in the first L planes of each bin
   const C* p_in;   // [H][M]: p = sum_l theta_l v_l of the previous iteration (scaled 1/N^2)
   C* p_out;        // [H][M]
@@ -90,6 +94,10 @@ template <typename T> struct CDArgs {
   T n2;            // N^2
 };
 template <typename T> cudaError_t launch_cd_solve(const CDArgs<T>& a, cudaStream_t s);
+// the column pass around it (column DFT, solve, inverse column DFT) in one kernel, one CTA per
+// (column, channel); fits: the L column spectra of a channel fit in shared memory
+template <typename T> bool cd_fused_fits(int N, int L);
+template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s);
 
 // 3D dictionary (Section IV-B, 3D case; csrc/convdict3d.cu): the same column layout for the
 // channel-domain spectra; theta holds Theta_l(kappa, w) at plane kappa*L + l of [H][M*L][CP].
