@@ -96,7 +96,8 @@ typedef struct cip_options {
                        and the TV, isotropic TV, DCT, l1 and dictionary (l1 on the codes) priors: 0 =
                        chosen by the autotuner together
                        with the column-pass form (timing whole iterations; the default width when
-                       column_pass != 0), 8 or 16 = that width; ignored for other plans */
+                       column_pass != 0; the l1 and dictionary priors at N = 256 also have the width
+                       32), 8 or 16 = that width; ignored for other plans */
   int reserved[11];
 } cip_options;
 
@@ -282,8 +283,8 @@ cip_status cip_get_timing(cip_plan* plan, double* prior_pass_ms, int* prior_pass
                           int* column_pass_n);
 
 /* Test-only fault switch for the bounded device waits (no counterpart in the paper).
- * kind 1: the prior pass of CIP_PRIOR_DCT8 / CIP_PRIOR_L1 plans (at sizes whose u rows it stages
- * in shared memory by a bulk copy) arms its copy barrier for two arrivals, gives one and issues no
+ * kind 1: the prior pass of CIP_PRIOR_DCT8 plans (at sizes whose u rows it stages in shared memory
+ * by a bulk copy) and of CIP_PRIOR_L1 plans (which stage nothing and arm a barrier for this test) arms its copy barrier for two arrivals, gives one and issues no
  * copy, then waits at most 64 polls: the wait gives up with nothing in flight, the kernel reads u
  * from global memory instead (the iterate is unchanged) and flags the plan, so that
  * cip_get_residuals (and the residual checks of cip_iterate) return CIP_ERR_TIMEOUT until the
@@ -293,7 +294,7 @@ cip_status cip_set_test_fault(cip_plan* plan, int kind);
 /* Number of CUDA kernels this plan has launched since creation. */
 cip_status cip_get_launches(cip_plan* plan, unsigned long long* launches);
 
-/* FFT elements per thread of the plan's prior-pass kernel (8 or 16; after cip_set_measurements
+/* FFT elements per thread of the plan's prior-pass kernel (8, 16 or 32; after cip_set_measurements
  * this is the autotuner's choice where it has one). */
 cip_status cip_get_prior_fft(cip_plan* plan, int* elems_per_thread);
 

@@ -21,6 +21,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 UNITS = [
     ("abi.cu", [], "abi.o"),
     ("passA.cu", [], "passA.o"),
+    ("rowpass.cu", [], "rowpass.o"),
     ("colpass.cu", [], "colpass.o"),
     ("fft_kernels.cu", [], "fft_kernels.o"),
     ("factor.cu", [], "factor.o"),

@@ -60,7 +60,7 @@ struct cip_plan {
   size_t esz = 4;
   int rowsA = 8, cc = 1, blocksA = 0, blocksB = 0;
   int colmode = 1;  // column pass: 1 fused kernel, 2 split (FFT / solve / FFT)
-  int avar = 0;     // prior-pass kernel variant (the other FFT width; complex64, N = 256 .. 1024)
+  int avar = 0;     // prior-pass kernel variant (1: the other FFT width, 2: 32; complex64, N = 256 .. 1024)
   int test_fault = 0;  // test-only fault switch (cip_set_test_fault)
   // TV at N >= kLowFixMinN: low-column correction of the x-update (launch_passB_split)
   void* lowbuf = nullptr;  // [2][kLowK][M][CP] low-frequency row DFTs of the components of t - u
@@ -276,7 +276,7 @@ template <typename T> cip_status alloc_state(cip_plan* p) {
     CIP_CUDA(p, cudaMemcpyAsync(p->wcos, c.data(), c.size() * sizeof(T), cudaMemcpyHostToDevice, p->ast));
     CIP_CUDA(p, cudaStreamSynchronize(p->ast));
   }
-  p->rowsA = passA_rows<T>(p->N, tile_kind(p->prior));
+  p->rowsA = prior_pass_kind(p) == PRIOR_L1 ? rowpass_rows(p->N) : passA_rows<T>(p->N, tile_kind(p->prior));
   p->blocksA = (p->N / p->rowsA) * smaps(p);
   CIP_CUDA(p, dmalloc(p, (void**)&p->partials, (size_t)p->blocksA * kNPart * sizeof(double)));
   return CIP_OK;
@@ -568,8 +568,7 @@ template <typename T> PassAArgs<T> passA_args(cip_plan* p, int flags) {
 
 template <typename T> PassBArgs<T> passB_args(cip_plan* p);
 
-// Row transforms between the column-layout row spectra and real rows ([maps][N][N]), run by the
-// prior-pass kernel without a prior: x = row IDFT of `spec` into `rows` (read-back, wavelet
+// Row transforms between the column-layout row spectra and real rows ([maps][N][N]): x = row IDFT of `spec` into `rows` (read-back, wavelet
 // chain), or spec = row DFT of scale * rows.
 template <typename T> cudaError_t rows_from_spec(cip_plan* p, const void* spec, int maps, void* rows, cudaStream_t s) {
   using C = typename CT<T>::type;
@@ -579,7 +578,7 @@ template <typename T> cudaError_t rows_from_spec(cip_plan* p, const void* spec, 
   a.err = p->conv + 1;
   a.tw = static_cast<const C*>(p->tw);
   a.M = maps;
-  return launch_passA<T>(a, p->N, ROWS_OUT, s);
+  return launch_rowpass<T>(a, p->N, ROWS_OUT, s);
 }
 template <typename T>
 cudaError_t spec_from_rows(cip_plan* p, const void* rows, int maps, double scale, void* spec, cudaStream_t s) {
@@ -591,7 +590,7 @@ cudaError_t spec_from_rows(cip_plan* p, const void* rows, int maps, double scale
   a.tw = static_cast<const C*>(p->tw);
   a.M = maps;
   a.qscale = (T)(0.5 * scale);  // the 1/2 of the pair extraction
-  return launch_passA<T>(a, p->N, ROWS_IN, s);
+  return launch_rowpass<T>(a, p->N, ROWS_IN, s);
 }
 
 // The prior pass: one fused kernel per row tile for TV, DCT and l1; for the wavelet (x) DCT prior
@@ -760,8 +759,12 @@ bool prior_has_variant(const cip_plan* p) {
          (p->prior == CIP_PRIOR_TV || p->prior == CIP_PRIOR_TV_ISO || p->prior == CIP_PRIOR_DCT8 ||
           p->prior == CIP_PRIOR_L1 || p->prior == CIP_PRIOR_CONVDICT);  // dictionaries: l1 on the codes
 }
+bool row_prior(const cip_plan* p) { return p->prior >= 0 && prior_pass_kind(p) == PRIOR_L1; }
+// T = I at N = 256 has a third width, 32, in which the last two FFT stages merge (rowpass.cu)
+bool has_wide_variant(const cip_plan* p) { return prior_has_variant(p) && row_prior(p) && p->N == 256; }
 // FFT elements per thread of the prior pass's default kernel (the device-side rule of passA.cu)
 int prior_fft_default(const cip_plan* p) {
+  if (row_prior(p)) return p->dtype == CIP_F32 ? rowpass_elems<float>(p->N, 0) : rowpass_elems<double>(p->N, 0);
   const bool tv = p->prior == CIP_PRIOR_TV || p->prior == CIP_PRIOR_TV_ISO;
   return (p->dtype == CIP_F32 && p->N <= 1024) ? ((p->N == 512 && !tv) ? 16 : 8) : 16;
 }
@@ -810,8 +813,8 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   }
   if (!p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));
   std::vector<TuneVal> cands;
-  for (int av = 0; av < (fav < 0 ? 2 : 1); ++av) {
-    if (fav >= 0) av = fav;
+  const int av0 = fav < 0 ? 0 : fav, av1 = fav < 0 ? (has_wide_variant(p) ? 2 : 1) : fav;
+  for (int av = av0; av <= av1; ++av) {
     if (is_cd(p)) {  // dictionary plans have one column-pass form; only the prior-pass width is tuned
       cands.push_back({p->colmode, p->cc, av});
       continue;
@@ -1738,7 +1741,7 @@ cip_status cip_get_launches(cip_plan* p, unsigned long long* n) {
 cip_status cip_get_prior_fft(cip_plan* p, int* elems) {
   if (!p || !elems) return CIP_ERR_INVALID_ARG;
   const int e = prior_fft_default(p);
-  *elems = (prior_has_variant(p) && p->avar == 1) ? 24 - e : e;
+  *elems = !prior_has_variant(p) || p->avar == 0 ? e : (p->avar == 1 ? 24 - e : 32);
   return CIP_OK;
 }
 

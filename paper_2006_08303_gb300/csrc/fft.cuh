@@ -140,7 +140,6 @@ __device__ __forceinline__ void stockham_stage(C* buf, int f, int tt, const C* _
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
-#pragma unroll
       if constexpr (R == 8) {
         const C w1 = ldg_tw(&tw[j * (kTwN / (LS * R))]), w4 = ldg_tw(&tw[4 * j * (kTwN / (LS * R))]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
@@ -235,7 +234,6 @@ __device__ __forceinline__ void fft_stage_io(int tt, const C* __restrict__ tw, I
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
-#pragma unroll
       if constexpr (R == 8) {
         const C w1 = ldg_tw(&tw[j * (kTwN / (LS * R))]), w4 = ldg_tw(&tw[4 * j * (kTwN / (LS * R))]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
@@ -307,6 +305,66 @@ __device__ __forceinline__ void fft_team_io(C* buf, int tt, const C* __restrict_
   constexpr int LSL = REM == 0 ? (1 << (3 * (S8 - 1))) : (1 << (3 * S8));
   if constexpr (OUTL_ALIAS) fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, bar, outL);
   else fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, none, outL);
+}
+
+// The last radix-8 stage and the radix-2/4 stage after it in one: for N = 8 LS R2 (R2 = 2 or 4) the
+// radix-R2 butterfly at j takes output j mod 8 LS of the R2 radix-8 butterflies whose indexes agree
+// mod LS, so a thread that holds those R2 butterflies (E = 8 R2 LS / TT elements, TT <= LS) needs no
+// exchange between the two stages.  The arithmetic is that of the two stages one after the other.
+// The outputs of thread tt are the E positions n = tt mod TT.
+template <typename C, int LOGN, int E> constexpr bool fft_merges() {
+  constexpr int REM = LOGN % 3, LS = 1 << (3 * (LOGN / 3 - 1)), TT = (1 << LOGN) / E;
+  return REM != 0 && LS > 1 && TT <= LS && E >= 8 * (REM == 1 ? 2 : 4);
+}
+template <typename C, int LOGN, int E, int SIGN, class In, class Mid, class Out>
+__device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw, In&& in, Mid&& mid, Out&& out) {
+  constexpr int N = 1 << LOGN, TT = N / E, LS = 1 << (3 * (LOGN / 3 - 1)), R2 = LOGN % 3 == 1 ? 2 : 4;
+  constexpr int B = E / 8, NB0 = LS / TT, LS2 = 8 * LS;
+  static_assert(fft_merges<C, LOGN, E>() && B == NB0 * R2, "");
+  C a[E];
+#pragma unroll
+  for (int b = 0; b < B; ++b)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[b * 8 + r] = in(tt + TT * b, r * (N / 8));
+  mid();
+#pragma unroll
+  for (int b0 = 0; b0 < NB0; ++b0) {
+    const int j = tt + TT * b0;  // = t mod LS of the butterflies b0 + NB0 i
+    C w[7];
+    {
+      const C w1 = ldg_tw(&tw[j * (kTwN / LS2)]), w4 = ldg_tw(&tw[4 * j * (kTwN / LS2)]);
+      const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
+      w[0] = w1; w[1] = w2; w[2] = w3; w[3] = w4; w[4] = cmul(w4, w1); w[5] = cmul(w4, w2); w[6] = cmul(w4, w3);
+      if (SIGN > 0) {
+#pragma unroll
+        for (int r = 0; r < 7; ++r) w[r].y = -w[r].y;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R2; ++i) {
+      C* v = &a[(b0 + NB0 * i) * 8];
+#pragma unroll
+      for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[r - 1]);
+      dft_r<8, SIGN>(v);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int j2 = j + LS * r;
+      C v[R2];
+#pragma unroll
+      for (int i = 0; i < R2; ++i) {
+        v[i] = a[(b0 + NB0 * i) * 8 + r];
+        if (i > 0) {
+          C wr = ldg_tw(&tw[i * j2 * (kTwN / N)]);
+          if (SIGN > 0) wr.y = -wr.y;
+          v[i] = cmul(v[i], wr);
+        }
+      }
+      dft_r<R2, SIGN>(v);
+#pragma unroll
+      for (int i = 0; i < R2; ++i) out(j2, LS2 * i, v[i]);
+    }
+  }
 }
 
 // ---- two real rows through one complex FFT ---------------------------------

@@ -45,7 +45,8 @@ template <typename T> struct PassAArgs {
   int flags;
   int test_fault;   // 1: the staged u copy is replaced by a barrier that never completes (test of
                     // the bounded wait: no copy is issued, the wait gives up after 64 polls)
-  int variant;      // 1: the kernel variant with the other FFT width (complex64, N = 256 .. 1024)
+  int variant;      // 1: the kernel variant with the other FFT width (complex64, N = 256 .. 1024); 2: 32
+                    // elements per thread (T = I, complex64, N = 256)
   C* lowbuf;        // TV: [2][kLowK][M][CP] row DFTs of the components of t - u' at k2 < kLowK
                     // for the low-column correction of the split column pass; NULL: not formed
   T dct[64];        // orthonormal DCT-II, dct[k*8+n]
@@ -163,6 +164,12 @@ cudaError_t launch_dl_rescale(typename CT<T>::type* spec, int L, int N, T f, cud
 template <typename Tin> cudaError_t launch_embed_filters(const Tin* d, double* out, int L, int P, int N, cudaStream_t s);
 template <typename T>
 cudaError_t launch_theta_store(const SetupC<T>* th64, typename CT<T>::type* th, int L, int N, cudaStream_t s);
+
+// The same for T = I (the l1 prior, dictionary codes) and the row transforms alone (csrc/rowpass.cu);
+// kind: PRIOR_L1, ROWS_OUT or ROWS_IN.  rows: rows per CTA; elems: FFT elements per thread.
+int rowpass_rows(int N);
+template <typename T> int rowpass_elems(int N, int variant);
+template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, cudaStream_t s);
 
 template <typename T> int passA_rows(int N, int prior);
 template <typename T> size_t passA_smem(int N, int prior);

@@ -6,8 +6,8 @@
 //   1. loads the row half-spectra of x (written by pass B) and inverts the row
 //      DFT two rows at a time (one complex FFT z = x_a + i x_b for two real
 //      rows, so shared memory holds the tile as row pairs);
-//   2. applies the analysis operator T (anisotropic TV differences, 8x8
-//      orthonormal block DCT, or identity), the soft-threshold t-update
+//   2. applies the analysis operator T (TV differences or the 8x8 orthonormal
+//      block DCT; T = I is rowpass.cu), the soft-threshold t-update
 //      (Eq. solt_trans) and the dual update (Eq. subu_trans), writing u; every
 //      thread works on both rows of a pair, so shared-memory accesses are
 //      whole 8- or 16-byte pairs;
@@ -19,6 +19,7 @@
 
 #include "fft.cuh"
 #include "kernels.h"
+#include "reduce.cuh"
 
 namespace cip {
 
@@ -31,36 +32,9 @@ namespace {
 #define PASSA_TV_RT32 64
 #endif
 
-template <typename T>
-__device__ __forceinline__ void block_reduce_store(const T (&v)[kNPart], double* out) {
-  __shared__ double red[32][kNPart];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double s[kNPart];
-#pragma unroll
-  for (int i = 0; i < kNPart; ++i) {
-    double x = (double)v[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    s[i] = x;
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < kNPart; ++i) red[warp][i] = s[i];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    for (int i = 0; i < kNPart; ++i) {
-      double acc = 0.0;
-      for (int w = 0; w < nw; ++w) acc += red[w][i];
-      out[i] = acc;
-    }
-  }
-}
-
 // FFT elements per thread: 8 for complex64 up to N = 1024 (more warps per
 // tile), 16 otherwise (keeps the CTA within 1024 threads).
-// (complex64 DCT / l1 tiles at N = 512 take 16: one warp per row-pair FFT, whose stage
+// (complex64 DCT tiles at N = 512 take 16: one warp per row-pair FFT, whose stage
 // barriers are then warp syncs, while TV, which needs more registers for its halo rows,
 // takes 8.)  Variant V = 1 of a complex64 iteration kernel at N = 256 .. 1024 takes the other
 // of 8 and 16; the plan's autotuner times both inside whole iterations and keeps the faster.
@@ -69,7 +43,7 @@ template <typename T> constexpr int elems_a(int N, int prior, int V = 0) {
   return V == 1 ? 24 - e : e;
 }
 template <typename T> constexpr bool has_variant(int N, int prior) {
-  return sizeof(T) == 4 && N >= 256 && N <= 1024 && prior < ROWS_OUT && prior != PRIOR_WDCT;
+  return sizeof(T) == 4 && N >= 256 && N <= 1024 && (prior_is_tv(prior) || prior == PRIOR_DCT8);
 }
 
 // Pitch of the row-pair FFT buffers (complex elements): the padded FFT layout plus 4 slots from
@@ -97,12 +71,12 @@ template <typename T> constexpr int rows_for(int N, int prior) { return 8; }
 // isotropic 512^2 x 10 39.2 -> 30.2, 2048^2 x 3 302 -> 191 us.
 constexpr int tv_rows(int N) { return N >= 512 ? 8 : (N >= 256 ? 4 : 2); }
 
-// DCT and l1 tiles stage their R rows of u in shared memory with one TMA bulk
+// DCT tiles stage their R rows of u in shared memory with one TMA bulk
 // copy issued before the grid dependency (u does not depend on the preceding
 // column pass), when the staging area keeps the CTA within ~100 KB
 template <typename T> constexpr bool u_staged(int N, int prior, int R) {
   using C = typename CT<T>::type;
-  return !prior_is_tv(prior) && prior < ROWS_OUT &&
+  return !prior_is_tv(prior) &&
          (size_t)(R / 2) * zs_of(N) * sizeof(C) + (size_t)R * N * sizeof(T) <= 100 * 1024;
 }
 
@@ -212,21 +186,6 @@ __device__ __forceinline__ void shrink(T w, T u, T tau, T& t, T& un) {
   un = u + w - t;
 }
 
-template <typename T>
-__device__ __forceinline__ void acc_resid(T (&part)[kNPart], T w, T t, T un, const T* tprev, size_t g) {
-  // a thread sums a few dozen terms at most, so the plan's precision suffices here; the
-  // block and grid reductions run in double (FP64 issue is scarce on this part)
-  const T r = w - t;
-  part[0] = fma(r, r, part[0]);
-  part[1] = fma(w, w, part[1]);
-  part[2] = fma(t, t, part[2]);
-  part[3] = fma(un, un, part[3]);
-  if (tprev) {
-    const T dt = t - tprev[g];
-    part[4] = fma(dt, dt, part[4]);
-  }
-}
-
 // sums of 16 values per lane over the warp by recursive halving: at xor distance 16, 8, 4, 2 a lane
 // keeps one half of its values (the upper half when that bit of the lane is set) and adds its
 // partner's; then v[0] of lane l is the warp's sum of value l >> 1
@@ -277,7 +236,7 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
   static_assert(!USTAGE || (NPIN * ZS * sizeof(C)) % 16 == 0, "the TMA destination must be 16-byte aligned");
   constexpr bool TVSTAGE = tv_staged<T>(N, PRIOR);
   static_assert(!TVSTAGE || (NPIN * ZS * sizeof(C)) % 16 == 0, "the TMA destination must be 16-byte aligned");
-  // USTAGE: [R][N] rows r0 .. of u_in; TVSTAGE: [2][R + 1][N] rows r0 - 1 .. of both components
+  // USTAGE (DCT): [R][N] rows r0 .. of u_in; TVSTAGE: [2][R + 1][N] rows r0 - 1 .. of both components
   T* us = reinterpret_cast<T*>(zb + NPIN * ZS);
   __shared__ unsigned long long ubar;
 
@@ -285,8 +244,7 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
   const int nth = blockDim.x;
   const int m = blockIdx.y;
   const int r0 = blockIdx.x * R;
-  constexpr bool ROWXF = PRIOR >= ROWS_OUT;  // row transform only (read-back, wavelet chain)
-  const bool import_mode = PRIOR == ROWS_IN || (a.flags & PA_IMPORT) != 0;
+  const bool import_mode = (a.flags & PA_IMPORT) != 0;
   const bool resid = (a.flags & PA_RESID) != 0;
   const bool store_t = (a.flags & PA_STORE_T) != 0;
   const T tau = a.tau;
@@ -339,7 +297,7 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     __syncthreads();  // the barrier is initialised before anyone waits on it
   }
   // L2 prefetch of the u rows (and t_prev rows) read after the inverse FFT
-  if (!ROWXF && tid < 2 * NCOMP && !((USTAGE || TVSTAGE) && (tid & 1) == 0)) {
+  if (tid < 2 * NCOMP && !((USTAGE || TVSTAGE) && (tid & 1) == 0)) {
     const T* src = (tid & 1) ? tprev_rd : u_in;
     if (src) {
       const size_t comp = (size_t)(tid >> 1) * plane;
@@ -400,17 +358,6 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     }
     __syncthreads();
   }
-  if constexpr (PRIOR == ROWS_OUT) {
-    // x rows r0 .. r0 + R - 1 of map m into u_out ([maps][N][N])
-    for (int idx = tid; idx < NPIN * N; idx += nth) {
-      const int p = idx / N, n = idx - p * N;
-      const C z = zb[p * ZS + spad(n)];
-      u_out[(size_t)(r0 + 2 * p) * N + n] = z.x;
-      u_out[(size_t)(r0 + 2 * p + 1) * N + n] = z.y;
-    }
-    return;
-  }
-
   // 2. analysis operator, shrinkage, dual update; 3. q = qscale T^T (t - u')
   if constexpr (prior_is_tv(PRIOR)) {
     constexpr bool WALK = N >= 1024, LOW = LOGN == 11;
@@ -737,38 +684,6 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
 #pragma unroll
       for (int n = 0; n < 8; ++n) zb[p * ZS + spad(c0 + n)] = mk<C>(o[n].x * a.qscale, o[n].y * a.qscale);
     }
-  } else if constexpr (PRIOR == ROWS_IN) {
-    // q rows from real rows: zb = qscale (u_in[r0 + 2p], u_in[r0 + 2p + 1])
-    for (int idx = tid; idx < NPOUT * N; idx += nth) {
-      const int p = idx / N, n = idx - p * N;
-      zb[p * ZS + spad(n)] = mk<C>(u_in[(size_t)(r0 + 2 * p) * N + n] * a.qscale,
-                                   u_in[(size_t)(r0 + 2 * p + 1) * N + n] * a.qscale);
-    }
-  } else {  // PRIOR_L1: T = I
-    if constexpr (USTAGE) u_ok = mbar_wait_bounded(&ubar, 0, a.err, a.test_fault ? 64 : (1 << 22));
-    for (int idx = tid; idx < NPOUT * N; idx += nth) {
-      const int p = idx / N, c = idx - p * N;
-      const C z = zb[p * ZS + spad(c)];
-      const T w[2] = {z.x, z.y};
-      T q[2];
-#pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        const size_t g = (size_t)(r0 + 2 * p + s) * N + c;
-        const T uo = (USTAGE && u_ok) ? us[(2 * p + s) * N + c] : u_in[g];
-        T t, un;
-        if (import_mode) {
-          t = timp[g];
-          un = uo;
-        } else {
-          shrink(w[s], uo, tau, t, un);
-        }
-        u_out[g] = un;
-        if (resid) acc_resid(part, import_mode ? T(0) : w[s], t, un, tprev_rd, g);
-        if (store_t) tprev[g] = t;
-        q[s] = (t - un) * a.qscale;
-      }
-      zb[p * ZS + spad(c)] = mk<C>(q[0], q[1]);
-    }
   }
   __syncthreads();
 
@@ -860,9 +775,7 @@ template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int
     case PRIOR_TV: return dispatchA<T, PRIOR_TV>(a, N, s);
     case PRIOR_TV_ISO: return dispatchA<T, PRIOR_TV_ISO>(a, N, s);
     case PRIOR_DCT8: return dispatchA<T, PRIOR_DCT8>(a, N, s);
-    case PRIOR_L1: return dispatchA<T, PRIOR_L1>(a, N, s);
-    case ROWS_OUT: return dispatchA<T, ROWS_OUT>(a, N, s);
-    case ROWS_IN: return dispatchA<T, ROWS_IN>(a, N, s);
+    case PRIOR_L1: return launch_rowpass<T>(a, N, PRIOR_L1, s);
     default: return cudaErrorInvalidValue;
   }
 }
