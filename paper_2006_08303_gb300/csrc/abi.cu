@@ -191,10 +191,11 @@ template <typename T> void fill_dct(T* d) {
   std::memcpy(d, t.v, sizeof(t.v));
 }
 
-// exp(-2 pi i k / 2048) with the angle reduced exactly through octant symmetry
+// exp(-2 pi i k / 2048) with the angle reduced exactly through octant symmetry, and behind them the
+// same values once per FFT stage in the order the stage reads them (tw_stage)
 void twiddles(std::vector<double>& re, std::vector<double>& im) {
-  re.resize(kTwN);
-  im.resize(kTwN);
+  re.resize(kTwAll);
+  im.resize(kTwAll);
   for (int k = 0; k < kTwN; ++k) {
     const double a = 2.0 * M_PI * (double)k / (double)kTwN;
     re[k] = std::cos(a);
@@ -206,6 +207,14 @@ void twiddles(std::vector<double>& re, std::vector<double>& im) {
     re[k] = (q == 0) ? 1.0 : (q == 2 ? -1.0 : 0.0);
     im[k] = (q == 1) ? -1.0 : (q == 3 ? 1.0 : 0.0);
   }
+  const int stages[][2] = {{8, 8}, {8, 64}, {2, 64}, {2, 512}, {4, 64}, {4, 512}};  // radix, LS
+  for (auto& st : stages)
+    for (int r = 1; r < st[0]; ++r)
+      for (int j = 0; j < st[1]; ++j) {
+        const int d = tw_stage(st[0], st[1]) + (r - 1) * st[1] + j, k = r * j * (kTwN / (st[0] * st[1]));
+        re[d] = re[k];
+        im[d] = im[k];
+      }
 }
 
 // Plan buffers use the stream-ordered allocator on the stream of the call that creates or frees
@@ -1228,7 +1237,7 @@ size_t cip_plan_bytes(int N, int K, int M, cip_dtype dtype, cip_prior prior) {
   b += (size_t)M * (M + 1) / 2 * N * P * 16;  // FP64 copy of pinv (data term at set_measurements)
   b += 3 * nc * M * real;                     // u[2], tprev
   b += (size_t)K * M * N * P * 16;            // FP64 PSF spectra
-  b += (size_t)kTwN * (16 + 2 * e) + N * 8;   // tables
+  b += (size_t)kTwAll * (16 + 2 * e) + N * 8;   // tables
   b += (size_t)(N / 2) * M * kNPart * 8 + 4096;
   if (prior == CIP_PRIOR_WDCT) b += 5 * M * real / 2 + (size_t)M * M * e;  // wavelet work planes, DCT matrix
   return b;
@@ -1292,8 +1301,8 @@ cip_status cip_plan_create_on_stream(cip_plan** out, int N, int K, int M, cip_dt
   ALLOC(p->xh, col_elems(p, M) * ce);
   ALLOC(p->qh, col_elems(p, M) * ce);
   ALLOC(p->bhat, col_elems(p, M) * ce);
-  ALLOC(p->tw, (size_t)kTwN * ce);
-  ALLOC(p->tw64, (size_t)kTwN * 16);  // complex double-float (complex64 plans) or complex128
+  ALLOC(p->tw, (size_t)kTwAll * ce);
+  ALLOC(p->tw64, (size_t)kTwAll * 16);  // complex double-float (complex64 plans) or complex128
   ALLOC(p->gs, (size_t)N * sizeof(double));
   ALLOC(p->resid, (kNPart + 2) * sizeof(double));
   ALLOC(p->conv, 2 * sizeof(int));  // [0] converged, [1] a kernel's bounded wait gave up
@@ -1302,10 +1311,10 @@ cip_status cip_plan_create_on_stream(cip_plan** out, int N, int K, int M, cip_dt
 #undef ALLOC
   std::vector<double> re, im;
   twiddles(re, im);
-  std::vector<double2> t64(kTwN);
-  std::vector<float2> t32(kTwN);
-  std::vector<cdf> tdf(kTwN);
-  for (int k = 0; k < kTwN; ++k) {
+  std::vector<double2> t64(kTwAll);
+  std::vector<float2> t32(kTwAll);
+  std::vector<cdf> tdf(kTwAll);
+  for (int k = 0; k < kTwAll; ++k) {
     t64[k] = make_double2(re[k], im[k]);
     tdf[k].x = df64_from_host(re[k]);
     tdf[k].y = df64_from_host(im[k]);
@@ -1320,11 +1329,11 @@ cip_status cip_plan_create_on_stream(cip_plan** out, int N, int K, int M, cip_dt
   gs[0] = 0.0;
   cudaError_t e = cudaStreamSynchronize(p->ast);  // buffers valid on every stream from here on
   if (e == cudaSuccess)
-    e = dtype == CIP_F64 ? cudaMemcpy(p->tw64, t64.data(), kTwN * sizeof(double2), cudaMemcpyHostToDevice)
-                         : cudaMemcpy(p->tw64, tdf.data(), kTwN * sizeof(cdf), cudaMemcpyHostToDevice);
+    e = dtype == CIP_F64 ? cudaMemcpy(p->tw64, t64.data(), kTwAll * sizeof(double2), cudaMemcpyHostToDevice)
+                         : cudaMemcpy(p->tw64, tdf.data(), kTwAll * sizeof(cdf), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = dtype == CIP_F64 ? cudaMemcpy(p->tw, t64.data(), kTwN * sizeof(double2), cudaMemcpyHostToDevice)
-                         : cudaMemcpy(p->tw, t32.data(), kTwN * sizeof(float2), cudaMemcpyHostToDevice);
+    e = dtype == CIP_F64 ? cudaMemcpy(p->tw, t64.data(), kTwAll * sizeof(double2), cudaMemcpyHostToDevice)
+                         : cudaMemcpy(p->tw, t32.data(), kTwAll * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->gs, gs.data(), N * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cip_plan_destroy(p);
@@ -2003,7 +2012,7 @@ size_t plan_resident_bytes(int N, int K, int M, cip_dtype dtype, cip_prior prior
   b += npk * H * CP * c;                      // factor
   b += (size_t)M * H * CP * c;                // column buffer of the split form
   b += 3 * nc * (size_t)M * N * N * e;        // u (two), t_prev
-  b += (size_t)kTwN * (16 + c) + N * 8 + (size_t)(N / 2) * M * kNPart * 8 + 8192;
+  b += (size_t)kTwAll * (16 + c) + N * 8 + (size_t)(N / 2) * M * kNPart * 8 + 8192;
   if (prior == CIP_PRIOR_WDCT) b += 5 * (size_t)M * N * N * e / 2 + (size_t)M * M * e;  // wavelet work planes
   return b;
 }

@@ -8,7 +8,18 @@
 
 namespace cip {
 
-constexpr int kTwN = 2048;  // twiddle table length (max FFT length)
+constexpr int kTwN = 2048;  // length of the twiddle table exp(-2 pi i k / kTwN) (max FFT length)
+// Behind it, the twiddles of every FFT stage that multiplies by some, laid out as the stage reads
+// them: exp(-2 pi i r j / (LS R)) at tw_stage(R, LS) + (r - 1) LS + j.  The lanes of a warp then read
+// consecutive entries; from the table above they read every (kTwN / (LS R))-th one, up to 32 cache
+// lines per load, which made twiddle loads the largest user of the load/store pipe (about half of the
+// 80% it ran at in the 256-point row pass).  With these tables: that pass over 160 maps 57.9 -> 39.9 us,
+// one iteration at 512^2 x 10 with the DCT prior 41.0 -> 37.1, 1024^2 x 10 198.7 -> 181.1 us.
+constexpr int tw_stage(int R, int LS) {
+  return kTwN + (R == 8 ? (LS == 8 ? 0 : 56)
+                        : (R == 2 ? 504 + (LS == 64 ? 0 : 64) : 1080 + (LS == 64 ? 0 : 192)));
+}
+constexpr int kTwAll = tw_stage(4, 512) + 3 * 512;
 
 // complex type per real type: float -> float2 (complex64), double -> double2 (complex128)
 template <typename T> struct CT;

@@ -9,8 +9,9 @@
 // not a multiple of 3).  Stage s reads x[t + r N/R], multiplies by the
 // twiddles w_{Ls R}^{r (t mod Ls)}, does a radix-R DFT in registers and
 // writes y[(t/Ls) Ls R + t mod Ls + r Ls] (autosorting Stockham, natural
-// order in and out).  Twiddles come from a table of exp(-2 pi i k / 2048)
-// computed on the host in FP64 and rounded once; a radix-8 butterfly loads
+// order in and out).  Twiddles come from tables computed on the host in FP64
+// and rounded once, one per stage in the order the stage reads them
+// (tw_stage); a radix-8 butterfly loads
 // only w^j and w^4j and forms w^2j, w^3j, w^5j, w^6j, w^7j by at most two
 // complex products (a few ulp), since table loads stalled the stages.
 #pragma once
@@ -141,12 +142,12 @@ __device__ __forceinline__ void stockham_stage(C* buf, int f, int tt, const C* _
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
       if constexpr (R == 8) {
-        const C w1 = ldg_tw(&tw[j * (kTwN / (LS * R))]), w4 = ldg_tw(&tw[4 * j * (kTwN / (LS * R))]);
+        const C w1 = ldg_tw(&tw[tw_stage(R, LS) + j]), w4 = ldg_tw(&tw[tw_stage(R, LS) + 3 * LS + j]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
         C* ww = &w[b * (R - 1)];
         ww[0] = w1; ww[1] = w2; ww[2] = w3; ww[3] = w4; ww[4] = cmul(w4, w1); ww[5] = cmul(w4, w2); ww[6] = cmul(w4, w3);
       } else {
-        for (int r = 1; r < R; ++r) w[b * (R - 1) + r - 1] = ldg_tw(&tw[r * j * (kTwN / (LS * R))]);
+        for (int r = 1; r < R; ++r) w[b * (R - 1) + r - 1] = ldg_tw(&tw[tw_stage(R, LS) + (r - 1) * LS + j]);
       }
     }
   }
@@ -235,12 +236,12 @@ __device__ __forceinline__ void fft_stage_io(int tt, const C* __restrict__ tw, I
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
       if constexpr (R == 8) {
-        const C w1 = ldg_tw(&tw[j * (kTwN / (LS * R))]), w4 = ldg_tw(&tw[4 * j * (kTwN / (LS * R))]);
+        const C w1 = ldg_tw(&tw[tw_stage(R, LS) + j]), w4 = ldg_tw(&tw[tw_stage(R, LS) + 3 * LS + j]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
         C* ww = &w[b * (R - 1)];
         ww[0] = w1; ww[1] = w2; ww[2] = w3; ww[3] = w4; ww[4] = cmul(w4, w1); ww[5] = cmul(w4, w2); ww[6] = cmul(w4, w3);
       } else {
-        for (int r = 1; r < R; ++r) w[b * (R - 1) + r - 1] = ldg_tw(&tw[r * j * (kTwN / (LS * R))]);
+        for (int r = 1; r < R; ++r) w[b * (R - 1) + r - 1] = ldg_tw(&tw[tw_stage(R, LS) + (r - 1) * LS + j]);
       }
     }
   }
@@ -258,7 +259,7 @@ __device__ __forceinline__ void fft_stage_io(int tt, const C* __restrict__ tw, I
     if constexpr (LS > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        C wr = HOIST ? w[b * (R - 1) + r - 1] : ldg_tw(&tw[r * j * (kTwN / (LS * R))]);
+        C wr = HOIST ? w[b * (R - 1) + r - 1] : ldg_tw(&tw[tw_stage(R, LS) + (r - 1) * LS + j]);
         if (SIGN > 0) wr.y = -wr.y;
         a[b * R + r] = cmul(a[b * R + r], wr);
       }
@@ -332,7 +333,7 @@ __device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw
     const int j = tt + TT * b0;  // = t mod LS of the butterflies b0 + NB0 i
     C w[7];
     {
-      const C w1 = ldg_tw(&tw[j * (kTwN / LS2)]), w4 = ldg_tw(&tw[4 * j * (kTwN / LS2)]);
+      const C w1 = ldg_tw(&tw[tw_stage(8, LS) + j]), w4 = ldg_tw(&tw[tw_stage(8, LS) + 3 * LS + j]);
       const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
       w[0] = w1; w[1] = w2; w[2] = w3; w[3] = w4; w[4] = cmul(w4, w1); w[5] = cmul(w4, w2); w[6] = cmul(w4, w3);
       if (SIGN > 0) {
@@ -355,7 +356,7 @@ __device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw
       for (int i = 0; i < R2; ++i) {
         v[i] = a[(b0 + NB0 * i) * 8 + r];
         if (i > 0) {
-          C wr = ldg_tw(&tw[i * j2 * (kTwN / N)]);
+          C wr = ldg_tw(&tw[tw_stage(R2, LS2) + (i - 1) * LS2 + j2]);
           if (SIGN > 0) wr.y = -wr.y;
           v[i] = cmul(v[i], wr);
         }

@@ -38,7 +38,7 @@ template <typename T> struct PassAArgs {
   const T* t_imp;   // [M][ncomp][N][N] (IMPORT)
   double* partials; // [gridDim.y * gridDim.x][kNPart] (RESID)
   int* err;         // set to 1 when a bounded wait on an asynchronous copy gives up
-  const C* tw;      // twiddle table, kTwN entries
+  const C* tw;      // twiddle tables, kTwAll entries
   int M;
   T tau;            // lambda / rho
   T qscale;         // rho / 2 (the 1/2 of the pair extraction is folded here)

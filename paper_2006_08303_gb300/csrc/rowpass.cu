@@ -11,7 +11,8 @@
 // Bound by shared-memory wavefronts (the general kernel ran its LSU pipe at 80% here): 12 accesses per
 // complex value at N = 256, E = 32, against 21 with the rows in shared memory and unmerged stages.
 // The l1 pass before (rows through shared memory) and now: 160 maps of 256^2 66.9 -> 57.9 us, 96 maps
-// 44.0 -> 37.5, 512^2 x 10 22.0 -> 19.4 us.
+// 44.0 -> 37.5, 512^2 x 10 22.0 -> 19.4 us; with the per-stage twiddle tables of common.cuh 39.9, 26.9
+// and 16.6 us.
 #include "fft.cuh"
 #include "kernels.h"
 #include "reduce.cuh"
