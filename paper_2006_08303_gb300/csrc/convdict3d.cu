@@ -11,8 +11,8 @@
 //       c_l = conj(Theta_l(kappa)) X(kappa) + G_l(kappa),   G = F_2D rho (t - u) / N^2,
 //       v = (c - conj(Theta) (Theta^T c) / (rho + ||Theta||^2)) / rho   (Sherman-Morrison, R10),
 //       V_{m,l} = (1/M) sum_kappa e^{+2 pi i m kappa / M} v_l(kappa)     (back to channels).
-// One CTA holds BB bins of one column k2 and all M channel frequencies: thread (b, kappa) owns
-// one 3D bin; the M-point DFTs along the channels go through shared memory.  The channel-domain
+// One CTA holds BB bins of one column k2 and all M channel frequencies; the M-point DFTs along the
+// channels are taken in registers.  The channel-domain
 // spectra stay in the 2D dictionary's layout ([k2][m*L + l][k1]), so the column DFTs around the
 // solve and the l1 pass on the code maps are the 2D path's kernels.
 #include "fft.cuh"
@@ -22,7 +22,7 @@ namespace cip {
 
 namespace {
 
-// bins per CTA: the shared tile [M][L][BB] complex stays within ~96 KB
+// bins per CTA of the import kernel: the shared tile [M][L][BB] complex stays within ~96 KB
 template <typename T> int cd3_bins(int M, int L) {
   const size_t per = (size_t)M * L * sizeof(typename CT<T>::type);
   if (32 * per <= 96 * 1024) return 32;
@@ -30,30 +30,75 @@ template <typename T> int cd3_bins(int M, int L) {
   return 8;
 }
 
-template <typename T, int LMAX>
-__global__ void __launch_bounds__(512) cd3_solve_kernel(CD3Args<T> a) {
+// M-point DFT in registers (SIGN = -1 forward, +1 inverse, unnormalised): the inputs m and M - m are
+// combined into their sum and difference, which only the cosines and only the sines multiply, and the
+// outputs k and M - k share both sums: M^2 real multiply-adds instead of 4 M^2.  w[j] = exp(-2 pi i j / M)
+// is a kernel parameter and every index a constant, so the factors are constant-bank operands.
+template <int M, int SIGN, typename T, typename C>
+__device__ __forceinline__ void chan_dft(const C* w, const C (&in)[M], C (&out)[M]) {
+  constexpr int HM = (M - 1) / 2;
+  C s[HM > 0 ? HM : 1], d[HM > 0 ? HM : 1];
+  C o0 = in[0];
+#pragma unroll
+  for (int m = 1; m <= HM; ++m) {
+    s[m - 1] = cadd(in[m], in[M - m]);
+    d[m - 1] = csub(in[m], in[M - m]);
+    o0 = cadd(o0, s[m - 1]);
+  }
+  if constexpr (M % 2 == 0) o0 = cadd(o0, in[M / 2]);
+  out[0] = o0;
+#pragma unroll
+  for (int k = 1; k <= M / 2; ++k) {
+    C A = in[0], B = mk<C>(0.0, 0.0);
+    if constexpr (M % 2 == 0) A = (k & 1) ? csub(A, in[M / 2]) : cadd(A, in[M / 2]);
+#pragma unroll
+    for (int m = 1; m <= HM; ++m) {
+      const T c = w[(k * m) % M].x, sn = -w[(k * m) % M].y;
+      A.x = fma(c, s[m - 1].x, A.x);
+      A.y = fma(c, s[m - 1].y, A.y);
+      B.x = fma(sn, d[m - 1].x, B.x);
+      B.y = fma(sn, d[m - 1].y, B.y);
+    }
+    if (2 * k == M) {  // the sines vanish
+      out[k] = A;
+    } else {
+      const C p = cpack<C>(A.x + B.y, A.y - B.x), q = cpack<C>(A.x - B.y, A.y + B.x);  // A - iB, A + iB
+      out[k] = SIGN < 0 ? p : q;
+      out[M - k] = SIGN < 0 ? q : p;
+    }
+  }
+}
+
+// BB bins of one column per CTA, threads as (group, bin).  The channel DFTs are taken whole by one
+// thread per (map, bin), in registers; shared memory carries the tile between the layouts (map, bin)
+// and (channel frequency, bin): two writes and two reads per value.  The previous form had a thread per
+// (channel frequency, bin) form its own output of every DFT, 2 M shared-memory reads per value and
+// M times the arithmetic (53 M warp instructions at 256^2 x 16 with 6 filters).  Column pass there (the
+// two column DFTs of the maps included) 94.8 -> 55.4 us.
+constexpr int kCd3Threads = 256;
+template <typename T, int M>
+__global__ void __launch_bounds__(kCd3Threads, sizeof(T) == 4 ? 2 : 1) cd3_solve_kernel(const CD3Args<T> a, int BB) {
   using C = typename CT<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = a.N, M = a.M, L = a.L, BB = blockDim.x;
-  const int CP = col_pitch(N);
-  const int b = threadIdx.x, m = threadIdx.y;  // m: channel index, then channel frequency kappa
+  const int N = a.N, L = a.L, CP = col_pitch(N);
+  const int b = threadIdx.x % BB, grp = threadIdx.x / BB, ngrp = kCd3Threads / BB;
   const int k1 = blockIdx.x * BB + b, k2 = blockIdx.y;
-  C* gs = reinterpret_cast<C*>(smem_raw);            // [M][L][BB]: G, then v
-  C* xs = gs + (size_t)M * L * BB;                    // [M][BB]: x, then p3
-  C* wt = xs + (size_t)M * BB;                        // [M][M]: e^{-2 pi i k m / M} (symmetric in k, m)
-  const int npk = M * (M + 1) / 2;
-  for (int i = m * BB + b; i < M * M; i += M * BB) wt[i] = a.w[((i / M) * (i % M)) % M];
-  // 1. G of channel m, and the channel's x-update (as in the 2D dictionary: p from the previous v)
-  C* gcol = a.colbuf + ((size_t)k2 * M * L + (size_t)m * L) * CP + k1;
-  for (int l = 0; l < L; ++l) gs[((size_t)m * L + l) * BB + b] = gcol[(size_t)l * CP];
-  {
+  C* gs = reinterpret_cast<C*>(smem_raw) + b;  // [M (kappa)][L][BB]: G, then v
+  C* xs = gs + (size_t)M * L * BB;             // [M][BB]: x, then p3
+  C* Xs = xs + (size_t)M * BB;                 // [M][BB]: X(kappa)
+  constexpr int npk = M * (M + 1) / 2;
+  C* gcol = a.colbuf + (size_t)k2 * M * L * CP + k1;
+  grid_dep_wait();
+  grid_dep_launch();
+  // 1. the channels' x-update (as in the 2D dictionary: p from the previous v)
+  for (int m = grp; m < M; m += ngrp) {
     const C* pin = a.p_in + (size_t)k2 * M * CP + k1;
     const C* pcol = a.pinv + binp(k2, 0, k1, npk, N);  // plane stride kBinBlock
     C acc = mk<C>(0.0, 0.0);
+#pragma unroll
     for (int j = 0; j < M; ++j) {
       const int i0 = min(m, j), j0 = max(m, j);
-      const int pk = i0 * M - (i0 * (i0 - 1)) / 2 + (j0 - i0);
-      const C pij = pcol[(size_t)pk * kBinBlock];
+      const C pij = pcol[(size_t)(i0 * M - (i0 * (i0 - 1)) / 2 + (j0 - i0)) * kBinBlock];
       const C pj = pin[(size_t)j * CP];
       if (m <= j) cfma(acc, pij, pj);
       else cfmac(acc, pij, pj);
@@ -62,63 +107,74 @@ __global__ void __launch_bounds__(512) cd3_solve_kernel(CD3Args<T> a) {
     x.x += a.n2 * acc.x;
     x.y += a.n2 * acc.y;
     a.xcol[((size_t)k2 * M + m) * CP + k1] = x;
-    xs[(size_t)m * BB + b] = x;
+    xs[m * BB] = x;
   }
   __syncthreads();
-  // 2. thread (b, kappa = m): DFTs along the channels, Sherman-Morrison in the 3D bin
-  const int kap = m;
-  C X = mk<C>(0.0, 0.0);
-  const C* wk = wt + (size_t)kap * M;  // the same row for the whole warp (one kappa per warp row)
-  for (int s = 0; s < M; ++s) cfma(X, wk[s], xs[(size_t)s * BB + b]);
-  const C* th = a.theta + ((size_t)k2 * M * L + (size_t)kap * L) * CP + k1;
-  C c[LMAX];
-  C sdot = mk<C>(0.0, 0.0);
-  T nrm = T(0);
-#pragma unroll
-  for (int l = 0; l < LMAX; ++l) {
+  // 2. DFTs along the channels: item l < L is map l's G, item L the image
+  for (int l = grp; l <= L; l += ngrp) {
+    C in[M], out[M];
     if (l < L) {
-      C g = mk<C>(0.0, 0.0);
-      for (int mm = 0; mm < M; ++mm) cfma(g, wk[mm], gs[((size_t)mm * L + l) * BB + b]);
-      const C t = th[(size_t)l * CP];
-      cfmac(g, t, X);
-      c[l] = g;
-      cfma(sdot, t, g);
+#pragma unroll
+      for (int m = 0; m < M; ++m) in[m] = gcol[((size_t)m * L + l) * CP];
+    } else {
+#pragma unroll
+      for (int m = 0; m < M; ++m) in[m] = xs[m * BB];
+    }
+    chan_dft<M, -1, T>(a.w, in, out);
+#pragma unroll
+    for (int k = 0; k < M; ++k) (l < L ? gs[((size_t)k * L + l) * BB] : Xs[k * BB]) = out[k];
+  }
+  __syncthreads();
+  // 3. Sherman-Morrison in the 3D bin (kappa, bin); c_l is formed again in the second loop
+  for (int kap = grp; kap < M; kap += ngrp) {
+    const C X = Xs[kap * BB];
+    const C* th = a.theta + ((size_t)k2 * M * L + (size_t)kap * L) * CP + k1;
+    C* g = gs + (size_t)kap * L * BB;
+    C sdot = mk<C>(0.0, 0.0);
+    T nrm = T(0);
+#pragma unroll 6
+    for (int l = 0; l < L; ++l) {
+      const C t = __ldg(th + (size_t)l * CP);
+      C c = g[l * BB];
+      cfmac(c, t, X);
+      cfma(sdot, t, c);
       nrm += t.x * t.x + t.y * t.y;
     }
-  }
-  const T inv_rho = T(1) / a.rho;
-  const T den = T(1) / (a.rho + nrm);
-  const C coef = mk<C>(sdot.x * den, sdot.y * den);
-  C p3 = mk<C>(0.0, 0.0);
-#pragma unroll
-  for (int l = 0; l < LMAX; ++l) {
-    if (l < L) {
-      const C t = th[(size_t)l * CP];
-      C v = c[l];
+    const T inv_rho = T(1) / a.rho;
+    const T den = T(1) / (a.rho + nrm);
+    const C coef = mk<C>(sdot.x * den, sdot.y * den);
+    C p3 = mk<C>(0.0, 0.0);
+#pragma unroll 6
+    for (int l = 0; l < L; ++l) {
+      const C t = __ldg(th + (size_t)l * CP);
+      C v = g[l * BB];
+      cfmac(v, t, X);
       v.x -= t.x * coef.x + t.y * coef.y;
       v.y -= t.x * coef.y - t.y * coef.x;
       v.x *= inv_rho;
       v.y *= inv_rho;
-      c[l] = v;
+      g[l * BB] = v;
       cfma(p3, t, v);
     }
+    xs[kap * BB] = p3;
   }
-  __syncthreads();  // every thread has read G and x
-#pragma unroll
-  for (int l = 0; l < LMAX; ++l)
-    if (l < L) gs[((size_t)kap * L + l) * BB + b] = c[l];
-  xs[(size_t)kap * BB + b] = p3;
   __syncthreads();
-  // 3. thread (b, m): back to the channels (inverse DFT along kappa, 1/M)
+  // 4. back to the channels (inverse DFT along kappa, 1/M): the maps, and p
   const T invM = T(1) / (T)M;
-  C p = mk<C>(0.0, 0.0);
-  const C* wm = wt + (size_t)m * M;
-  for (int k = 0; k < M; ++k) cfmac(p, wm[k], xs[(size_t)k * BB + b]);
-  a.p_out[((size_t)k2 * M + m) * CP + k1] = mk<C>(p.x * invM, p.y * invM);
-  for (int l = 0; l < L; ++l) {
-    C v = mk<C>(0.0, 0.0);
-    for (int k = 0; k < M; ++k) cfmac(v, wm[k], gs[((size_t)k * L + l) * BB + b]);
-    gcol[(size_t)l * CP] = mk<C>(v.x * invM, v.y * invM);
+  for (int l = grp; l <= L; l += ngrp) {
+    C in[M], out[M];
+    if (l < L) {
+#pragma unroll
+      for (int k = 0; k < M; ++k) in[k] = gs[((size_t)k * L + l) * BB];
+    } else {
+#pragma unroll
+      for (int k = 0; k < M; ++k) in[k] = xs[k * BB];
+    }
+    chan_dft<M, +1, T>(a.w, in, out);
+    C* dst = l < L ? gcol + (size_t)l * CP : a.p_out + (size_t)k2 * M * CP + k1;
+    const size_t stride = (l < L ? (size_t)L : (size_t)1) * CP;
+#pragma unroll
+    for (int m = 0; m < M; ++m) dst[m * stride] = cpack<C>(out[m].x * invM, out[m].y * invM);
   }
 }
 
@@ -198,19 +254,28 @@ template <typename T> size_t cd3_smem(int M, int L, int BB) {
 
 }  // namespace
 
+namespace {
+template <typename T, int M> cudaError_t launch_cd3_m(const CD3Args<T>& a, cudaStream_t s) {
+  auto bytes = [&](int BB) { return ((size_t)M * a.L + 2 * M) * BB * sizeof(typename CT<T>::type); };
+  const int BB = bytes(32) <= 200 * 1024 ? 32 : 16;  // 16: complex128 with M L > 384
+  auto k = cd3_solve_kernel<T, M>;
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3(a.N / BB, a.N / 2 + 1), dim3(kCd3Threads), bytes(BB), s, 0, a, BB);
+}
+}  // namespace
+
 template <typename T> cudaError_t launch_cd3_solve(const CD3Args<T>& a, cudaStream_t s) {
-  if (a.L > 32 || a.M > 16) return cudaErrorInvalidValue;
-  const int BB = cd3_bins<T>(a.M, a.L);
-  const size_t sm = cd3_smem<T>(a.M, a.L, BB);
-  const dim3 grid(a.N / BB, a.N / 2 + 1), block(BB, a.M);
-  auto k8 = cd3_solve_kernel<T, 8>;
-  auto k32 = cd3_solve_kernel<T, 32>;
-  auto k = a.L <= 8 ? k8 : k32;
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+  if (a.L < 1 || a.L > 32) return cudaErrorInvalidValue;
+  switch (a.M) {
+#define CD3_CASE(m) \
+  case m: return launch_cd3_m<T, m>(a, s);
+    CD3_CASE(1) CD3_CASE(2) CD3_CASE(3) CD3_CASE(4) CD3_CASE(5) CD3_CASE(6) CD3_CASE(7) CD3_CASE(8)
+    CD3_CASE(9) CD3_CASE(10) CD3_CASE(11) CD3_CASE(12) CD3_CASE(13) CD3_CASE(14) CD3_CASE(15) CD3_CASE(16)
+#undef CD3_CASE
+    default: return cudaErrorInvalidValue;
   }
-  return launch_plain(k, grid, block, sm, s, a);
 }
 
 template <typename T>
