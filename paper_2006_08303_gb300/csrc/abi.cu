@@ -298,8 +298,8 @@ template <typename T> cip_status reset_state(cip_plan* p, cudaStream_t s) {
   CIP_CUDA(p, cudaMemsetAsync(p->xh, 0, col_elems(p, S) * sizeof(C), s));
   CIP_CUDA(p, cudaMemsetAsync(p->qh, 0, col_elems(p, S) * sizeof(C), s));
   CIP_CUDA(p, cudaMemsetAsync(p->conv, 0, 2 * sizeof(int), s));
+  // (the other u buffer is written before it is read)
   CIP_CUDA(p, cudaMemsetAsync(p->u[0], 0, real_elems(p, S) * nc * sizeof(T), s));
-  CIP_CUDA(p, cudaMemsetAsync(p->u[1], 0, real_elems(p, S) * nc * sizeof(T), s));
   CIP_CUDA(p, cudaMemsetAsync(p->tprev, 0, real_elems(p, S) * nc * sizeof(T), s));
   if (p->lowbuf) CIP_CUDA(p, cudaMemsetAsync(p->lowbuf, 0, 2 * low_elems(p) * sizeof(C), s));
   if (is_cd(p)) {
@@ -440,7 +440,7 @@ template <typename T> cip_status do_set_dictionary(cip_plan* p, const void* d, c
   if (e == cudaSuccess)
     e = p->Q > 0 ? launch_embed_filters3d<T>(static_cast<const T*>(dd), emb, p->L, p->Q, p->Pf, p->M, p->N, s)
                  : launch_embed_filters<T>(static_cast<const T*>(dd), emb, p->L, p->Pf, p->N, s);
-  if (e == cudaSuccess) e = launch_row_r2c<R, double>(emb, th64, p->N, planes * p->N, R(1.0f), setup_buf<T>(p->tw64), s);
+  if (e == cudaSuccess) e = launch_row_r2c<R, double>(emb, th64, p->N, planes * p->N, setup_buf<T>(p->tw64), s);
   if (e == cudaSuccess) e = launch_col_c2c<R>(th64, p->N, planes, -1, setup_buf<T>(p->tw64), s);
   if (e == cudaSuccess)
     e = p->Q > 0 ? launch_theta3_store<T>(th64, static_cast<C*>(p->theta), static_cast<const double2*>(p->w3), p->L,
@@ -492,7 +492,7 @@ template <typename T> cip_status do_set_psfs(cip_plan* p, const void* h, cudaStr
   const int nrows = p->K * p->M * p->N;
   SetupC<T>* lam = setup_buf<T>(p->lam64);
   const SetupC<T>* tw = setup_buf<T>(p->tw64);
-  CIP_LAUNCH(p, (launch_row_r2c<R, T>(static_cast<const T*>(dh), lam, p->N, nrows, R(1.0f), tw, s)));
+  CIP_LAUNCH(p, (launch_row_r2c<R, T>(static_cast<const T*>(dh), lam, p->N, nrows, tw, s)));
   CIP_LAUNCH(p, launch_col_c2c<R>(lam, p->N, p->K * p->M, -1, tw, s));
   p->have_psfs = true;
   r = form_factor<T>(p, s);
@@ -530,7 +530,7 @@ template <typename T> cip_status do_set_y(cip_plan* p, const void* y, cudaStream
   if (!fs->lam64 || !fs->pinv64) return fail(p, CIP_ERR_STATE, "the PSF spectra were released (cip_set_psfs again)");
   CIP_CUDA(p, cudaMallocAsync((void**)&yhat, half_elems(p, p->K) * sizeof(SetupC<T>), s));
   const SetupC<T>* tw = setup_buf<T>(p->tw64);
-  cudaError_t e = launch_row_r2c<R, T>(static_cast<const T*>(dy), yhat, p->N, p->K * p->N, R(1.0f), tw, s);
+  cudaError_t e = launch_row_r2c<R, T>(static_cast<const T*>(dy), yhat, p->N, p->K * p->N, tw, s);
   if (e == cudaSuccess) e = launch_col_c2c<R>(yhat, p->N, p->K, -1, tw, s);
   if (e == cudaSuccess) e = form_data_term<T>(p, yhat, s);
   if (e == cudaSuccess) p->launches += 3;

@@ -495,19 +495,38 @@ __global__ void __launch_bounds__(32) factor_pinv_kernel(const SetupC<Tout>* __r
 // iterations, so the ill-conditioned product with Psi^{-1} (cancellation at
 // bins where the PSFs are nearly dependent) is taken once at high precision and
 // the per-iteration column pass only adds Psi^{-1} rho F T^H (t - u).
+// Thread = bin.  The K M PSF spectra and M (M + 1) / 2 factor entries of a bin are read once, in plane
+// order, in chunks (a measurement row, a row of the packed triangle); each thread copies the next
+// chunk asynchronously into its own slots (no barrier) while it works on the present one.  With plain
+// loads a row's loads and its double-float arithmetic took turns: 202 -> 120 us at 512^2 x 10, 611 -> 483 at
+// 1024^2 x 10, 157 -> 116 at 2048^2 x 3, 254 -> 148 at 256^2 x 16.  Now bound by that arithmetic and the
+// register count of its two accumulators per channel.
+constexpr int kRhsThreads = 128;
 template <typename Tout, int MMAX>
-__global__ void __launch_bounds__(128) rhs_kernel(const SetupC<Tout>* __restrict__ lam,
-                                                  const SetupC<Tout>* __restrict__ yhat,
-                                                  const SetupC<Tout>* __restrict__ pinv64, int K, int M, int N,
-                                                  double beta, typename CT<Tout>::type* __restrict__ xb) {
+__global__ void __launch_bounds__(kRhsThreads) rhs_kernel(const SetupC<Tout>* __restrict__ lam,
+                                                          const SetupC<Tout>* __restrict__ yhat,
+                                                          const SetupC<Tout>* __restrict__ pinv64, int K, int M,
+                                                          int N, double beta, typename CT<Tout>::type* __restrict__ xb) {
   using C = typename CT<Tout>::type;
   using R = typename SetupReal<Tout>::type;
   using S = SetupC<Tout>;
+  static_assert(sizeof(S) == 16, "one asynchronous copy per entry");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const int H = N / 2 + 1, P = half_pitch(N);
-  const int bin = blockIdx.x * blockDim.x + threadIdx.x;
+  const int bin = blockIdx.x * kRhsThreads + threadIdx.x;
   if (bin >= N * H) return;
   const int k1 = bin / H, k2 = bin - k1 * H;
   const size_t off = (size_t)k1 * P + k2, mplane = (size_t)N * P;
+  // two chunk buffers of MMAX entries per thread, entry m of buffer s at buf[(s MMAX + m) kRhsThreads]
+  S* buf = reinterpret_cast<S*>(smem_raw) + threadIdx.x;
+  auto issue = [&](int s, const S* src, int n) {
+    for (int m = 0; m < n; ++m, src += mplane)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(buf + (s * MMAX + m) * kRhsThreads)),
+                   "l"(src)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto ready = [] { asm volatile("cp.async.wait_group 1;" ::: "memory"); };  // all but the newest chunk
   const R bd(beta);
   const S zero = mk<S>(0.0, 0.0);
   S b[MMAX], x[MMAX];
@@ -516,26 +535,39 @@ __global__ void __launch_bounds__(128) rhs_kernel(const SetupC<Tout>* __restrict
     b[m] = zero;
     x[m] = zero;
   }
+  issue(0, lam + off, M);
+  S yn = yhat[off];
   for (int k = 0; k < K; ++k) {
-    const S yk = yhat[(size_t)k * mplane + off];
+    const S yk = yn;
+    if (k + 1 < K) {
+      yn = yhat[(size_t)(k + 1) * mplane + off];
+      issue((k + 1) & 1, lam + (size_t)(k + 1) * M * mplane + off, M);
+    } else {
+      issue(K & 1, pinv64 + off, M);
+    }
+    ready();
+    const S* l = buf + (k & 1) * MMAX * kRhsThreads;
 #pragma unroll
     for (int m = 0; m < MMAX; ++m)
-      if (m < M) cfmac(b[m], lam[(size_t)(k * M + m) * mplane + off], yk);
+      if (m < M) cfmac(b[m], l[m * kRhsThreads], yk);
   }
 #pragma unroll
   for (int m = 0; m < MMAX; ++m) {
     b[m].x = b[m].x * bd;
     b[m].y = b[m].y * bd;
   }
-  int pk = 0;
+  const S* prow = pinv64 + off;
 #pragma unroll
   for (int i = 0; i < MMAX; ++i) {
     if (i < M) {
+      prow += (size_t)(M - i) * mplane;
+      issue((K + i + 1) & 1, prow, M - i - 1);
+      ready();
+      const S* l = buf + ((K + i) & 1) * MMAX * kRhsThreads;
 #pragma unroll
       for (int j = i; j < MMAX; ++j) {
         if (j < M) {
-          const S pij = pinv64[(size_t)pk * mplane + off];
-          ++pk;
+          const S pij = l[(j - i) * kRhsThreads];
           cfma(x[i], pij, b[j]);
           if (j != i) cfmac(x[j], pij, b[i]);
         }
@@ -623,18 +655,28 @@ cudaError_t launch_factor_pinv(const SetupC<Tout>* lam, const double* gs, int us
   return cudaGetLastError();
 }
 
+template <typename Tout, int MMAX>
+cudaError_t launch_rhs_m(const SetupC<Tout>* lam, const SetupC<Tout>* yhat, const SetupC<Tout>* pinv64, int K, int M,
+                         int N, double beta, typename CT<Tout>::type* xb, cudaStream_t s) {
+  constexpr int sm = 2 * MMAX * kRhsThreads * 16;
+  auto k = rhs_kernel<Tout, MMAX>;
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); });
+  if (e != cudaSuccess) return e;
+  const int nb = N * (N / 2 + 1);
+  k<<<(nb + kRhsThreads - 1) / kRhsThreads, kRhsThreads, sm, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
+  return cudaGetLastError();
+}
+
 template <typename Tout>
 cudaError_t launch_rhs(const SetupC<Tout>* lam, const SetupC<Tout>* yhat, const SetupC<Tout>* pinv64, int K, int M,
                        int N, double beta, typename CT<Tout>::type* xb, cudaStream_t s) {
-  const int nb = N * (N / 2 + 1);
-  const dim3 grid((nb + 127) / 128), block(128);
-  if (M <= 4) rhs_kernel<Tout, 4><<<grid, block, 0, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
-  else if (M <= 8) rhs_kernel<Tout, 8><<<grid, block, 0, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
-  else if (M <= 10) rhs_kernel<Tout, 10><<<grid, block, 0, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
-  else if (M <= 12) rhs_kernel<Tout, 12><<<grid, block, 0, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
-  else if (M <= kMaxM) rhs_kernel<Tout, 16><<<grid, block, 0, s>>>(lam, yhat, pinv64, K, M, N, beta, xb);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (M <= 4) return launch_rhs_m<Tout, 4>(lam, yhat, pinv64, K, M, N, beta, xb, s);
+  if (M <= 8) return launch_rhs_m<Tout, 8>(lam, yhat, pinv64, K, M, N, beta, xb, s);
+  if (M <= 10) return launch_rhs_m<Tout, 10>(lam, yhat, pinv64, K, M, N, beta, xb, s);
+  if (M <= 12) return launch_rhs_m<Tout, 12>(lam, yhat, pinv64, K, M, N, beta, xb, s);
+  if (M <= kMaxM) return launch_rhs_m<Tout, 16>(lam, yhat, pinv64, K, M, N, beta, xb, s);
+  return cudaErrorInvalidValue;
 }
 
 template <typename T>

@@ -13,8 +13,10 @@
 // and rounded once, one per stage in the order the stage reads them
 // (tw_stage); a radix-8 butterfly loads
 // only w^j and w^4j and forms w^2j, w^3j, w^5j, w^6j, w^7j by at most two
-// complex products (a few ulp), since table loads stalled the stages.
+// complex products (a few ulp), except in complex128.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace cip {
@@ -126,6 +128,13 @@ template <int R, int SIGN, typename C> __device__ __forceinline__ void dft_r(C* 
   else dft8<SIGN>(a);
 }
 
+// Twiddles of a radix-8 butterfly: w^j and w^4j are loaded and the other five formed by products (the
+// stages wait for the load/store pipe); complex128, whose stages wait for the FP64 pipe (an SM issues
+// two FP64 multiply-adds a cycle), loads all seven: 256^2 x 5 complex128, 40 iterations, 6.00 -> 5.82 ms.
+// Double-float keeps the products although it would gain 10%: other factors would round the factor of
+// a TV plan differently, whose error near DC changes by tens of percent either way with its last bits.
+template <typename C> constexpr bool tw_products() { return std::is_same<C, double2>::value == false; }
+
 template <typename C, int LOGN, int NF, int E, int SIGN, int R, int LS>
 __device__ __forceinline__ void stockham_stage(C* buf, int f, int tt, const C* __restrict__ tw, const TeamSync& ts,
                                                bool active) {
@@ -141,7 +150,7 @@ __device__ __forceinline__ void stockham_stage(C* buf, int f, int tt, const C* _
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
-      if constexpr (R == 8) {
+      if constexpr (R == 8 && tw_products<C>()) {
         const C w1 = ldg_tw(&tw[tw_stage(R, LS) + j]), w4 = ldg_tw(&tw[tw_stage(R, LS) + 3 * LS + j]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
         C* ww = &w[b * (R - 1)];
@@ -235,7 +244,7 @@ __device__ __forceinline__ void fft_stage_io(int tt, const C* __restrict__ tw, I
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int j = (tt + TT * b) & (LS - 1);
-      if constexpr (R == 8) {
+      if constexpr (R == 8 && tw_products<C>()) {
         const C w1 = ldg_tw(&tw[tw_stage(R, LS) + j]), w4 = ldg_tw(&tw[tw_stage(R, LS) + 3 * LS + j]);
         const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
         C* ww = &w[b * (R - 1)];
@@ -332,7 +341,13 @@ __device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw
   for (int b0 = 0; b0 < NB0; ++b0) {
     const int j = tt + TT * b0;  // = t mod LS of the butterflies b0 + NB0 i
     C w[7];
-    {
+    if constexpr (!tw_products<C>()) {
+#pragma unroll
+      for (int r = 0; r < 7; ++r) {
+        w[r] = ldg_tw(&tw[tw_stage(8, LS) + r * LS + j]);
+        if (SIGN > 0) w[r].y = -w[r].y;
+      }
+    } else {
       const C w1 = ldg_tw(&tw[tw_stage(8, LS) + j]), w4 = ldg_tw(&tw[tw_stage(8, LS) + 3 * LS + j]);
       const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
       w[0] = w1; w[1] = w2; w[2] = w3; w[3] = w4; w[4] = cmul(w4, w1); w[5] = cmul(w4, w2); w[6] = cmul(w4, w3);

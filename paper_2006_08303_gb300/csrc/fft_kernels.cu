@@ -17,7 +17,7 @@ constexpr int kE = SETUP_FFT_E;  // FFT elements per thread in these kernels (8 
 template <typename Tc, typename Tin, int LOGN>
 __global__ void __launch_bounds__(kRowThreads) row_r2c_kernel(const Tin* __restrict__ in,
                                                                 typename CT<Tc>::type* __restrict__ out, int nrows,
-                                                                Tc scale, const typename CT<Tc>::type* tw) {
+                                                                const typename CT<Tc>::type* tw) {
   using C = typename CT<Tc>::type;
   constexpr int N = 1 << LOGN, H = N / 2 + 1, P = half_pitch(N), ZS = spad(N), TEAM = N / kE;
   constexpr int PAIRS = kRowThreads / TEAM;
@@ -28,9 +28,10 @@ __global__ void __launch_bounds__(kRowThreads) row_r2c_kernel(const Tin* __restr
   for (int idx = tid; idx < PAIRS * N; idx += kRowThreads) {
     const int p = idx / N, n = idx - p * N;
     const int ra = row0 + 2 * p, rb = ra + 1;
-    const Tc xa = ra < nrows ? (Tc)in[(size_t)ra * N + n] : Tc(0);
-    const Tc xb = rb < nrows ? (Tc)in[(size_t)rb * N + n] : Tc(0);
-    zb[p * ZS + spad(n)] = cpack<C>(xa * scale * Tc(0.5f), xb * scale * Tc(0.5f));
+    // the 1/2 of the pair extraction, exact on the input
+    const Tin xa = ra < nrows ? in[(size_t)ra * N + n] * Tin(0.5) : Tin(0);
+    const Tin xb = rb < nrows ? in[(size_t)rb * N + n] * Tin(0.5) : Tin(0);
+    zb[p * ZS + spad(n)] = cpack<C>((Tc)xa, (Tc)xb);
   }
   __syncthreads();
   const int team = tid / TEAM;
@@ -75,7 +76,7 @@ __global__ void col_c2c_kernel(typename CT<Tc>::type* data, const typename CT<Tc
 }
 
 template <typename Tc, typename Tin, int LOGN>
-cudaError_t rr2c(const Tin* in, typename CT<Tc>::type* out, int nrows, Tc scale, const typename CT<Tc>::type* tw,
+cudaError_t rr2c(const Tin* in, typename CT<Tc>::type* out, int nrows, const typename CT<Tc>::type* tw,
                  cudaStream_t s) {
   using C = typename CT<Tc>::type;
   constexpr int N = 1 << LOGN, PAIRS = kRowThreads / (N / kE);
@@ -83,7 +84,7 @@ cudaError_t rr2c(const Tin* in, typename CT<Tc>::type* out, int nrows, Tc scale,
   auto k = row_r2c_kernel<Tc, Tin, LOGN>;
   if (sm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   const int nblk = (nrows + 2 * PAIRS - 1) / (2 * PAIRS);
-  k<<<nblk, kRowThreads, sm, s>>>(in, out, nrows, scale, tw);
+  k<<<nblk, kRowThreads, sm, s>>>(in, out, nrows, tw);
   return cudaGetLastError();
 }
 
@@ -119,9 +120,9 @@ cudaError_t cc2c(typename CT<Tc>::type* data, int nmaps, int sign, const typenam
   }
 
 template <typename Tc, typename Tin>
-cudaError_t launch_row_r2c(const Tin* in, typename CT<Tc>::type* out, int N, int nrows, Tc scale,
+cudaError_t launch_row_r2c(const Tin* in, typename CT<Tc>::type* out, int N, int nrows,
                            const typename CT<Tc>::type* tw, cudaStream_t s) {
-  CIP_SWITCH_N(N, (rr2c<Tc, Tin, L>(in, out, nrows, scale, tw, s)))
+  CIP_SWITCH_N(N, (rr2c<Tc, Tin, L>(in, out, nrows, tw, s)))
 }
 
 template <typename Tc>
@@ -130,11 +131,11 @@ cudaError_t launch_col_c2c(typename CT<Tc>::type* data, int N, int nmaps, int si
   CIP_SWITCH_N(N, (cc2c<Tc, L>(data, nmaps, sign, tw, s)))
 }
 
-template cudaError_t launch_row_r2c<df64, float>(const float*, cdf*, int, int, df64, const cdf*, cudaStream_t);
-template cudaError_t launch_row_r2c<df64, double>(const double*, cdf*, int, int, df64, const cdf*, cudaStream_t);
-template cudaError_t launch_row_r2c<double, double>(const double*, double2*, int, int, double, const double2*,
+template cudaError_t launch_row_r2c<df64, float>(const float*, cdf*, int, int, const cdf*, cudaStream_t);
+template cudaError_t launch_row_r2c<df64, double>(const double*, cdf*, int, int, const cdf*, cudaStream_t);
+template cudaError_t launch_row_r2c<double, double>(const double*, double2*, int, int, const double2*,
                                                     cudaStream_t);
-template cudaError_t launch_row_r2c<float, float>(const float*, float2*, int, int, float, const float2*,
+template cudaError_t launch_row_r2c<float, float>(const float*, float2*, int, int, const float2*,
                                                   cudaStream_t);
 template cudaError_t launch_col_c2c<float>(float2*, int, int, int, const float2*, cudaStream_t);
 template cudaError_t launch_col_c2c<double>(double2*, int, int, int, const double2*, cudaStream_t);

@@ -202,7 +202,7 @@ cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colb
 // Setup / read-back FFTs (not fused).
 // rows: nrows real rows of length N -> half spectra with pitch P (unnormalised forward DFT)
 template <typename Tc, typename Tin>
-cudaError_t launch_row_r2c(const Tin* in, typename CT<Tc>::type* out, int N, int nrows, Tc scale,
+cudaError_t launch_row_r2c(const Tin* in, typename CT<Tc>::type* out, int N, int nrows,
                            const typename CT<Tc>::type* tw, cudaStream_t s);
 // in-place column DFT of nmaps [N][P] half-spectrum maps
 template <typename Tc>
