@@ -287,6 +287,8 @@ template <typename T> cip_status alloc_state(cip_plan* p) {
   }
   p->rowsA = prior_pass_kind(p) == PRIOR_L1 ? rowpass_rows(p->N) : passA_rows<T>(p->N, tile_kind(p->prior));
   p->blocksA = (p->N / p->rowsA) * smaps(p);
+  // the wavelet prior's shrinkage: a thread per pixel (all channels), at most 2048 blocks
+  if (p->prior == CIP_PRIOR_WDCT) p->blocksA = std::min(p->N * p->N / 256, 2048);
   CIP_CUDA(p, dmalloc(p, (void**)&p->partials, (size_t)p->blocksA * kNPart * sizeof(double)));
   return CIP_OK;
 }

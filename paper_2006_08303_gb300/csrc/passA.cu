@@ -607,8 +607,16 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
           }
           if constexpr (LOW) {
             if (a.lowbuf && tid < 12) {  // value tid of rows 2i, 2i + 1: the warps' sums in order
-              T s = T(0);
-              for (int wp = 0; wp < NT / 32; ++wp) s += lows[i & 1][wp][tid];
+              static_assert(NT % 128 == 0, "");
+              T s4[NT / 128];  // four warps' sums at a time, then theirs: shorter chain, smaller rounding error
+#pragma unroll
+              for (int w4 = 0; w4 < NT / 128; ++w4) {
+                const T(*l)[12] = &lows[i & 1][4 * w4];
+                s4[w4] = (l[0][tid] + l[1][tid]) + (l[2][tid] + l[3][tid]);
+              }
+              T s = s4[0];
+#pragma unroll
+              for (int w4 = 1; w4 < NT / 128; ++w4) s += s4[w4];
               const int r = tid / 6, comp = (tid / 3) & 1, e = tid % 3;
               T* dst = reinterpret_cast<T*>(a.lowbuf + ((size_t)(comp * kLowK + (e > 0)) * a.M + m) * CP + r0 + 2 * i + r);
               if (e == 0) {

@@ -156,31 +156,56 @@ bool symlet_lowpass(int p, double* h) {
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-// Forward level: a CTA makes the 16 x 16 tile (i0, j0) of each of the four subbands from the
-// 46 x 46 input tile starting at (2 i0, 2 j0) (periodic in n): a_i = sum_k h_k x[(2i + k) mod n]
-// along the rows into shared memory, then the same along the columns.  The three detail subbands
-// go to det (Mallat positions of the band, pitch N, plane N^2); the LL subband to ll.
-template <typename T>
+// The tiled level kernels: TS x TS tiles of the four subbands per CTA.  The taps are kernel parameters
+// (constant-bank operands of the multiply-adds); what else a thread issues is kept small by 16-byte
+// global and shared-memory accesses along the rows and by making several outputs from each loaded
+// window.  TS = 32 (a 78 x 78 input tile for 64 x 64 pixels) filters 1.2 rows per output row, TS = 16
+// 1.4; it is taken where it leaves at least two CTAs per SM (wave_tile).
+// At 512^2 x 10 (all kernels of the chain launched programmatically too) the wavelet prior pass went
+// from 119 to 77 us; at 1024^2 x 10 from 331 to 208 us.
+template <typename T> struct alignas(16) Vec16 { T v[16 / sizeof(T)]; };
+
+// Forward level: the TS x TS tiles (i0, j0) from the input tile starting at (2 i0, 2 j0) (periodic in
+// n): a_i = sum_k h_k x[(2i + k) mod n] along the rows into shared memory, then the same along the
+// columns.  The three detail subbands go to det (Mallat positions of the band, pitch N, plane N^2); the
+// LL subband to ll.
+template <typename T, int TS> struct FwdTile {
+  static constexpr int ROWS = 2 * TS + 14, VE = 16 / (int)sizeof(T), COLS = 2 * TS + 16, RP = 2 * TS + 2;
+  static constexpr size_t bytes = ((size_t)ROWS * COLS + (size_t)ROWS * RP) * sizeof(T);
+};
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) dwt2_fwd_kernel(const T* __restrict__ in, int in_pitch, size_t in_plane,
                                                        T* __restrict__ det, int N, T* __restrict__ ll, int ll_pitch,
-                                                       size_t ll_plane, int n, WaveFilt<T> f) {
-  __shared__ T S[46][47];
-  __shared__ T R[46][33];
-  const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16, ch = blockIdx.z;
+                                                       size_t ll_plane, int n, const WaveFilt<T> f) {
+  using F = FwdTile<T, TS>;
+  using V = Vec16<T>;
+  constexpr int ROWS = F::ROWS, COLS = F::COLS, VE = F::VE, RP = F::RP;
+  extern __shared__ __align__(16) unsigned char wsm[];
+  T* S = reinterpret_cast<T*>(wsm);  // [ROWS][COLS]: the input tile
+  T* R = S + ROWS * COLS;            // [ROWS][RP]: low outputs, high outputs of every row
+  const int i0 = blockIdx.y * TS, j0 = blockIdx.x * TS, ch = blockIdx.z;
   const int tid = threadIdx.x;
+  grid_dep_wait();
+  grid_dep_launch();
   const T* src = in + (size_t)ch * in_plane;
-  for (int idx = tid; idx < 46 * 46; idx += 256) {
-    const int r = idx / 46, c = idx - r * 46;
-    S[r][c] = src[(size_t)((2 * i0 + r) & (n - 1)) * in_pitch + ((2 * j0 + c) & (n - 1))];
+  // 16-byte pieces: 2 j0 and n are multiples of 32, so a piece never wraps inside
+  for (int idx = tid; idx < ROWS * (COLS / VE); idx += 256) {
+    const int r = idx / (COLS / VE), c = (idx - r * (COLS / VE)) * VE;
+    *reinterpret_cast<V*>(&S[r * COLS + c]) =
+        *reinterpret_cast<const V*>(&src[(size_t)((2 * i0 + r) & (n - 1)) * in_pitch + ((2 * j0 + c) & (n - 1))]);
   }
   __syncthreads();
-  // rows: a thread makes the low and high outputs 2q and 2q + 1 of row r, which read the 18
-  // inputs 4q .. 4q + 17 (four outputs per 18 shared-memory loads instead of one per 16)
-  for (int it = tid; it < 46 * 8; it += 256) {
-    const int r = it >> 3, q = it & 7;
-    T x[18];
+  // rows: the low and high outputs 2q, 2q + 1 of row r, from the 18 inputs 4q .. 4q + 17
+  for (int it = tid; it < ROWS * (TS / 2); it += 256) {
+    const int r = it / (TS / 2), q = it - r * (TS / 2);
+    constexpr int NV = (18 + VE - 1) / VE;
+    T x[NV * VE];
 #pragma unroll
-    for (int m = 0; m < 18; ++m) x[m] = S[r][4 * q + m];
+    for (int i = 0; i < NV; ++i) {
+      const V v = *reinterpret_cast<const V*>(&S[r * COLS + 4 * q + i * VE]);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) x[i * VE + e] = v.v[e];
+    }
     T l0 = T(0), h0 = T(0), l1 = T(0), h1 = T(0);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -189,66 +214,81 @@ __global__ void __launch_bounds__(256) dwt2_fwd_kernel(const T* __restrict__ in,
       l1 = fma(f.h[k], x[k + 2], l1);
       h1 = fma(f.g[k], x[k + 2], h1);
     }
-    R[r][2 * q] = l0;
-    R[r][2 * q + 1] = l1;
-    R[r][16 + 2 * q] = h0;
-    R[r][16 + 2 * q + 1] = h1;
+    T* d = &R[r * RP + 2 * q];
+    d[0] = l0;
+    d[1] = l1;
+    d[TS] = h0;
+    d[TS + 1] = h1;
   }
   __syncthreads();
-  // columns: the same on the output rows 2q, 2q + 1 of column o (one item per thread)
+  // columns: the same on the output rows 4q .. 4q + 3 of column o, from 22 rows
   const int half = n / 2;
-  {
-    const int q = tid >> 5, o = tid & 31;
-    T x[18];
+  for (int it = tid; it < (TS / 4) * 2 * TS; it += 256) {
+    const int q = it / (2 * TS), o = it - q * 2 * TS;
+    T x[22];
 #pragma unroll
-    for (int m = 0; m < 18; ++m) x[m] = R[4 * q + m][o];
-    T v[4] = {T(0), T(0), T(0), T(0)};  // low 2q, low 2q + 1, high 2q, high 2q + 1
+    for (int m = 0; m < 22; ++m) x[m] = R[(8 * q + m) * RP + o];
+    T lo[4] = {T(0), T(0), T(0), T(0)}, hi[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      v[0] = fma(f.h[k], x[k], v[0]);
-      v[1] = fma(f.h[k], x[k + 2], v[1]);
-      v[2] = fma(f.g[k], x[k], v[2]);
-      v[3] = fma(f.g[k], x[k + 2], v[3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        lo[e] = fma(f.h[k], x[k + 2 * e], lo[e]);
+        hi[e] = fma(f.g[k], x[k + 2 * e], hi[e]);
+      }
     }
-    const int cb = o >> 4, col = j0 + (o & 15);
+    const int cb = o / TS, col = j0 + (o & (TS - 1)), row = i0 + 4 * q;
+    T* d = det + (size_t)ch * N * N + cb * half + col;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int rb = e >> 1, row = i0 + 2 * q + (e & 1);
-      if (rb == 0 && cb == 0) ll[(size_t)ch * ll_plane + (size_t)row * ll_pitch + col] = v[e];
-      else det[(size_t)ch * N * N + (size_t)(rb * half + row) * N + cb * half + col] = v[e];
+      if (cb == 0) ll[(size_t)ch * ll_plane + (size_t)(row + e) * ll_pitch + col] = lo[e];
+      else d[(size_t)(row + e) * N] = lo[e];
+      d[(size_t)(half + row + e) * N] = hi[e];
     }
   }
 }
 
-// Inverse level (the transpose): a CTA makes the 32 x 32 output tile (y0, x0) of the n x n band
-// from the 23 x 23 coefficient tiles of the four subbands starting at (y0/2 - 7, x0/2 - 7)
-// (periodic in n/2): x_j = sum over k = j mod 2 of h_k a_i + g_k d_i, i = (j - k)/2, first along
-// the columns, then along the rows.  LL comes from ll, the details from det (Mallat positions).
-template <typename T>
+// Inverse level (the transpose): the 2 TS x 2 TS output tile (y0, x0) of the n x n band from the
+// coefficient tiles of the four subbands starting at (y0/2 - 7, x0/2 - 8) (periodic in n/2): x_j = sum
+// over k = j mod 2 of h_k a_i + g_k d_i, i = (j - k)/2, first along the columns, then along the rows.
+// LL comes from ll, the details from det (Mallat positions).
+template <typename T, int TS> struct InvTile {
+  static constexpr int CR = TS + 7, CC = TS + 8, VE = 16 / (int)sizeof(T), VP = TS + 8 + (sizeof(T) == 4 ? 2 : 0);
+  static constexpr size_t bytes = ((size_t)4 * CR * CC + (size_t)2 * 2 * TS * VP) * sizeof(T);
+};
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* __restrict__ ll, int ll_pitch, size_t ll_plane,
                                                        const T* __restrict__ det, int N, T* __restrict__ out,
-                                                       int out_pitch, size_t out_plane, int n, WaveFilt<T> f) {
-  __shared__ T C[4][23][24];  // subband rb * 2 + cb
-  __shared__ T V[2][32][24];  // after the column inverse: [cb][output row][coefficient column]
-  const int y0 = blockIdx.y * 32, x0 = blockIdx.x * 32, ch = blockIdx.z;
+                                                       int out_pitch, size_t out_plane, int n, const WaveFilt<T> f) {
+  using F = InvTile<T, TS>;
+  using V16 = Vec16<T>;
+  constexpr int CR = F::CR, CC = F::CC, VE = F::VE, VP = F::VP, ON = 2 * TS;
+  extern __shared__ __align__(16) unsigned char wsm[];
+  T* C = reinterpret_cast<T*>(wsm);  // [4][CR][CC]: subband rb * 2 + cb
+  T* W = C + 4 * CR * CC;            // [2][ON][VP]: after the column inverse, [cb][output row][coefficient column]
+  const int y0 = blockIdx.y * ON, x0 = blockIdx.x * ON, ch = blockIdx.z;
   const int tid = threadIdx.x, half = n / 2;
-  for (int idx = tid; idx < 4 * 23 * 23; idx += 256) {
-    const int sb = idx / 529, rem = idx - sb * 529, a = rem / 23, b = rem - a * 23;
-    const int ri = (y0 / 2 - 7 + a + half) & (half - 1), ci = (x0 / 2 - 7 + b + half) & (half - 1);
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int idx = tid; idx < 4 * CR * (CC / VE); idx += 256) {
+    const int sb = idx / (CR * (CC / VE)), rem = idx - sb * (CR * (CC / VE)), a = rem / (CC / VE),
+              c = (rem - a * (CC / VE)) * VE;
+    const int ri = (y0 / 2 - 7 + a + half) & (half - 1), ci = (x0 / 2 - 8 + c + half) & (half - 1);
     const int rb = sb >> 1, cb = sb & 1;
-    C[sb][a][b] = sb == 0 ? ll[(size_t)ch * ll_plane + (size_t)ri * ll_pitch + ci]
-                          : det[(size_t)ch * N * N + (size_t)(rb * half + ri) * N + cb * half + ci];
+    const T* p = sb == 0 ? &ll[(size_t)ch * ll_plane + (size_t)ri * ll_pitch + ci]
+                         : &det[(size_t)ch * N * N + (size_t)(rb * half + ri) * N + cb * half + ci];
+    *reinterpret_cast<V16*>(&C[(sb * CR + a) * CC + c]) = *reinterpret_cast<const V16*>(p);
   }
   __syncthreads();
-  // columns: a thread makes the outputs jj = 4p .. 4p + 3 of coefficient column b, which read the
-  // coefficient rows a = 2p .. 2p + 8 of both subbands (four outputs per 18 loads instead of 16 each)
-  for (int it = tid; it < 2 * 8 * 23; it += 256) {
-    const int cb = it / (8 * 23), rem = it - cb * 8 * 23, p = rem / 23, b = rem - p * 23;
+  // columns: outputs jj = 4p .. 4p + 3 of coefficient column b, from the coefficient rows
+  // 2p .. 2p + 8 of both subbands
+  for (int it = tid; it < 2 * (ON / 4) * CC; it += 256) {
+    const int cb = it / ((ON / 4) * CC), rem = it - cb * (ON / 4) * CC, p = rem / CC, b = rem - p * CC;
     T cl[9], chh[9];
 #pragma unroll
     for (int m = 0; m < 9; ++m) {
-      cl[m] = C[cb][2 * p + m][b];
-      chh[m] = C[2 + cb][2 * p + m][b];
+      cl[m] = C[(cb * CR + 2 * p + m) * CC + b];
+      chh[m] = C[((2 + cb) * CR + 2 * p + m) * CC + b];
     }
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
@@ -261,21 +301,26 @@ __global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* __restrict__ ll,
           acc = fma(f.h[k], cl[m], acc);
           acc = fma(f.g[k], chh[m], acc);
         }
-        V[cb][4 * p + 2 * d + e][b] = acc;
+        W[(cb * ON + 4 * p + 2 * d + e) * VP + b] = acc;
       }
     }
   }
   __syncthreads();
-  // rows: the same along the row, outputs xx = 4p .. 4p + 3 of output row jj (one item per thread)
-  {
-    const int jj = tid >> 3, p = tid & 7;
-    T v0[9], v1[9];
+  // rows: outputs xx = 4p .. 4p + 3 of output row jj, from the coefficient columns 2p + 1 .. 2p + 9
+  struct alignas(2 * sizeof(T)) Two { T a, b; };
+  for (int it = tid; it < ON * (ON / 4); it += 256) {
+    const int jj = it / (ON / 4), p = it - jj * (ON / 4);
+    T v0[10], v1[10];
 #pragma unroll
-    for (int m = 0; m < 9; ++m) {
-      v0[m] = V[0][jj][2 * p + m];
-      v1[m] = V[1][jj][2 * p + m];
+    for (int m = 0; m < 10; m += 2) {
+      const Two a = *reinterpret_cast<const Two*>(&W[jj * VP + 2 * p + m]);
+      const Two c = *reinterpret_cast<const Two*>(&W[(ON + jj) * VP + 2 * p + m]);
+      v0[m] = a.a;
+      v0[m + 1] = a.b;
+      v1[m] = c.a;
+      v1[m + 1] = c.b;
     }
-    T* o = out + (size_t)ch * out_plane + (size_t)(y0 + jj) * out_pitch + x0 + 4 * p;
+    alignas(16) T o[4];
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
 #pragma unroll
@@ -283,13 +328,16 @@ __global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* __restrict__ ll,
         T acc = T(0);
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-          const int k = e + 2 * t, m = d + 7 - t;
+          const int k = e + 2 * t, m = d + 7 - t + 1;
           acc = fma(f.h[k], v0[m], acc);
           acc = fma(f.g[k], v1[m], acc);
         }
         o[2 * d + e] = acc;
       }
     }
+    T* dst = out + (size_t)ch * out_plane + (size_t)(y0 + jj) * out_pitch + x0 + 4 * p;
+#pragma unroll
+    for (int e = 0; e < 4; e += VE) *reinterpret_cast<V16*>(dst + e) = *reinterpret_cast<const V16*>(&o[e]);
   }
 }
 
@@ -305,6 +353,8 @@ __global__ void __launch_bounds__(512) dwt2_fwd_fused_kernel(const T* __restrict
   T* X = reinterpret_cast<T*>(wsm);  // [n0][n0 + 1]: the band of the current level
   T* R = X + (size_t)n0 * pp;          // [n0][n0 + 1]: after the row filters
   const int ch = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+  grid_dep_wait();
+  grid_dep_launch();
   const T* src = in + (size_t)ch * in_plane;
   T* dst = A + (size_t)ch * N * N;
   for (int idx = tid; idx < n0 * n0; idx += nth) {
@@ -376,6 +426,8 @@ __global__ void __launch_bounds__(512) dwt2_inv_fused_kernel(const T* __restrict
   T* C = reinterpret_cast<T*>(wsm);  // [4][q0][q0 + 1]: subband rb * 2 + cb of the current level
   T* V = C + (size_t)4 * q0 * qp;      // [2][n0][q0 + 1]: after the column inverse
   const int ch = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+  grid_dep_wait();
+  grid_dep_launch();
   const T* a = A + (size_t)ch * N * N;
   for (int idx = tid; idx < 16 * 16; idx += nth) C[(idx >> 4) * qp + (idx & 15)] = a[(size_t)(idx >> 4) * N + (idx & 15)];
   for (int n = 32; n <= n0; n <<= 1) {
@@ -452,6 +504,8 @@ __global__ void __launch_bounds__(256) wdct_shrink_kernel(T* __restrict__ coef, 
                                                           T* __restrict__ tprev, const T* __restrict__ t_imp,
                                                           double* __restrict__ partials, int N, T tau, int flags) {
   __shared__ double red[8][kNPart];
+  grid_dep_wait();
+  grid_dep_launch();
   const T* cv = cmat.c;  // kernel parameter: constant-bank operands, the same for every thread
   const bool import_mode = (flags & PA_IMPORT) != 0;
   const bool resid = (flags & PA_RESID) != 0;
@@ -523,22 +577,48 @@ __global__ void __launch_bounds__(256) wdct_shrink_kernel(T* __restrict__ coef, 
 
 }  // namespace
 
+namespace {
+// 32-wide subband tiles where they still give every SM two CTAs
+int wave_tile(int n, int M) { return n >= 64 && (n / 64) * (n / 64) * M >= 2 * 152 ? 32 : 16; }
+
+template <typename T, int TS>
+cudaError_t fwd_level(const T* in, int in_pitch, size_t in_plane, T* det, int N, T* ll, int ll_pitch, size_t ll_plane,
+                      int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+  auto k = dwt2_fwd_kernel<T, TS>;
+  constexpr size_t sm = FwdTile<T, TS>::bytes;
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3(n / 2 / TS, n / 2 / TS, M), dim3(256), sm, s, 0, in, in_pitch, in_plane, det, N, ll, ll_pitch,
+                    ll_plane, n, f);
+}
+template <typename T, int TS>
+cudaError_t inv_level(const T* ll, int ll_pitch, size_t ll_plane, const T* det, int N, T* out, int out_pitch,
+                      size_t out_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+  auto k = dwt2_inv_kernel<T, TS>;
+  constexpr size_t sm = InvTile<T, TS>::bytes;
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3(n / 2 / TS, n / 2 / TS, M), dim3(256), sm, s, 0, ll, ll_pitch, ll_plane, det, N, out,
+                    out_pitch, out_plane, n, f);
+}
+}  // namespace
+
 template <typename T>
 cudaError_t launch_dwt2_fwd(const T* in, int in_pitch, size_t in_plane, T* det, int N, T* ll, int ll_pitch,
                             size_t ll_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
   if (n < 32 || n > N || (n & (n - 1))) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)(n / 32), (unsigned)(n / 32), (unsigned)M);
-  dwt2_fwd_kernel<T><<<grid, 256, 0, s>>>(in, in_pitch, in_plane, det, N, ll, ll_pitch, ll_plane, n, f);
-  return cudaGetLastError();
+  return wave_tile(n, M) == 32 ? fwd_level<T, 32>(in, in_pitch, in_plane, det, N, ll, ll_pitch, ll_plane, n, M, f, s)
+                               : fwd_level<T, 16>(in, in_pitch, in_plane, det, N, ll, ll_pitch, ll_plane, n, M, f, s);
 }
 
 template <typename T>
 cudaError_t launch_dwt2_inv(const T* ll, int ll_pitch, size_t ll_plane, const T* det, int N, T* out, int out_pitch,
                             size_t out_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
   if (n < 32 || n > N || (n & (n - 1))) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)(n / 32), (unsigned)(n / 32), (unsigned)M);
-  dwt2_inv_kernel<T><<<grid, 256, 0, s>>>(ll, ll_pitch, ll_plane, det, N, out, out_pitch, out_plane, n, f);
-  return cudaGetLastError();
+  return wave_tile(n, M) == 32 ? inv_level<T, 32>(ll, ll_pitch, ll_plane, det, N, out, out_pitch, out_plane, n, M, f, s)
+                               : inv_level<T, 16>(ll, ll_pitch, ll_plane, det, N, out, out_pitch, out_plane, n, M, f, s);
 }
 
 template <typename T> int wave_fuse_band(int N) { return N < wave_fuse_n<T>() ? N : wave_fuse_n<T>(); }
@@ -554,8 +634,7 @@ cudaError_t launch_dwt2_fwd_fused(const T* in, int in_pitch, size_t in_plane, T*
                                 (int)(2 * (size_t)wave_fuse_n<T>() * (wave_fuse_n<T>() + 1) * sizeof(T)));
   });
   if (e != cudaSuccess) return e;
-  dwt2_fwd_fused_kernel<T><<<M, 512, sm, s>>>(in, in_pitch, in_plane, A, N, n0, f);
-  return cudaGetLastError();
+  return launch_pdl(dwt2_fwd_fused_kernel<T>, dim3(M), dim3(512), sm, s, 0, in, in_pitch, in_plane, A, N, n0, f);
 }
 
 template <typename T>
@@ -570,8 +649,7 @@ cudaError_t launch_dwt2_inv_fused(const T* A, int N, T* out, int out_pitch, size
                                 (int)(8 * (size_t)q * (q + 1) * sizeof(T)));
   });
   if (e != cudaSuccess) return e;
-  dwt2_inv_fused_kernel<T><<<M, 512, sm, s>>>(A, N, out, out_pitch, out_plane, n0, f);
-  return cudaGetLastError();
+  return launch_pdl(dwt2_inv_fused_kernel<T>, dim3(M), dim3(512), sm, s, 0, A, N, out, out_pitch, out_plane, n0, f);
 }
 
 template <typename T>
@@ -581,14 +659,13 @@ cudaError_t launch_wdct_shrink(T* coef, const ChanDCT<T>& cmat, const T* u_in, T
   switch (M) {
 #define WS_CASE(m)                                                                                              \
   case m:                                                                                                      \
-    wdct_shrink_kernel<T, m><<<blocks, 256, 0, s>>>(coef, cmat, u_in, u_out, tprev, t_imp, partials, N, tau, flags); \
-    break;
+    return launch_pdl(wdct_shrink_kernel<T, m>, dim3(blocks), dim3(256), 0, s, 0, coef, cmat, u_in, u_out, tprev,  \
+                      t_imp, partials, N, tau, flags);
     WS_CASE(1) WS_CASE(2) WS_CASE(3) WS_CASE(4) WS_CASE(5) WS_CASE(6) WS_CASE(7) WS_CASE(8)
     WS_CASE(9) WS_CASE(10) WS_CASE(11) WS_CASE(12) WS_CASE(13) WS_CASE(14) WS_CASE(15) WS_CASE(16)
 #undef WS_CASE
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template cudaError_t launch_dwt2_fwd<float>(const float*, int, size_t, float*, int, float*, int, size_t, int, int,
