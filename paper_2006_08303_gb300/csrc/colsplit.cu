@@ -12,13 +12,18 @@ namespace cip {
 namespace {
 
 // X = xb + Pinv Q at every bin, in place on colbuf; thread = (k2, k1), k1 fastest.
-// 128-thread CTAs at <= ~72 registers (complex64) keep every bin of a
-// 512 x 512 x 10 problem resident in one wave; before waiting for the forward
-// column DFTs, each CTA prefetches its slab of the factor and the data term
-// (independent of them) into L2.
-constexpr int kSolveThreads = 128;
+// A bin's factor is read once, row by row of the packed triangle; each thread copies the rows ahead
+// asynchronously into its own shared-memory slots (no barrier), kRowBufs rows deep, so the loads in
+// flight are not bounded by its registers.  The first rows and the data term are requested before the
+// grid dependency, since they do not depend on the forward column DFTs.  Plain loads (72
+// registers of them in flight at most) ran at 2.5 TB/s; split column pass before and now: 1024^2 x 10
+// 127.8 -> 106.8 us, 1024^2 x 16 384 -> 206, 512^2 x 10 43.9 -> 30.3, 256^2 x 5 13.1 -> 11.2 us.
+constexpr int kSolveThreads = 128, kRowBufs = 3;
 template <typename T, int MMAX> constexpr int solve_minblocks() {
-  return sizeof(T) == 4 ? (MMAX <= 12 ? 7 : 5) : 3;
+  return sizeof(T) == 4 ? (MMAX <= 12 ? 7 : 4) : 3;
+}
+template <typename T, int MMAX> constexpr size_t solve_smem() {
+  return (size_t)kRowBufs * MMAX * kSolveThreads * 2 * sizeof(T);
 }
 
 template <typename T, int MMAX>
@@ -30,24 +35,35 @@ __global__ void __launch_bounds__(kSolveThreads, solve_minblocks<T, MMAX>())
   using C = typename CT<T>::type;
   const int k1 = blockIdx.x * kSolveThreads + threadIdx.x;
   const int k2 = blockIdx.y;
-  {
-    // the CTA's bins [k1lo, k1lo + 128) are whole 32-bin blocks: one contiguous run of the
-    // blocked factor and one of the data term
-    const int npk = M * (M + 1) / 2;
-    const int k1lo = blockIdx.x * kSolveThreads;
-    const int cnt = min(kSolveThreads, N - k1lo);
-    if (threadIdx.x == 0) prefetch_l2(pinv + binp(k2, 0, k1lo, npk, N), (size_t)cnt * npk * sizeof(C));
-    if (threadIdx.x == 1) prefetch_l2(xb + binp(k2, 0, k1lo, M, N), (size_t)cnt * M * sizeof(C));
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw) + threadIdx.x;  // entry j of row buffer s at buf[(s MMAX + j) kSolveThreads]
+  const int npk = M * (M + 1) / 2;
+  const bool on = k1 < N;
+  const C* prow = pinv + binp(k2, 0, on ? k1 : 0, npk, N);  // plane stride kBinBlock
+  auto issue = [&](int i) {
+    if (on) {
+      for (int j = 0; j < M - i; ++j, prow += kBinBlock) {
+        const unsigned dst = smem_addr(buf + ((i % kRowBufs) * MMAX + j) * kSolveThreads);
+        if constexpr (sizeof(C) == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(prow) : "memory");
+        else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(prow) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  C r[MMAX], x[MMAX];
+#pragma unroll
+  for (int i = 0; i < kRowBufs - 1; ++i) issue(i);
+  if (on) {
+    const C* xcol = xb + binp(k2, 0, k1, M, N);  // plane stride kBinBlock
+#pragma unroll
+    for (int i = 0; i < MMAX; ++i)
+      if (i < M) x[i] = xcol[(size_t)i * kBinBlock];
   }
   grid_dep_wait();  // the forward column DFTs are complete from here on
   grid_dep_launch();
-  if (k1 >= N) return;
-  const int npk = M * (M + 1) / 2;
+  if (!on) return;
   const int CP = col_pitch(N);
   C* col = colbuf + (size_t)k2 * M * CP + k1;
-  const C* xcol = xb + binp(k2, 0, k1, M, N);      // plane stride kBinBlock
-  const C* pcol = pinv + binp(k2, 0, k1, npk, N);  // plane stride kBinBlock
-  C r[MMAX], x[MMAX];
   // columns k2 < kLowK of a TV plan with the low-column correction: Q from the column DFTs of the
   // components of t - u, the differences applied as spectral products
   const bool low = lowcol && k2 < kLowK;
@@ -68,22 +84,22 @@ __global__ void __launch_bounds__(kSolveThreads, solve_minblocks<T, MMAX>())
       } else {
         r[i] = col[(size_t)i * CP];
       }
-      x[i] = xcol[(size_t)i * kBinBlock];
       if (plain) {  // plain FP32 method: X = Pinv (b + Q)
         r[i] = cadd(r[i], x[i]);
         x[i] = mk<C>(0.0, 0.0);
       }
     }
   }
-  int pk = 0;
 #pragma unroll
   for (int i = 0; i < MMAX; ++i) {
     if (i < M) {
+      issue(i + kRowBufs - 1);  // (past the last row: an empty group)
+      asm volatile("cp.async.wait_group %0;" ::"n"(kRowBufs - 1) : "memory");
+      const C* p = buf + (i % kRowBufs) * MMAX * kSolveThreads;
 #pragma unroll
       for (int j = i; j < MMAX; ++j) {
         if (j < M) {
-          const C pij = pcol[(size_t)pk * kBinBlock];
-          ++pk;
+          const C pij = p[(j - i) * kSolveThreads];
           cfma(x[i], pij, r[j]);
           if (j != i) cfmac(x[j], pij, r[i]);
         }
@@ -95,13 +111,29 @@ __global__ void __launch_bounds__(kSolveThreads, solve_minblocks<T, MMAX>())
     if (i < M) col[(size_t)i * CP] = x[i];
 }
 
+template <typename T, int MMAX>
+cudaError_t solve_launch(typename CT<T>::type* colbuf, const typename CT<T>::type* pinv, const typename CT<T>::type* xb,
+                         int N, int M, int plain, const typename CT<T>::type* lowcol, const typename CT<T>::type* tw,
+                         T rho, cudaStream_t s) {
+  auto k = solve_split_kernel<T, MMAX>;
+  constexpr size_t sm = solve_smem<T, MMAX>();
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] {
+    cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (r != cudaSuccess) return r;
+    return cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3((N + kSolveThreads - 1) / kSolveThreads, N / 2 + 1), dim3(kSolveThreads), sm, s, 0, colbuf,
+                    pinv, xb, N, M, plain, lowcol, tw, rho);
+}
+
 template <typename T>
 cudaError_t solve_m(typename CT<T>::type* colbuf, const typename CT<T>::type* pinv, const typename CT<T>::type* xb,
                     int N, int M, int plain, const typename CT<T>::type* lowcol, const typename CT<T>::type* tw,
                     T rho, cudaStream_t s) {
-  const dim3 grid((N + kSolveThreads - 1) / kSolveThreads, N / 2 + 1), block(kSolveThreads);
 #define CIP_SOLVE(MM) \
-  return launch_pdl(solve_split_kernel<T, MM>, grid, block, 0, s, 0, colbuf, pinv, xb, N, M, plain, lowcol, tw, rho)
+  return solve_launch<T, MM>(colbuf, pinv, xb, N, M, plain, lowcol, tw, rho, s)
   if (M <= 4) CIP_SOLVE(4);
   if (M <= 8) CIP_SOLVE(8);
   if (M <= 10) CIP_SOLVE(10);
