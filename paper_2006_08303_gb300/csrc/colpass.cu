@@ -121,7 +121,7 @@ cudaError_t launch_cols(const typename CT<T>::type* src, typename CT<T>::type* d
                         int ncols, cudaStream_t s, const typename CT<T>::type* src2, typename CT<T>::type* dst2,
                         int ncols2) {
   using C = typename CT<T>::type;
-  constexpr int N = 1 << LOGN, TT = cp_team<T>(N), TEAMS = kColThreads / TT;
+  constexpr int N = 1 << LOGN, TT = N / cp_elems<T>(N), TEAMS = kColThreads / TT;
   const size_t sm = (size_t)TEAMS * spad(N) * sizeof(C);
   auto k = colfft_cols_kernel<T, LOGN, SIGN>;
   static PerDeviceOnce once;

@@ -200,6 +200,73 @@ __device__ __forceinline__ void stockham_stage(C* buf, int f, int tt, const C* _
   ts.sync();
 }
 
+// The last radix-8 stage and the radix-2/4 stage after it in one: for N = 8 LS R2 (R2 = 2 or 4) the
+// radix-R2 butterfly at j takes output j mod 8 LS of the R2 radix-8 butterflies whose indexes agree
+// mod LS, so a thread that holds those R2 butterflies (E = 8 R2 LS / TT elements, TT <= LS) needs no
+// exchange between the two stages.  The arithmetic is that of the two stages one after the other.
+// The outputs of thread tt are the E positions n = tt mod TT.
+template <typename C, int LOGN, int E> constexpr bool fft_merges() {
+  constexpr int REM = LOGN % 3, LS = 1 << (3 * (LOGN / 3 - 1)), TT = (1 << LOGN) / E;
+  return REM != 0 && LS > 1 && TT <= LS && E >= 8 * (REM == 1 ? 2 : 4);
+}
+// DIRECT: twiddles as fft_stage_io takes them for more than two butterflies per thread, all from the table.
+template <typename C, int LOGN, int E, int SIGN, bool DIRECT = false, class In, class Mid, class Out>
+__device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw, In&& in, Mid&& mid, Out&& out) {
+  constexpr int N = 1 << LOGN, TT = N / E, LS = 1 << (3 * (LOGN / 3 - 1)), R2 = LOGN % 3 == 1 ? 2 : 4;
+  constexpr int B = E / 8, NB0 = LS / TT, LS2 = 8 * LS;
+  static_assert(fft_merges<C, LOGN, E>() && B == NB0 * R2, "");
+  C a[E];
+#pragma unroll
+  for (int b = 0; b < B; ++b)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[b * 8 + r] = in(tt + TT * b, r * (N / 8));
+  mid();
+#pragma unroll
+  for (int b0 = 0; b0 < NB0; ++b0) {
+    const int j = tt + TT * b0;  // = t mod LS of the butterflies b0 + NB0 i
+    C w[7];
+    if constexpr (DIRECT || !tw_products<C>()) {
+#pragma unroll
+      for (int r = 0; r < 7; ++r) {
+        w[r] = ldg_tw(&tw[tw_stage(8, LS) + r * LS + j]);
+        if (SIGN > 0) w[r].y = -w[r].y;
+      }
+    } else {
+      const C w1 = ldg_tw(&tw[tw_stage(8, LS) + j]), w4 = ldg_tw(&tw[tw_stage(8, LS) + 3 * LS + j]);
+      const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
+      w[0] = w1; w[1] = w2; w[2] = w3; w[3] = w4; w[4] = cmul(w4, w1); w[5] = cmul(w4, w2); w[6] = cmul(w4, w3);
+      if (SIGN > 0) {
+#pragma unroll
+        for (int r = 0; r < 7; ++r) w[r].y = -w[r].y;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R2; ++i) {
+      C* v = &a[(b0 + NB0 * i) * 8];
+#pragma unroll
+      for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[r - 1]);
+      dft_r<8, SIGN>(v);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int j2 = j + LS * r;
+      C v[R2];
+#pragma unroll
+      for (int i = 0; i < R2; ++i) {
+        v[i] = a[(b0 + NB0 * i) * 8 + r];
+        if (i > 0) {
+          C wr = ldg_tw(&tw[tw_stage(R2, LS2) + (i - 1) * LS2 + j2]);
+          if (SIGN > 0) wr.y = -wr.y;
+          v[i] = cmul(v[i], wr);
+        }
+      }
+      dft_r<R2, SIGN>(v);
+#pragma unroll
+      for (int i = 0; i < R2; ++i) out(j2, LS2 * i, v[i]);
+    }
+  }
+}
+
 // NF interleaved length-2^LOGN FFTs executed by the team's NTH = N*NF/E threads;
 // `tid` is the thread's index inside the team.
 // With a CTA-wide TeamSync, threads outside every team call this with
@@ -211,11 +278,25 @@ __device__ __forceinline__ void fft_team(C* buf, int tid, const C* __restrict__ 
   constexpr int REM = LOGN % 3;
   const int f = tid % NF;
   const int tt = tid / NF;
+  constexpr bool MERGE = NF == 1 && fft_merges<C, LOGN, E>();  // the last two stages without an exchange between
   if constexpr (S8 >= 1) stockham_stage<C, LOGN, NF, E, SIGN, 8, 1>(buf, f, tt, tw, ts, active);
-  if constexpr (S8 >= 2) stockham_stage<C, LOGN, NF, E, SIGN, 8, 8>(buf, f, tt, tw, ts, active);
-  if constexpr (S8 >= 3) stockham_stage<C, LOGN, NF, E, SIGN, 8, 64>(buf, f, tt, tw, ts, active);
-  if constexpr (REM == 1) stockham_stage<C, LOGN, NF, E, SIGN, 2, (1 << (3 * S8))>(buf, f, tt, tw, ts, active);
-  if constexpr (REM == 2) stockham_stage<C, LOGN, NF, E, SIGN, 4, (1 << (3 * S8))>(buf, f, tt, tw, ts, active);
+  if constexpr (S8 >= 2 && !(MERGE && S8 == 2)) stockham_stage<C, LOGN, NF, E, SIGN, 8, 8>(buf, f, tt, tw, ts, active);
+  if constexpr (S8 >= 3 && !MERGE) stockham_stage<C, LOGN, NF, E, SIGN, 8, 64>(buf, f, tt, tw, ts, active);
+  if constexpr (MERGE) {
+    static_assert(E / 8 <= 2, "twiddles as stockham_stage");
+    auto bar = [&]() { ts.sync(); };
+    if (active) {
+      fft_last_merged<C, LOGN, E, SIGN>(
+          tt, tw, [&](int i0, int off) { return buf[spad(i0) + off + (off >> 4)]; }, bar,
+          [&](int i0, int off, C v) { buf[spad(i0) + off + (off >> 4)] = v; });
+    } else {
+      ts.sync();
+    }
+    ts.sync();
+  } else {
+    if constexpr (REM == 1) stockham_stage<C, LOGN, NF, E, SIGN, 2, (1 << (3 * S8))>(buf, f, tt, tw, ts, active);
+    if constexpr (REM == 2) stockham_stage<C, LOGN, NF, E, SIGN, 4, (1 << (3 * S8))>(buf, f, tt, tw, ts, active);
+  }
 }
 
 // ---- stages with separate input and output accessors ------------------------
@@ -287,7 +368,8 @@ __device__ __forceinline__ void fft_stage_io(int tt, const C* __restrict__ tw, I
 // complete before any write; when outL writes to `buf`, the last stage's
 // writes follow a barrier after its reads.  outL_alias says whether outL
 // writes memory that the last stage reads (then a barrier separates them).
-template <typename C, int LOGN, int E, int SIGN, bool OUTL_ALIAS, class In0, class OutL, class Sync>
+template <typename C, int LOGN, int E, int SIGN, bool OUTL_ALIAS, bool DIRECT = (E / 8 > 2), class In0, class OutL,
+          class Sync>
 __device__ __forceinline__ void fft_team_io(C* buf, int tt, const C* __restrict__ tw, const Sync& sync, In0&& in0,
                                             OutL&& outL) {
   constexpr int S8 = LOGN / 3;
@@ -301,85 +383,27 @@ __device__ __forceinline__ void fft_team_io(C* buf, int tt, const C* __restrict_
   // stage 0 (LS = 1, radix 8): in0 -> padded
   fft_stage_io<C, LOGN, E, SIGN, 8, 1>(tt, tw, in0, bar, pout);
   sync();
+  // with more than two butterflies per thread the last two stages merge (see fft_last_merged)
+  constexpr bool MERGE = E / 8 > 2 && fft_merges<C, LOGN, E>();
   // middle radix-8 stages
-  if constexpr (NST >= 3) {
+  if constexpr (NST >= (MERGE ? 4 : 3)) {
     fft_stage_io<C, LOGN, E, SIGN, 8, 8>(tt, tw, pin, bar, pout);
     sync();
   }
-  if constexpr (NST >= 4) {
+  if constexpr (NST >= 4 && !MERGE) {
     fft_stage_io<C, LOGN, E, SIGN, 8, 64>(tt, tw, pin, bar, pout);
     sync();
+  }
+  if constexpr (MERGE) {
+    if constexpr (OUTL_ALIAS) fft_last_merged<C, LOGN, E, SIGN, DIRECT>(tt, tw, pin, bar, outL);
+    else fft_last_merged<C, LOGN, E, SIGN, DIRECT>(tt, tw, pin, none, outL);
   }
   // last stage: radix 8 at LS = 8^(S8-1) when REM == 0, else radix 2/4 at LS = 8^S8
   constexpr int RL = REM == 0 ? 8 : (REM == 1 ? 2 : 4);
   constexpr int LSL = REM == 0 ? (1 << (3 * (S8 - 1))) : (1 << (3 * S8));
-  if constexpr (OUTL_ALIAS) fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, bar, outL);
-  else fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, none, outL);
-}
-
-// The last radix-8 stage and the radix-2/4 stage after it in one: for N = 8 LS R2 (R2 = 2 or 4) the
-// radix-R2 butterfly at j takes output j mod 8 LS of the R2 radix-8 butterflies whose indexes agree
-// mod LS, so a thread that holds those R2 butterflies (E = 8 R2 LS / TT elements, TT <= LS) needs no
-// exchange between the two stages.  The arithmetic is that of the two stages one after the other.
-// The outputs of thread tt are the E positions n = tt mod TT.
-template <typename C, int LOGN, int E> constexpr bool fft_merges() {
-  constexpr int REM = LOGN % 3, LS = 1 << (3 * (LOGN / 3 - 1)), TT = (1 << LOGN) / E;
-  return REM != 0 && LS > 1 && TT <= LS && E >= 8 * (REM == 1 ? 2 : 4);
-}
-template <typename C, int LOGN, int E, int SIGN, class In, class Mid, class Out>
-__device__ __forceinline__ void fft_last_merged(int tt, const C* __restrict__ tw, In&& in, Mid&& mid, Out&& out) {
-  constexpr int N = 1 << LOGN, TT = N / E, LS = 1 << (3 * (LOGN / 3 - 1)), R2 = LOGN % 3 == 1 ? 2 : 4;
-  constexpr int B = E / 8, NB0 = LS / TT, LS2 = 8 * LS;
-  static_assert(fft_merges<C, LOGN, E>() && B == NB0 * R2, "");
-  C a[E];
-#pragma unroll
-  for (int b = 0; b < B; ++b)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) a[b * 8 + r] = in(tt + TT * b, r * (N / 8));
-  mid();
-#pragma unroll
-  for (int b0 = 0; b0 < NB0; ++b0) {
-    const int j = tt + TT * b0;  // = t mod LS of the butterflies b0 + NB0 i
-    C w[7];
-    if constexpr (!tw_products<C>()) {
-#pragma unroll
-      for (int r = 0; r < 7; ++r) {
-        w[r] = ldg_tw(&tw[tw_stage(8, LS) + r * LS + j]);
-        if (SIGN > 0) w[r].y = -w[r].y;
-      }
-    } else {
-      const C w1 = ldg_tw(&tw[tw_stage(8, LS) + j]), w4 = ldg_tw(&tw[tw_stage(8, LS) + 3 * LS + j]);
-      const C w2 = cmul(w1, w1), w3 = cmul(w1, w2);
-      w[0] = w1; w[1] = w2; w[2] = w3; w[3] = w4; w[4] = cmul(w4, w1); w[5] = cmul(w4, w2); w[6] = cmul(w4, w3);
-      if (SIGN > 0) {
-#pragma unroll
-        for (int r = 0; r < 7; ++r) w[r].y = -w[r].y;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < R2; ++i) {
-      C* v = &a[(b0 + NB0 * i) * 8];
-#pragma unroll
-      for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[r - 1]);
-      dft_r<8, SIGN>(v);
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int j2 = j + LS * r;
-      C v[R2];
-#pragma unroll
-      for (int i = 0; i < R2; ++i) {
-        v[i] = a[(b0 + NB0 * i) * 8 + r];
-        if (i > 0) {
-          C wr = ldg_tw(&tw[tw_stage(R2, LS2) + (i - 1) * LS2 + j2]);
-          if (SIGN > 0) wr.y = -wr.y;
-          v[i] = cmul(v[i], wr);
-        }
-      }
-      dft_r<R2, SIGN>(v);
-#pragma unroll
-      for (int i = 0; i < R2; ++i) out(j2, LS2 * i, v[i]);
-    }
+  if constexpr (!MERGE) {
+    if constexpr (OUTL_ALIAS) fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, bar, outL);
+    else fft_stage_io<C, LOGN, E, SIGN, RL, LSL>(tt, tw, pin, none, outL);
   }
 }
 
