@@ -23,6 +23,7 @@ UNITS = [
     ("passA.cu", [], "passA.o"),
     ("rowpass.cu", [], "rowpass.o"),
     ("colpass.cu", [], "colpass.o"),
+    ("coldirect.cu", [], "coldirect.o"),
     ("fft_kernels.cu", [], "fft_kernels.o"),
     ("factor.cu", [], "factor.o"),
     ("noalloc.cu", [], "noalloc.o"),

@@ -59,7 +59,7 @@ struct cip_plan {
   int cur = 0;  // index of the u buffer holding the current u
   size_t esz = 4;
   int rowsA = 8, cc = 1, blocksA = 0, blocksB = 0;
-  int colmode = 1;  // column pass: 1 fused kernel, 2 split (FFT / solve / FFT)
+  int colmode = 1;  // column pass: 1 fused kernel, 2 split (FFT / solve / FFT), 3 fused without the ring
   int avar = 0;     // prior-pass kernel variant (1: the other FFT width, 2: 32; complex64, N = 256 .. 1024)
   int test_fault = 0;  // test-only fault switch (cip_set_test_fault)
   // TV at N >= kLowFixMinN: low-column correction of the x-update (launch_passB_split)
@@ -732,6 +732,12 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
     p->launches += n;
   } else {
     (void)cc;
+    if constexpr (sizeof(T) == 4) {
+      if (mode == 3) {
+        CIP_LAUNCH(p, launch_coldirect(b, smaps(p), s));
+        return CIP_OK;
+      }
+    }
     CIP_LAUNCH(p, launch_colpass_fused<T>(b, smaps(p), p->conv + 1, s));
   }
   return CIP_OK;
@@ -786,14 +792,18 @@ int forced_avar(const cip_plan* p) {
   return p->opt.prior_fft == prior_fft_default(p) ? 0 : 1;
 }
 
+// the fused form without the ring is a choice of the autotuner only
+bool direct_ok(const cip_plan* p) { return p->dtype == CIP_F32 && !is_cd(p) && coldirect_fits(p->N, p->M); }
+
 template <typename T> void set_colmode(cip_plan* p, int mode, int cc) {
+  if (mode == 3 && !direct_ok(p)) mode = 1;  // (a decision read from a file)
   p->colmode = mode;
   if (mode == 1) p->cc = cc;
-  p->blocksB = mode == 1 ? p->N / 2 + 1 : p->M * (p->N / 2 + 1);
+  p->blocksB = mode != 2 ? p->N / 2 + 1 : p->M * (p->N / 2 + 1);
 }
 
 // Autotuner: times whole iterations (column pass, then prior pass, launched back to back as in
-// cip_iterate) for every column-pass form (fused kernel; split FFT / solve / FFT) and both
+// cip_iterate) for every column-pass form (fused kernel, with and without the ring; split FFT / solve / FFT) and both
 // prior-pass FFT widths where a variant exists, on this plan's buffers, and keeps the fastest,
 // cached per (N, M, dtype, prior, forced width) for the process: plans with one width (wavelet
 // prior, complex128, N < 256, N = 2048) and plans with a forced one time their candidates once as
@@ -830,7 +840,10 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
       cands.push_back({p->colmode, p->cc, av});
       continue;
     }
-    if (colpass_fused_fits<T>(p->N, p->M)) cands.push_back({1, 1, av});
+    if (colpass_fused_fits<T>(p->N, p->M)) {
+      cands.push_back({1, 1, av});
+      if (direct_ok(p)) cands.push_back({3, 1, av});
+    }
     cands.push_back({2, 0, av});
   }
   cudaEvent_t e0, e1;
@@ -1077,9 +1090,10 @@ template <typename T> cip_status iterate_impl(cip_plan* p, int max_iter, double 
 }
 
 // One iteration (column pass, prior pass) enqueued with no host synchronisation and no timing
-// events, so that it can be recorded into a CUDA graph.
+// events, so that it can be recorded into a CUDA graph.  Its kernels share the device with other plans'
+// (batch, server): the fused column pass runs in its ring form (coldirect.cu says why; the bits are the same).
 template <typename T> cip_status enqueue_iteration(cip_plan* p, cudaStream_t s, int flags) {
-  cip_status cst = column_pass<T>(p, s, p->colmode, p->cc);
+  cip_status cst = column_pass<T>(p, s, p->colmode == 3 ? 1 : p->colmode, p->cc);
   if (cst != CIP_OK) return cst;
   if (p->dl_sigma > 0) {
     cst = dict_step<T>(p, s);
@@ -1759,7 +1773,7 @@ cip_status cip_get_prior_fft(cip_plan* p, int* elems) {
 cip_status cip_get_config(cip_plan* p, int* rows, int* cc, int* blocksA, int* blocksB, int* column_pass) {
   if (!p) return CIP_ERR_INVALID_ARG;
   if (rows) *rows = p->rowsA;
-  if (column_pass) *column_pass = p->colmode;
+  if (column_pass) *column_pass = p->colmode == 2 ? 2 : 1;
   if (cc) *cc = p->cc;
   if (blocksA) *blocksA = p->blocksA;
   if (blocksB) *blocksB = p->blocksB;

@@ -181,6 +181,9 @@ template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int
 template <typename T> bool colpass_fused_fits(int N, int M);
 template <typename T> size_t colpass_fused_smem(int N, int M);
 template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, int S, int* err, cudaStream_t s);
+// The same for few channels without the ring (csrc/coldirect.cu): faster alone on the device.
+bool coldirect_fits(int N, int M);
+cudaError_t launch_coldirect(const PassBArgs<float>& b, int S, cudaStream_t s);
 // column DFTs of every (k2, map) column of the column layout, src -> dst (may alias);
 // sign < 0 forward, > 0 inverse (unnormalised)
 template <typename T>
