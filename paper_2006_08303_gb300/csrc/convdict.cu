@@ -14,6 +14,8 @@
 // maps (the l1 prior pass over L*M maps) are the analysis path's kernels.
 #include <algorithm>
 
+#include <type_traits>
+
 #include "fft.cuh"
 #include "kernels.h"
 
@@ -278,69 +280,90 @@ __device__ __forceinline__ C tw_at(const C* __restrict__ tw, int j, int N) {
   return t;
 }
 
-// Warp reduce-scatter by recursive halving over PM entries per lane (PM a power of two <= 32): at
-// xor distance O a lane keeps one half of its LIVE entries (the upper half when bit O of the lane
-// is set) and adds its partner's copy of that half.  Afterwards v[0] of lane i holds the warp's sum
-// of entry i >> log2(32 / PM), after PM - 1 + log2(32 / PM) exchanges (5 PM for separate sums).
-template <int LIVE, int O, int PM, typename C>
-__device__ __forceinline__ void reduce_scatter(C (&v)[PM], int lane) {
-  if constexpr (LIVE > 1) {
-    const bool up = (lane & O) != 0;
-#pragma unroll
-    for (int i = 0; i < LIVE / 2; ++i) {
-      const C lo = v[i], hi = v[i + LIVE / 2];
-      C keep = up ? hi : lo;
-      const C send = up ? lo : hi;
-      keep.x += __shfl_xor_sync(0xffffffffu, send.x, O);
-      keep.y += __shfl_xor_sync(0xffffffffu, send.y, O);
-      v[i] = keep;
-    }
-    reduce_scatter<LIVE / 2, O / 2>(v, lane);
-  } else if constexpr (O >= 1) {
-    v[0].x += __shfl_xor_sync(0xffffffffu, v[0].x, O);
-    v[0].y += __shfl_xor_sync(0xffffffffu, v[0].y, O);
-    reduce_scatter<1, O / 2>(v, lane);
-  }
-}
-
-constexpr int ilog2c(int v) { return v <= 1 ? 0 : 1 + ilog2c(v / 2); }
-
-// block sum of one double per thread (blockDim a multiple of 32, <= 1024; red holds a value per
-// warp); every thread gets it
-__device__ __forceinline__ double block_sum256(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();  // red may still be read from a previous call
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  return t;
-}
-
 // Per frequency, one thread (k1 = block offset + thread, k2 = blockIdx.y, so that the warps read
 // the column layout contiguously): the filter normal equation summed over the M channels,
 // (sigma I + W W^H) d = b with W = [conj(zhat_{l,s})] (L x M) and b = W xhat + sigma F(g - e), by
 // the Woodbury identity d = (b - W alpha) / sigma, (sigma I_M + W^H W) alpha = W^H b.  The L
 // filters are streamed twice: once to accumulate W^H W and W^H b, once to form d; the M x M system
 // is solved by Cholesky in registers.  Then w = d + e-hat is stored and its partial inverse DFT
-// along k1 at the P support rows is summed over the CTA's bins (reduce-scatter across each warp);
-// the last CTA of a column to finish adds the column's CTA sums in a fixed order, so the result
+// along k1 at the P support rows is summed over the CTA's bins: a small matrix product of the tile of
+// w with the bins' exponentials, both in shared memory (62 shuffles per bin and filter as a
+// reduce-scatter across each warp took more issue slots than the rest of the step); the last CTA of a column to finish adds the column's CTA sums in a fixed order, so the result
 // does not depend on the order in which CTAs run.
+// Two groups of kDLBlock threads share a bin: bound by the latency of the loads, one thread per bin left
+// an SM seven warps to hide it behind.  They divide the entries of W^H b and W^H W (each sum still runs
+// over all filters in order, so its rounding does not depend on the split); group 0 collects them in
+// shared memory and solves the M x M system (both solving it cost 7% at M = 8, L = 9); then they divide
+// the filters of the second pass.  Dividing
+// the filters of the first pass as well was 4 us faster at 256^2 x 5, L = 32, but rounds differently, and
+// the cancellation in b - W alpha turns that into 5e-5 of x at M = 8; four groups leave the 516 CTAs of
+// N = 256 in two waves (146 us an iteration against 134).  dl_solve + dl_filter + dl_spec before and now,
+// 256^2 x 5, L = 32, 11 x 11: 42 + 16 + 31 -> 36 + 14 + 18 us; an iteration 163 -> 136 us.
+constexpr int kDLGroups = 2, kDLThreads = kDLGroups * kDLBlock;
+// resident CTAs the registers are held to: four keep the 516 CTAs of N = 256 in one wave
+template <typename T> constexpr int dl_blocks(int M, int PM) { return sizeof(T) == 4 ? (M <= 5 && PM <= 16 ? 4 : 2) : 1; }
+// filters whose operands a thread loads together (the registers of complex128 hold one)
+template <typename T> constexpr int dl_unroll() { return sizeof(T) == 4 ? 4 : 1; }
+// entries of the triangle of W^H W that group 0 takes beside b (M products) and W^H b (M products)
+constexpr int dl_first(int M) { return M * (M + 1) / 2 > 2 * M ? (M * (M + 1) / 2 - 2 * M) / 2 : 0; }
+// elements of the region that holds the entries of group 1 and then the tile of w
+template <int M> constexpr int dl_part() {
+  constexpr int e = (M * (M + 1) / 2 - dl_first(M)) * kDLBlock, t = 32 * (kDLBlock + 1);
+  return e > t ? e : t;
+}
+// acc[j] = sum over 32 bins k of w[j WS + k] E[k ES]: pairs at distance 16 first, then 8, 4, 2, 1 (the
+// order of a butterfly over a warp's lanes), the partial sums of the open levels held in registers
+template <int ES, int WS, int NL, typename C>
+__device__ __forceinline__ void dl_tree(const C* __restrict__ E, const C* __restrict__ w, C (&acc)[NL]) {
+  C h4[NL], h2[NL], h1[NL];
+#pragma unroll 1
+  for (int t = 0; t < 8; ++t) {
+    const int b = ((t & 1) << 2) | (t & 2) | (t >> 2);
+    const C* e = E + b * ES;
+    const C e0 = e[0], e1 = e[16 * ES], e2 = e[8 * ES], e3 = e[24 * ES];
+#pragma unroll
+    for (int j = 0; j < NL; ++j) {
+      const C* v = w + j * WS + b;
+      acc[j] = cadd(cadd(cmul(v[0], e0), cmul(v[16], e1)), cadd(cmul(v[8], e2), cmul(v[24], e3)));
+    }
+    auto level = [&](C (&h)[NL], bool open) {
+#pragma unroll
+      for (int j = 0; j < NL; ++j) {
+        if (open) h[j] = acc[j];
+        else acc[j] = cadd(h[j], acc[j]);
+      }
+    };
+    level(h4, (t & 1) == 0);
+    if (t & 1) level(h2, (t & 2) == 0);
+    if ((t & 3) == 3) level(h1, (t & 4) == 0);
+  }
+}
 template <typename T, int M, int PM>
-__global__ void __launch_bounds__(kDLBlock) dl_solve_kernel(const DLArgs<T> a) {
+__global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kernel(const DLArgs<T> a) {
   using C = typename CT<T>::type;
-  static_assert(kDLBlock == 64, "two warps per CTA");
+  static_assert(kDLBlock == 64 && kDLGroups == 2, "two groups of two warps");
   const int N = a.N, L = a.L, P = a.P;
   const int CP = col_pitch(N), H = N / 2 + 1;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int grp = threadIdx.x / kDLBlock, bt = threadIdx.x - grp * kDLBlock;
+  const int tid = threadIdx.x;
   const int kb = blockIdx.x, nkb = gridDim.x;
-  const int k1 = kb * kDLBlock + tid, k2 = blockIdx.y;
+  const int k1 = kb * kDLBlock + bt, k2 = blockIdx.y;
   const T n2 = (T)N * (T)N;
   const T sigma = a.sigma;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  C* E = reinterpret_cast<C*>(dsm);                // [kDLBlock][PM]: exp(+2 pi i k1 (a - P/2) / N)
+  C* part = E + kDLBlock * PM;                     // [entries of group 1][kDLBlock] of W^H W, then
+  C* wt = part;                                    // [32][kDLBlock + 1]: w of this CTA's bins
+  C* als = part + dl_part<M>();                    // [M][kDLBlock]: alpha
   const C* zb = a.zcol + (size_t)k2 * M * L * CP + k1;  // z_{l,s} at zb[(s L + l) CP]
   const C* th = a.spec + (size_t)k2 * 2 * L * CP + k1;  // theta_l at th[l CP], F(g - e)_l at th[(L + l) CP]
   C x[M], c[M], G[M][M];
+  for (int i = tid; i < kDLBlock * PM; i += kDLThreads) {
+    const int ai = i % PM;
+    E[i] = ai < P ? tw_at<+1>(a.tw, (kb * kDLBlock + i / PM) * (ai - P / 2), N) : mk<C>(0.0, 0.0);
+  }
+  grid_dep_wait();
+  grid_dep_launch();
 #pragma unroll
   for (int s = 0; s < M; ++s) {
     const C v = a.xcol[((size_t)k2 * M + s) * CP + k1];
@@ -349,121 +372,167 @@ __global__ void __launch_bounds__(kDLBlock) dl_solve_kernel(const DLArgs<T> a) {
 #pragma unroll
     for (int t = 0; t < M; ++t) G[s][t] = mk<C>(0.0, 0.0);
   }
-  // b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s
-  auto load_b = [&](int l, C (&z)[M]) {
-    const C ge = __ldg(th + (size_t)(L + l) * CP);
-    C b = mk<C>(sigma * ge.x, sigma * ge.y);
+  // group 0: b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s, W^H b and the first E0 entries of the
+  // triangle of W^H W; group 1: the others.  Each sum runs over all filters in order.
+  constexpr int E0 = dl_first(M);
+  auto each = [&](auto f) {  // f(entry, s, t) over the triangle
+#pragma unroll
+    for (int s = 0; s < M; ++s)
+#pragma unroll
+      for (int t = 0; t <= s; ++t) f(s * (s + 1) / 2 + t, s, t);
+  };
+  auto load_z = [&](int l, C (&z)[M]) {
 #pragma unroll
     for (int s = 0; s < M; ++s) {
-      const C v = __ldg(zb + ((size_t)s * L + l) * CP);
+      const C v = zb[((size_t)s * L + l) * CP];
       z[s] = mk<C>(v.x * n2, v.y * n2);
-      cfmac(b, z[s], x[s]);
     }
-    return b;
   };
+  if (grp == 0) {
 #pragma unroll 4
-  for (int l = 0; l < L; ++l) {
-    C z[M];
-    const C b = load_b(l, z);
+    for (int l = 0; l < L; ++l) {
+      const C ge = th[(size_t)(L + l) * CP];
+      C z[M], b = mk<C>(sigma * ge.x, sigma * ge.y);
+      load_z(l, z);
 #pragma unroll
-    for (int s = 0; s < M; ++s) {
-      cfma(c[s], z[s], b);  // W^H b
+      for (int s = 0; s < M; ++s) cfmac(b, z[s], x[s]);
 #pragma unroll
-      for (int t = 0; t <= s; ++t) cfmac(G[s][t], z[t], z[s]);  // z_s conj(z_t)
+      for (int s = 0; s < M; ++s) cfma(c[s], z[s], b);
+      each([&](int e, int s, int t) {
+        if (e < E0) cfmac(G[s][t], z[t], z[s]);  // z_s conj(z_t)
+      });
+    }
+  } else {
+#pragma unroll 4
+    for (int l = 0; l < L; ++l) {
+      C z[M];
+      load_z(l, z);
+      each([&](int e, int s, int t) {
+        if (e >= E0) cfmac(G[s][t], z[t], z[s]);
+      });
     }
   }
-  // Cholesky of sigma I + G = R R^H (lower, in place), then R w = c and R^H alpha = w
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    T d = sigma + G[j][j].x;
-#pragma unroll
-    for (int k = 0; k < j; ++k) d -= G[j][k].x * G[j][k].x + G[j][k].y * G[j][k].y;
-    const T r = sqrt(d > T(0) ? d : T(0)), inv = r > T(0) ? T(1) / r : T(0);
-    G[j][j] = mk<C>(r, 0.0);
-#pragma unroll
-    for (int i = j + 1; i < M; ++i) {
-      C acc = G[i][j];
-#pragma unroll
-      for (int k = 0; k < j; ++k) {  // acc -= G_ik conj(G_jk)
-        const C u = G[i][k], v = G[j][k];
-        acc.x -= u.x * v.x + u.y * v.y;
-        acc.y -= u.y * v.x - u.x * v.y;
-      }
-      G[i][j] = mk<C>(acc.x * inv, acc.y * inv);
-    }
-  }
-  C w[M], al[M];
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    C acc = c[i];
-#pragma unroll
-    for (int k = 0; k < i; ++k) {
-      acc.x -= G[i][k].x * w[k].x - G[i][k].y * w[k].y;
-      acc.y -= G[i][k].x * w[k].y + G[i][k].y * w[k].x;
-    }
-    const T inv = T(1) / G[i][i].x;
-    w[i] = mk<C>(acc.x * inv, acc.y * inv);
-  }
-#pragma unroll
-  for (int i = M - 1; i >= 0; --i) {
-    C acc = w[i];
-#pragma unroll
-    for (int k = i + 1; k < M; ++k) {  // acc -= conj(G_ki) alpha_k
-      acc.x -= G[k][i].x * al[k].x + G[k][i].y * al[k].y;
-      acc.y -= G[k][i].x * al[k].y - G[k][i].y * al[k].x;
-    }
-    const T inv = T(1) / G[i][i].x;
-    al[i] = mk<C>(acc.x * inv, acc.y * inv);
-  }
-  // exp(+2 pi i k1 (a - P/2) / N) for the support rows a < P (zero beyond P)
-  const int cen = P / 2;
-  C wa[PM];
-#pragma unroll
-  for (int i = 0; i < PM; ++i) wa[i] = i < P ? tw_at<+1>(a.tw, k1 * (i - cen), N) : mk<C>(0.0, 0.0);
-  __shared__ C red[2][32][PM];  // [warp][l][a]
-  constexpr int SH = ilog2c(32 / PM);
-  const T isg = T(1) / sigma;
-  C* wb = a.wcol + (size_t)k2 * L * CP + k1;
-  // the operands of filter l + 1 are loaded while filter l is processed (one thread per bin leaves
-  // few warps per SM, so the loads in flight per thread set the bandwidth)
-  C zn[M], gen, tn;
-  auto load_l = [&](int l) {
-#pragma unroll
-    for (int s = 0; s < M; ++s) zn[s] = __ldg(zb + ((size_t)s * L + l) * CP);
-    gen = __ldg(th + (size_t)(L + l) * CP);
-    tn = __ldg(th + (size_t)l * CP);
-  };
-  load_l(0);
-#pragma unroll 1
-  for (int l = 0; l < L; ++l) {
-    C z[M];
-#pragma unroll
-    for (int s = 0; s < M; ++s) z[s] = mk<C>(zn[s].x * n2, zn[s].y * n2);
-    const C ge = gen, t = tn;
-    if (l + 1 < L) load_l(l + 1);
-    // b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s, then d -= conj(z_s) alpha_s
-    C d = mk<C>(sigma * ge.x, sigma * ge.y);
-#pragma unroll
-    for (int s = 0; s < M; ++s) {
-      cfmac(d, z[s], x[s]);
-      d.x -= z[s].x * al[s].x + z[s].y * al[s].y;
-      d.y -= z[s].x * al[s].y - z[s].y * al[s].x;
-    }
-    // w = d-hat + e-hat, e-hat = theta - F(g - e)
-    const C wl = mk<C>(fma(d.x, isg, t.x - ge.x), fma(d.y, isg, t.y - ge.y));
-    wb[(size_t)l * CP] = wl;
-    C v[PM];
-#pragma unroll
-    for (int i = 0; i < PM; ++i) v[i] = cmul(wl, wa[i]);
-    reduce_scatter<PM, 16>(v, lane);
-    if ((lane & ((1 << SH) - 1)) == 0) red[warp][l][lane >> SH] = v[0];
+  if (grp) {
+    each([&](int e, int s, int t) {
+      if (e >= E0) part[(e - E0) * kDLBlock + bt] = G[s][t];
+    });
   }
   __syncthreads();
-  C* yp = a.ypart + ((size_t)k2 * nkb + kb) * L * P;
-  for (int i = tid; i < L * P; i += kDLBlock) {
-    const int l = i / P, ai = i - l * P;
-    const C s0 = red[0][l][ai], s1 = red[1][l][ai];
-    yp[i] = mk<C>(s0.x + s1.x, s0.y + s1.y);
+  C al[M];
+  if (grp == 0) {
+    each([&](int e, int s, int t) {
+      if (e >= E0) G[s][t] = part[(e - E0) * kDLBlock + bt];
+    });
+    // Cholesky of sigma I + G = R R^H (lower, in place), then R w = c and R^H alpha = w
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      T d = sigma + G[j][j].x;
+#pragma unroll
+      for (int k = 0; k < j; ++k) d -= G[j][k].x * G[j][k].x + G[j][k].y * G[j][k].y;
+      const T r = sqrt(d > T(0) ? d : T(0)), inv = r > T(0) ? T(1) / r : T(0);
+      G[j][j] = mk<C>(r, 0.0);
+#pragma unroll
+      for (int i = j + 1; i < M; ++i) {
+        C acc = G[i][j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) {  // acc -= G_ik conj(G_jk)
+          const C u = G[i][k], v = G[j][k];
+          acc.x -= u.x * v.x + u.y * v.y;
+          acc.y -= u.y * v.x - u.x * v.y;
+        }
+        G[i][j] = mk<C>(acc.x * inv, acc.y * inv);
+      }
+    }
+    C w[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      C acc = c[i];
+#pragma unroll
+      for (int k = 0; k < i; ++k) {
+        acc.x -= G[i][k].x * w[k].x - G[i][k].y * w[k].y;
+        acc.y -= G[i][k].x * w[k].y + G[i][k].y * w[k].x;
+      }
+      const T inv = T(1) / G[i][i].x;
+      w[i] = mk<C>(acc.x * inv, acc.y * inv);
+    }
+#pragma unroll
+    for (int i = M - 1; i >= 0; --i) {
+      C acc = w[i];
+#pragma unroll
+      for (int k = i + 1; k < M; ++k) {  // acc -= conj(G_ki) alpha_k
+        acc.x -= G[k][i].x * al[k].x + G[k][i].y * al[k].y;
+        acc.y -= G[k][i].x * al[k].y - G[k][i].y * al[k].x;
+      }
+      const T inv = T(1) / G[i][i].x;
+      al[i] = mk<C>(acc.x * inv, acc.y * inv);
+    }
+#pragma unroll
+    for (int s = 0; s < M; ++s) als[s * kDLBlock + bt] = al[s];
+  }
+  __syncthreads();  // part is free from here on (als is not part of it)
+#pragma unroll
+  for (int s = 0; s < M; ++s) al[s] = als[s * kDLBlock + bt];
+  const T isg = T(1) / sigma;
+  C* wb = a.wcol + (size_t)k2 * L * CP + k1;
+  // the operands of U filters are loaded together
+  constexpr int U = dl_unroll<T>();
+#pragma unroll 1
+  for (int lb = grp; lb < L; lb += U * kDLGroups) {
+    C z[U][M], ge[U], t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int l = lb + u * kDLGroups;
+      if (l < L) {
+#pragma unroll
+        for (int s = 0; s < M; ++s) z[u][s] = zb[((size_t)s * L + l) * CP];
+        ge[u] = th[(size_t)(L + l) * CP];
+        t[u] = th[(size_t)l * CP];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int l = lb + u * kDLGroups;
+      if (l >= L) break;
+      // b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s, then d -= conj(z_s) alpha_s
+      C d = mk<C>(sigma * ge[u].x, sigma * ge[u].y);
+#pragma unroll
+      for (int s = 0; s < M; ++s) {
+        const C zs = mk<C>(z[u][s].x * n2, z[u][s].y * n2);
+        cfmac(d, zs, x[s]);
+        d.x -= zs.x * al[s].x + zs.y * al[s].y;
+        d.y -= zs.x * al[s].y - zs.y * al[s].x;
+      }
+      // w = d-hat + e-hat, e-hat = theta - F(g - e)
+      const C wl = mk<C>(fma(d.x, isg, t[u].x - ge[u].x), fma(d.y, isg, t[u].y - ge[u].y));
+      wb[(size_t)l * CP] = wl;
+      wt[l * (kDLBlock + 1) + bt] = wl;
+    }
+  }
+  __syncthreads();
+  // the support rows of the CTA's bins: thread = row a, filters l0, l0 + LSTEP, ...
+  {
+    constexpr int LSTEP = kDLThreads / PM;
+    const int ai = tid % PM;
+    C* yp = a.ypart + ((size_t)k2 * nkb + kb) * L * P;
+    auto rows = [&](auto nl) {
+      constexpr int NL = decltype(nl)::value;
+#pragma unroll 1
+      for (int l0 = tid / PM; l0 < L; l0 += NL * LSTEP) {
+        const C* wr = wt + l0 * (kDLBlock + 1);
+        C acc[2][NL];
+        dl_tree<PM, LSTEP * (kDLBlock + 1)>(E + ai, wr, acc[0]);
+        dl_tree<PM, LSTEP * (kDLBlock + 1)>(E + 32 * PM + ai, wr + 32, acc[1]);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+          const int l = l0 + j * LSTEP;
+          if (l < L && ai < P) yp[l * P + ai] = cadd(acc[0][j], acc[1][j]);
+        }
+      }
+    };
+    // as many at a time as few filters have (of the fixed four, L = 9 would compute 23 in vain)
+    if (L <= LSTEP) rows(std::integral_constant<int, 1>());
+    else if (L <= 2 * LSTEP) rows(std::integral_constant<int, 2>());
+    else rows(std::integral_constant<int, 4>());
   }
   __shared__ int last;
   __threadfence();  // this CTA's sums are visible device-wide before it is counted
@@ -473,7 +542,7 @@ __global__ void __launch_bounds__(kDLBlock) dl_solve_kernel(const DLArgs<T> a) {
   if (last) {
     __threadfence();
     const C* y0 = a.ypart + (size_t)k2 * nkb * L * P;
-    for (int i = tid; i < L * P; i += kDLBlock) {
+    for (int i = tid; i < L * P; i += kDLThreads) {
       C acc = mk<C>(0.0, 0.0);
       for (int b = 0; b < nkb; ++b) {
         const C v = __ldcg(y0 + (size_t)b * L * P + i);
@@ -512,27 +581,30 @@ __global__ void __launch_bounds__(kFiltThreads) dl_filter_kernel(const DLArgs<T>
   C* ws = ys + (size_t)P * chunk;       // [P][chunk]: exp(-2 pi i k2 (b - P/2) / N)
   __shared__ T vs[kDLMaxP * kDLMaxP];
   __shared__ T part[kFiltSplit][kFiltThreads / kFiltSplit];
-  __shared__ double red[kFiltThreads / 32];
+  __shared__ T sinv;
   const T inv_n = T(1) / ((T)N * (T)N);
   const C* Y = a.yfull + (size_t)l * P * H;
   const int sub = tid % kFiltSplit, o0 = tid / kFiltSplit;
   constexpr int OSTEP = kFiltThreads / kFiltSplit;
-  auto stage = [&](int c0, int nc, bool with_y) {
+  auto stage = [&](int c0, int nc, bool with_y, bool with_w) {
     __syncthreads();  // the previous chunk is consumed
     for (int i = tid; i < P * nc; i += kFiltThreads) {
       const int r = i / nc, c = i - r * nc;
       if (with_y) ys[(size_t)r * chunk + c] = Y[(size_t)r * H + c0 + c];
-      ws[(size_t)r * chunk + c] = tw_at<-1>(a.tw, (c0 + c) * (r - cen), N);
+      if (with_w) ws[(size_t)r * chunk + c] = tw_at<-1>(a.tw, (c0 + c) * (r - cen), N);
     }
     __syncthreads();
   };
+  if (chunk == H) stage(0, H, false, true);  // a single chunk's twiddles, while dl_solve finishes
+  grid_dep_wait();
+  grid_dep_launch();
   for (int ob = 0; ob < PP; ob += OSTEP) {  // outputs ob .. ob + OSTEP - 1 (one pass for P <= 11)
     const int o = ob + o0;
     const int ai = o < PP ? o / P : 0, bi = o < PP ? o - ai * P : 0;
     T acc = T(0);
     for (int c0 = 0; c0 < H; c0 += chunk) {
       const int nc = H - c0 < chunk ? H - c0 : chunk;
-      if (ob == 0 || nc < H) stage(c0, nc, true);  // a single chunk is staged once
+      if (ob == 0 || nc < H) stage(c0, nc, true, nc < H);  // a single chunk is staged once
       if (o < PP) {
         for (int c = sub; c < nc; c += kFiltSplit) {
           const C y = ys[(size_t)ai * chunk + c], t = ws[(size_t)bi * chunk + c];  // Re(y conj(t))
@@ -544,30 +616,46 @@ __global__ void __launch_bounds__(kFiltThreads) dl_filter_kernel(const DLArgs<T>
     }
     if (o < PP) part[sub][o0] = acc;
     __syncthreads();
-    if (sub == 0 && o < PP) vs[o] = (((part[0][o0] + part[1][o0]) + part[2][o0]) + part[3][o0]) * inv_n;
+    if (sub == 0 && o < PP) {
+      T v = part[0][o0];
+#pragma unroll
+      for (int i = 1; i < kFiltSplit; ++i) v += part[i][o0];
+      vs[o] = v * inv_n;
+    }
     __syncthreads();
   }
-  double nn = 0.0;
-  for (int o = tid; o < PP; o += kFiltThreads) nn += (double)vs[o] * (double)vs[o];
-  nn = block_sum256(nn, red);
-  const T inv = nn > 0.0 ? (T)(1.0 / sqrt(nn)) : T(0);
+  // one warp takes the norm (and one lane its reciprocal): the FP64 units retire about two operations
+  // per cycle and SM, so 512 threads summing in doubles cost more than the rest of the kernel
   T* g = a.gs + (size_t)l * PP;
-  double ds = 0.0;
+  if (tid < 32) {
+    double nn = 0.0;
+    for (int o = tid; o < PP; o += 32) nn += (double)vs[o] * (double)vs[o];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
+    if (tid == 0) sinv = nn > 0.0 ? (T)(1.0 / sqrt(nn)) : T(0);
+  }
+  __syncthreads();
+  const T inv = sinv;
+  if (a.check && tid < 32) {
+    double ds = 0.0;
+    for (int o = tid; o < PP; o += 32) {
+      const double dg = (double)(T)(vs[o] * inv) - (double)g[o];
+      ds += dg * dg;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    if (tid == 0) a.spart[l] = ds;
+  }
+  if (a.check) __syncthreads();  // g and vs are read above
   for (int o = tid; o < PP; o += kFiltThreads) {
     const T gn = vs[o] * inv;
-    const double dg = (double)gn - (double)g[o];
-    ds += dg * dg;
     g[o] = gn;
     vs[o] = gn;
-  }
-  if (a.check) {
-    ds = block_sum256(ds, red);
-    if (tid == 0) a.spart[l] = ds;
   }
   // G(a, k2) = sum_b g(a, b) ws[b][k2] over the same chunks (twiddles staged again when chunked)
   for (int c0 = 0; c0 < H; c0 += chunk) {
     const int nc = H - c0 < chunk ? H - c0 : chunk;
-    if (nc < H) stage(c0, nc, false);
+    if (nc < H) stage(c0, nc, false, true);
     else __syncthreads();  // vs is final
     for (int o = tid; o < P * nc; o += kFiltThreads) {
       const int ai = o / nc, c = o - ai * nc;
@@ -587,68 +675,85 @@ __global__ void __launch_bounds__(kFiltThreads) dl_filter_kernel(const DLArgs<T>
 // filters; the dual update e-hat <- e-hat + d-hat - g-hat = w - g-hat (Eq. h_admm), stored as
 // F(g - e) = 2 g-hat - w; p = sum_l theta_l z_l for the next x-update; and, before a check, the
 // primal residual |F(d - g)|^2 = |w - e-hat_old - g-hat|^2 (Parseval on the half spectrum).
+// The two groups divide the filters for g-hat, left in shared memory, and then the channels for p (each
+// p still a sum over all filters in order): 31 -> 18 us at 256^2 x 5, L = 32.
 template <typename T, int M, int PM>
-__global__ void __launch_bounds__(kDLBlock) dl_spec_kernel(const DLArgs<T> a) {
+__global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kernel(const DLArgs<T> a) {
   using C = typename CT<T>::type;
   const int N = a.N, L = a.L, P = a.P, CP = col_pitch(N);
-  const int tid = threadIdx.x;
-  const int k1 = blockIdx.x * kDLBlock + tid, k2 = blockIdx.y;
-  __shared__ C gk[32][PM];
-  __shared__ double red[8];
-  for (int i = tid; i < 32 * PM; i += kDLBlock) {
+  const int tid = threadIdx.x, grp = tid / kDLBlock, bt = tid - grp * kDLBlock;
+  const int k1 = blockIdx.x * kDLBlock + bt, k2 = blockIdx.y;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  C* gk = reinterpret_cast<C*>(dsm);  // [32][PM]
+  C* gs = gk + 32 * PM;               // [L][kDLBlock]: g-hat of this CTA's bins
+  __shared__ double red[kDLThreads / 32];
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int i = tid; i < 32 * PM; i += kDLThreads) {
     const int l = i / PM, ai = i - l * PM;
-    gk[l][ai] = (l < L && ai < P) ? a.gfac[((size_t)k2 * L + l) * P + ai] : mk<C>(0.0, 0.0);
+    gk[i] = (l < L && ai < P) ? a.gfac[((size_t)k2 * L + l) * P + ai] : mk<C>(0.0, 0.0);
   }
   __syncthreads();
   const int cen = P / 2;
   C wa[PM];
 #pragma unroll
   for (int i = 0; i < PM; ++i) wa[i] = i < P ? tw_at<-1>(a.tw, k1 * (i - cen), N) : mk<C>(0.0, 0.0);
-  C pm[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) pm[m] = mk<C>(0.0, 0.0);
   T r2 = T(0);
   C* th = a.spec + (size_t)k2 * 2 * L * CP + k1;
   const C* wb = a.wcol + (size_t)k2 * L * CP + k1;
   const C* zb = a.zcol + (size_t)k2 * M * L * CP + k1;
-  // operands of filter l + 1 loaded while filter l is processed
-  C wn = wb[0], zn[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) zn[m] = zb[(size_t)m * L * CP];
+  constexpr int U = dl_unroll<T>();
 #pragma unroll 1
-  for (int l = 0; l < L; ++l) {
-    C gh = mk<C>(0.0, 0.0);
+  for (int lb = grp; lb < L; lb += U * kDLGroups) {
+    C wl[U];
 #pragma unroll
-    for (int i = 0; i < PM; ++i) cfma(gh, wa[i], gk[l][i]);
-    const C w = wn;
-    C z[M];
+    for (int u = 0; u < U; ++u)
+      if (lb + u * kDLGroups < L) wl[u] = wb[(size_t)(lb + u * kDLGroups) * CP];
 #pragma unroll
-    for (int m = 0; m < M; ++m) z[m] = zn[m];
-    if (l + 1 < L) {
-      wn = wb[(size_t)(l + 1) * CP];
+    for (int u = 0; u < U; ++u) {
+      const int l = lb + u * kDLGroups;
+      if (l >= L) break;
+      C gh = mk<C>(0.0, 0.0);
 #pragma unroll
-      for (int m = 0; m < M; ++m) zn[m] = zb[((size_t)m * L + l + 1) * CP];
+      for (int i = 0; i < PM; ++i) cfma(gh, wa[i], gk[l * PM + i]);
+      const C w = wl[u];
+      if (a.check) {
+        const C t0 = th[(size_t)l * CP], ge0 = th[(size_t)(L + l) * CP];
+        const T dx = w.x - t0.x + ge0.x - gh.x, dy = w.y - t0.y + ge0.y - gh.y;
+        r2 = fma(dx, dx, fma(dy, dy, r2));
+      }
+      gs[l * kDLBlock + bt] = gh;
+      th[(size_t)l * CP] = gh;
+      th[(size_t)(L + l) * CP] = mk<C>(T(2) * gh.x - w.x, T(2) * gh.y - w.y);
     }
-    if (a.check) {
-      const C t0 = th[(size_t)l * CP], ge0 = th[(size_t)(L + l) * CP];
-      const T dx = w.x - t0.x + ge0.x - gh.x, dy = w.y - t0.y + ge0.y - gh.y;
-      r2 = fma(dx, dx, fma(dy, dy, r2));
-    }
-    th[(size_t)l * CP] = gh;
-    th[(size_t)(L + l) * CP] = mk<C>(T(2) * gh.x - w.x, T(2) * gh.y - w.y);
-#pragma unroll
-    for (int m = 0; m < M; ++m) cfma(pm[m], gh, z[m]);
   }
-#pragma unroll
-  for (int m = 0; m < M; ++m) a.p_out[((size_t)k2 * M + m) * CP + k1] = pm[m];
   if (a.check) {
     const double wgt = (k2 == 0 || k2 == N / 2) ? 1.0 : 2.0;
     double v = wgt * (double)r2;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) a.rpart[(size_t)k2 * gridDim.x + blockIdx.x] = red[0] + red[1];
+  }
+  __syncthreads();
+  // p of channels grp, grp + kDLGroups, ...: each sum runs over all filters in order
+  constexpr int MG = (M + kDLGroups - 1) / kDLGroups;
+  C pm[MG];
+#pragma unroll
+  for (int m = 0; m < MG; ++m) pm[m] = mk<C>(0.0, 0.0);
+#pragma unroll 8
+  for (int l = 0; l < L; ++l) {
+    const C gh = gs[l * kDLBlock + bt];
+#pragma unroll
+    for (int m = 0; m < MG; ++m)
+      if (grp + m * kDLGroups < M) cfma(pm[m], gh, zb[((size_t)(grp + m * kDLGroups) * L + l) * CP]);
+  }
+#pragma unroll
+  for (int m = 0; m < MG; ++m)
+    if (grp + m * kDLGroups < M) a.p_out[((size_t)k2 * M + grp + m * kDLGroups) * CP + k1] = pm[m];
+  if (a.check && tid == 0) {
+    double v = 0.0;
+    for (int w = 0; w < kDLThreads / 32; ++w) v += red[w];
+    a.rpart[(size_t)k2 * gridDim.x + blockIdx.x] = v;
   }
 }
 
@@ -668,19 +773,29 @@ __global__ void dl_rescale_kernel(typename CT<T>::type* __restrict__ spec, int L
   }
 }
 
+template <typename T, int M, int PM> cudaError_t dl_launch(const DLArgs<T>& a, bool spec, cudaStream_t s) {
+  using C = typename CT<T>::type;
+  const dim3 grid(a.N / kDLBlock, a.N / 2 + 1), block(kDLThreads);
+  constexpr size_t sm = (size_t)(kDLBlock * (PM + M) + dl_part<M>()) * sizeof(C);
+  constexpr size_t spec_max = (size_t)32 * (PM + kDLBlock) * sizeof(C);
+  static PerDeviceOnce once;
+  cudaError_t e = once([&] {
+    cudaError_t r = cudaFuncSetAttribute(dl_solve_kernel<T, M, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (r != cudaSuccess) return r;
+    return cudaFuncSetAttribute(dl_spec_kernel<T, M, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spec_max);
+  });
+  if (e != cudaSuccess) return e;
+  if (spec) return launch_pdl(dl_spec_kernel<T, M, PM>, grid, block, (size_t)(32 * PM + a.L * kDLBlock) * sizeof(C), s, 0, a);
+  return launch_pdl(dl_solve_kernel<T, M, PM>, grid, block, sm, s, 0, a);
+}
 template <typename T, int PM> cudaError_t dl_by_m(const DLArgs<T>& a, bool spec, cudaStream_t s) {
-  const dim3 grid(a.N / kDLBlock, a.N / 2 + 1);
   switch (a.M) {
-#define DL_CASE(m)                                                          \
-  case m:                                                                   \
-    if (spec) dl_spec_kernel<T, m, PM><<<grid, kDLBlock, 0, s>>>(a);        \
-    else dl_solve_kernel<T, m, PM><<<grid, kDLBlock, 0, s>>>(a);            \
-    break;
+#define DL_CASE(m) \
+  case m: return dl_launch<T, m, PM>(a, spec, s);
     DL_CASE(1) DL_CASE(2) DL_CASE(3) DL_CASE(4) DL_CASE(5) DL_CASE(6) DL_CASE(7) DL_CASE(8)
 #undef DL_CASE
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 template <typename T> bool dl_args_ok(const DLArgs<T>& a) {
   return a.N % kDLBlock == 0 && a.N <= kTwN && a.L >= 1 && a.L <= 32 && a.P >= 1 && a.P <= kDLMaxP &&
@@ -702,8 +817,7 @@ template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, cudaStrea
     return cudaFuncSetAttribute(dl_filter_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFiltSmem);
   });
   if (e != cudaSuccess) return e;
-  dl_filter_kernel<T><<<a.L, kFiltThreads, sm, s>>>(a, chunk);
-  return cudaGetLastError();
+  return launch_pdl(dl_filter_kernel<T>, dim3(a.L), dim3(kFiltThreads), sm, s, 0, a, chunk);
 }
 template <typename T> cudaError_t launch_dl_spec(const DLArgs<T>& a, cudaStream_t s) {
   if (!dl_args_ok(a)) return cudaErrorInvalidValue;
