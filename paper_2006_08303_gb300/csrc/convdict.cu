@@ -100,7 +100,8 @@ __global__ void __launch_bounds__(128) cd_solve_kernel(CDArgs<T> a) {
 // DFT / cd_solve_kernel / column DFT, moves them six times).
 // What bounds it: shared-memory traffic of the FFT stages (16 passes over the tile, ~20 us at 256^2 x 5
 // with 32 filters); HBM needs 12 us for the two passes over the spectra.  Column pass there 95.7 ->
-// 46.1 us, 128^2 x 3 with 8 filters 16.9 -> 10.0, 512^2 x 3 with 16 filters 100 -> 54 us.
+// 46.1 us (40 with the twiddles of each stage in a table of their own), 128^2 x 3 with 8 filters 16.9 ->
+// 10.0, 512^2 x 3 with 16 filters 100 -> 54 us.
 constexpr int kFuseThreads = 256;
 template <typename T> constexpr int fuse_elems(int N) {  // FFT elements per thread: teams stay inside a warp
   if (sizeof(T) == 4) return N <= 256 ? 8 : (N == 512 ? 16 : 32);
