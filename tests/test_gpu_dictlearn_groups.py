@@ -29,3 +29,26 @@ def test_filter_groups(torch, N, M, L, P, dtype, tol):  # noqa: F811
     assert rel(f, f_or) <= tol, rel(f, f_or)
     assert rel(x, x_or) <= tol, rel(x, x_or)
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+
+
+def test_learning_in_a_batch_equals_alone(torch):  # noqa: F811
+    """The three launches recorded into a batch's graph: bit for bit the plan alone."""
+    from paper_2006_08303_gb300 import api
+
+    def plans():
+        out = []
+        for N, M, L, P in ((64, 3, 5, 7), (128, 5, 9, 11)):
+            h, y, d0 = problem(seed=23, N=N, K=2, M=M, L=L, Pf=P)
+            out.append(learning_plan(torch, h, y, d0, LAM, RHO, BETA, 5.0)[0])
+        return out
+
+    alone, together = plans(), plans()
+    for p in alone:
+        p.iterate(8)
+    batch = api.Batch(together)
+    batch.iterate(8)
+    for a, b in zip(alone, together):
+        assert torch.equal(a.get_x(), b.get_x()) and torch.equal(a.get_dictionary(), b.get_dictionary())
+    batch.close()
+    for p in alone + together:
+        p.close()
