@@ -15,7 +15,8 @@ namespace {
 // A bin's factor is read once, row by row of the packed triangle; each thread copies the rows ahead
 // asynchronously into its own shared-memory slots (no barrier), kRowBufs rows deep, so the loads in
 // flight are not bounded by its registers.  The first rows and the data term are requested before the
-// grid dependency, since they do not depend on the forward column DFTs.  Plain loads (72
+// grid dependency, since they do not depend on the forward column DFTs (lowcol does: no const
+// __restrict__, whose read-only loads the wait does not order).  Plain loads (72
 // registers of them in flight at most) ran at 2.5 TB/s; split column pass before and now: 1024^2 x 10
 // 127.8 -> 106.8 us, 1024^2 x 16 384 -> 206, 512^2 x 10 43.9 -> 30.3, 256^2 x 5 13.1 -> 11.2 us.
 constexpr int kSolveThreads = 128, kRowBufs = 3;
@@ -28,10 +29,9 @@ template <typename T, int MMAX> constexpr size_t solve_smem() {
 
 template <typename T, int MMAX>
 __global__ void __launch_bounds__(kSolveThreads, solve_minblocks<T, MMAX>())
-    solve_split_kernel(typename CT<T>::type* __restrict__ colbuf, const typename CT<T>::type* __restrict__ pinv,
-                       const typename CT<T>::type* __restrict__ xb, int N, int M, int plain,
-                       const typename CT<T>::type* __restrict__ lowcol, const typename CT<T>::type* __restrict__ tw,
-                       T rho) {
+    solve_split_kernel(typename CT<T>::type* __restrict__ colbuf, const typename CT<T>::type* pinv,
+                       const typename CT<T>::type* xb, int N, int M, int plain, const typename CT<T>::type* lowcol,
+                       const typename CT<T>::type* __restrict__ tw, T rho) {
   using C = typename CT<T>::type;
   const int k1 = blockIdx.x * kSolveThreads + threadIdx.x;
   const int k2 = blockIdx.y;

@@ -161,6 +161,8 @@ namespace {
 // global and shared-memory accesses along the rows and by making several outputs from each loaded
 // window.  TS = 32 (a 78 x 78 input tile for 64 x 64 pixels) filters 1.2 rows per output row, TS = 16
 // 1.4; it is taken where it leaves at least two CTAs per SM (wave_tile).
+// A kernel of this chain is resident while the kernel before it still writes what it reads: no
+// const __restrict__ on those pointers, whose read-only loads griddepcontrol.wait does not order.
 // At 512^2 x 10 (all kernels of the chain launched programmatically too) the wavelet prior pass went
 // from 119 to 77 us; at 1024^2 x 10 from 331 to 208 us.
 template <typename T> struct alignas(16) Vec16 { T v[16 / sizeof(T)]; };
@@ -174,7 +176,7 @@ template <typename T, int TS> struct FwdTile {
   static constexpr size_t bytes = ((size_t)ROWS * COLS + (size_t)ROWS * RP) * sizeof(T);
 };
 template <typename T, int TS>
-__global__ void __launch_bounds__(256) dwt2_fwd_kernel(const T* __restrict__ in, int in_pitch, size_t in_plane,
+__global__ void __launch_bounds__(256) dwt2_fwd_kernel(const T* in, int in_pitch, size_t in_plane,
                                                        T* __restrict__ det, int N, T* __restrict__ ll, int ll_pitch,
                                                        size_t ll_plane, int n, const WaveFilt<T> f) {
   using F = FwdTile<T, TS>;
@@ -257,8 +259,8 @@ template <typename T, int TS> struct InvTile {
   static constexpr size_t bytes = ((size_t)4 * CR * CC + (size_t)2 * 2 * TS * VP) * sizeof(T);
 };
 template <typename T, int TS>
-__global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* __restrict__ ll, int ll_pitch, size_t ll_plane,
-                                                       const T* __restrict__ det, int N, T* __restrict__ out,
+__global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* ll, int ll_pitch, size_t ll_plane,
+                                                       const T* det, int N, T* __restrict__ out,
                                                        int out_pitch, size_t out_plane, int n, const WaveFilt<T> f) {
   using F = InvTile<T, TS>;
   using V16 = Vec16<T>;
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(256) dwt2_inv_kernel(const T* __restrict__ ll,
 // the next level, the detail subbands to their Mallat positions in A (pitch N), the final 16 x 16
 // LL to A's corner.  The same filtering as dwt2_fwd_kernel; only the tiling differs.
 template <typename T>
-__global__ void __launch_bounds__(512) dwt2_fwd_fused_kernel(const T* __restrict__ in, int in_pitch, size_t in_plane,
+__global__ void __launch_bounds__(512) dwt2_fwd_fused_kernel(const T* in, int in_pitch, size_t in_plane,
                                                              T* __restrict__ A, int N, int n0, WaveFilt<T> f) {
   extern __shared__ __align__(16) unsigned char wsm[];
   const int pp = n0 + 1;
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(512) dwt2_fwd_fused_kernel(const T* __restrict
 // column inverse then the row inverse of dwt2_inv_kernel over the whole band; the result of the
 // last level goes to out (pitch out_pitch), the others stay in shared memory as the next LL.
 template <typename T>
-__global__ void __launch_bounds__(512) dwt2_inv_fused_kernel(const T* __restrict__ A, int N, T* __restrict__ out,
+__global__ void __launch_bounds__(512) dwt2_inv_fused_kernel(const T* A, int N, T* __restrict__ out,
                                                              int out_pitch, size_t out_plane, int n0, WaveFilt<T> f) {
   extern __shared__ __align__(16) unsigned char wsm[];
   const int q0 = n0 / 2, qp = q0 + 1;
@@ -500,8 +502,8 @@ __global__ void __launch_bounds__(512) dwt2_inv_fused_kernel(const T* __restrict
 // per block (the same five sums and order as the other prior passes) into partials[block].
 template <typename T, int M>
 __global__ void __launch_bounds__(256) wdct_shrink_kernel(T* __restrict__ coef, const ChanDCT<T> cmat,
-                                                          const T* __restrict__ u_in, T* __restrict__ u_out,
-                                                          T* __restrict__ tprev, const T* __restrict__ t_imp,
+                                                          const T* u_in, T* __restrict__ u_out,
+                                                          T* __restrict__ tprev, const T* t_imp,
                                                           double* __restrict__ partials, int N, T tau, int flags) {
   __shared__ double red[8][kNPart];
   grid_dep_wait();
