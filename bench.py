@@ -34,25 +34,40 @@ WORKLOAD = f"spectral_dct_{N}x{N}x{M} (K={K}, 8x8 DCT l1, lambda=1e-3, rho=1e-2,
 METRIC = "ADMM voxel-iter/s"
 # DRAM bytes (read + write) per launch of each pass on this workload, from one ncu capture, with
 # the hash of the kernel sources the capture was taken from (kernel_sources_hash()).  The figure
-# is reported only while the sources still hash to that value; any change to a kernel makes it
-# null until the kernels are captured again.
-TRAFFIC_CAPTURE = {"sources": "dd160a41b14c8130", "bytes": {"column_pass": 81.51e6, "prior_pass": 21.06e6}}
-KERNEL_SOURCES = ("colpass.cu", "passA.cu", "fft.cuh", "common.cuh", "kernels.h")
+# is reported only while the sources still hash to that value (any change to a kernel makes it
+# null until the kernels are captured again) and only for the column pass of the captured form.
+TRAFFIC_CAPTURE = {"sources": "7887b7cc9476df63", "bytes": {"column_pass": 81.51e6, "prior_pass": 21.06e6}}
+KERNEL_UNITS = ("colpass.cu", "passA.cu")  # of the two captured kernels
+CAPTURED_FORM = "fused"                    # column-pass form captured (colpass_fused_kernel)
+
+
+def kernel_sources() -> list:
+    """The captured kernels' units and, in the order met, every header they include from csrc."""
+    csrc = os.path.join(ROOT, "paper_2006_08303_gb300", "csrc")
+    out = list(KERNEL_UNITS)
+    for f in out:  # grows while it is walked
+        with open(os.path.join(csrc, f)) as fh:
+            for line in fh:
+                name = line.split('"')[1] if line.startswith('#include "') else None
+                if name and name not in out and os.path.exists(os.path.join(csrc, name)):
+                    out.append(name)
+    return out
 
 
 def kernel_sources_hash() -> str:
     """sha256 (16 hex digits) over the CUDA sources of the two passes of an iteration."""
     import hashlib
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES:
+    for f in kernel_sources():
         with open(os.path.join(ROOT, "paper_2006_08303_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def measured_traffic(kernel: str):
-    """ncu DRAM bytes per launch of `kernel`, or None when the capture predates the sources."""
-    if TRAFFIC_CAPTURE["sources"] != kernel_sources_hash():
+def measured_traffic(kernel: str, form: str = CAPTURED_FORM):
+    """ncu DRAM bytes per launch of `kernel`, or None when the capture predates the sources or (column
+    pass) the plan runs another form than the captured one."""
+    if TRAFFIC_CAPTURE["sources"] != kernel_sources_hash() or (kernel == "column_pass" and form != CAPTURED_FORM):
         return None
     return TRAFFIC_CAPTURE["bytes"].get(kernel)
 
@@ -898,7 +913,7 @@ def main():
     peak = pk["hbm_gbs"] if pk else 6800.0
     achieved = byts / (avg / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-            "frac": round(achieved / peak, 4), "traffic": measured_traffic(dom), "kernel": dom,
+            "frac": round(achieved / peak, 4), "traffic": measured_traffic(dom, plan.config()["column_pass"]), "kernel": dom,
             "kernel_sources": kernel_sources_hash(),
             "peak_source": "measured" if pk else "fallback",
             "avg_launch_us": {"column_pass": round(avgB * 1e3, 2), "prior_pass": round(avgA * 1e3, 2)},
