@@ -80,9 +80,10 @@ typedef struct cip_options {
   int check_every;  /* residual check period for cip_iterate with tol > 0; 0 = 10 */
   int column_pass;  /* 0 = autotuned at cip_set_measurements (fused vs split, tile width; cached per
                        N, M, dtype and prior for the process, and in the file named by the environment
-                       variable CIP_TUNE_CACHE when set, one "N M dtype prior mode cc variant" line per
+                       variable CIP_TUNE_CACHE when set, one "N M dtype prior mode cc variant recorded" line per
                        decision, read on first use; mode 1 and 3 = fused with and without the factor's ring, 2 =
-                       split), 1 = fused kernel (one CTA per half-spectrum column, factor
+                       split; recorded = the mode, 1 or 2, of iterations in a batch or on the server, which a
+                       line may leave out: then mode, or 1 where that is 3), 1 = fused kernel (one CTA per half-spectrum column, factor
                        streamed by TMA bulk copies; CIP_ERR_UNSUPPORTED where its tile does not fit
                        in shared memory), 2 = split (column FFT / solve / FFT).  TV plans with
                        N >= 2048 always use the split form: it carries their low-column correction

@@ -9,6 +9,7 @@
 #include <fstream>
 #include <map>
 #include <mutex>
+#include <sstream>
 #include <tuple>
 #include <string>
 #include <vector>
@@ -60,6 +61,7 @@ struct cip_plan {
   size_t esz = 4;
   int rowsA = 8, cc = 1, blocksA = 0, blocksB = 0;
   int colmode = 1;  // column pass: 1 fused kernel, 2 split (FFT / solve / FFT), 3 fused without the ring
+  int recmode = 1;  // with colmode 3: the form of recorded iterations (batch, server), 1 or 2
   int avar = 0;     // prior-pass kernel variant (1: the other FFT width, 2: 32; complex64, N = 256 .. 1024)
   int test_fault = 0;  // test-only fault switch (cip_set_test_fault)
   // TV at N >= kLowFixMinN: low-column correction of the x-update (launch_passB_split)
@@ -745,9 +747,9 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
 
 std::mutex g_tune_mu;
 // (N, M, dtype, prior, forced prior-pass variant or -1) -> (column-pass form, fused tile width,
-// prior-pass variant)
+// prior-pass variant, column-pass form of recorded iterations)
 using TuneKey = std::tuple<int, int, int, int, int>;
-using TuneVal = std::tuple<int, int, int>;
+using TuneVal = std::tuple<int, int, int, int>;
 std::map<TuneKey, TuneVal> g_tune;
 bool g_tune_loaded = false;
 
@@ -760,15 +762,20 @@ void tune_cache_load() {
   const char* path = std::getenv("CIP_TUNE_CACHE");
   if (!path || !*path) return;
   std::ifstream in(path);
-  int n, m, dt, pr, mode, cc, av;
-  while (in >> n >> m >> dt >> pr >> mode >> cc >> av) g_tune[std::make_tuple(n, m, dt, pr, -1)] = {mode, cc, av};
+  for (std::string line; std::getline(in, line);) {
+    std::istringstream f(line);
+    int n, m, dt, pr, mode, cc, av, rec;
+    if (!(f >> n >> m >> dt >> pr >> mode >> cc >> av)) continue;
+    if (!(f >> rec)) rec = mode == 3 ? 1 : mode;  // a line without the recorded form
+    g_tune[std::make_tuple(n, m, dt, pr, -1)] = {mode, cc, av, rec};
+  }
 }
 void tune_cache_store(const TuneKey& key, const TuneVal& v) {
   const char* path = std::getenv("CIP_TUNE_CACHE");
   if (!path || !*path || std::get<4>(key) >= 0) return;  // the file holds unforced decisions only
   std::ofstream out(path, std::ios::app);
   out << std::get<0>(key) << ' ' << std::get<1>(key) << ' ' << std::get<2>(key) << ' ' << std::get<3>(key) << ' '
-      << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << '\n';
+      << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << ' ' << std::get<3>(v) << '\n';
 }
 
 bool prior_has_variant(const cip_plan* p) {
@@ -801,6 +808,10 @@ template <typename T> void set_colmode(cip_plan* p, int mode, int cc) {
   if (mode == 1) p->cc = cc;
   p->blocksB = mode != 2 ? p->N / 2 + 1 : p->M * (p->N / 2 + 1);
 }
+// The form of recorded iterations.  Their kernels share the device with other plans' (batch, server), where
+// the form without the ring is no gain (coldirect.cu): they take the faster of the other two, with the
+// same prior-pass width and so the same bits as the plan alone.
+int rec_form(const cip_plan* p) { return p->colmode == 3 ? p->recmode : p->colmode; }
 
 // Autotuner: times whole iterations (column pass, then prior pass, launched back to back as in
 // cip_iterate) for every column-pass form (fused kernel, with and without the ring; split FFT / solve / FFT) and both
@@ -810,7 +821,8 @@ template <typename T> void set_colmode(cip_plan* p, int mode, int cc) {
 // well, not at every cip_set_measurements (14 to 28 iterations and the event waits between them:
 // 2.5 ms of the 8.6 ms of a 40-iteration 512 x 512 x 10 wavelet reconstruction).  The prior pass reads u[cur] and writes the
 // other u buffer and q-hat without moving cur, so repeating an iteration keeps its inputs; the
-// state is reset afterwards (cip_set_measurements).
+// state is reset afterwards (cip_set_measurements).  Where the form without the ring wins, the faster of
+// the other two at the same width is kept beside it for recorded iterations (rec_form).
 template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   using C = typename CT<T>::type;
   const int fav = forced_avar(p);
@@ -827,8 +839,9 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
     if (it != g_tune.end()) {
       set_colmode<T>(p, std::get<0>(it->second), std::get<1>(it->second));
       p->avar = std::get<2>(it->second);
+      p->recmode = std::get<3>(it->second) == 2 ? 2 : 1;
       // a cached choice of the split form still needs this plan's own column buffer
-      if (p->colmode == 2 && !p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));
+      if (rec_form(p) == 2 && !p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));
       return CIP_OK;
     }
   }
@@ -837,20 +850,21 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   const int av0 = fav < 0 ? 0 : fav, av1 = fav < 0 ? (has_wide_variant(p) ? 2 : 1) : fav;
   for (int av = av0; av <= av1; ++av) {
     if (is_cd(p)) {  // dictionary plans have one column-pass form; only the prior-pass width is tuned
-      cands.push_back({p->colmode, p->cc, av});
+      cands.push_back({p->colmode, p->cc, av, p->colmode});
       continue;
     }
     if (colpass_fused_fits<T>(p->N, p->M)) {
-      cands.push_back({1, 1, av});
-      if (direct_ok(p)) cands.push_back({3, 1, av});
+      cands.push_back({1, 1, av, 1});
+      if (direct_ok(p)) cands.push_back({3, 1, av, 1});
     }
-    cands.push_back({2, 0, av});
+    cands.push_back({2, 0, av, 2});
   }
   cudaEvent_t e0, e1;
   CIP_CUDA(p, cudaEventCreate(&e0));
   CIP_CUDA(p, cudaEventCreate(&e1));
-  float best = 1e30f;
-  TuneVal pick = {p->colmode, p->cc, p->avar};
+  float best = 1e30f, best_rec = 1e30f;
+  std::vector<float> took;
+  TuneVal pick = {p->colmode, p->cc, p->avar, p->colmode};
   auto iteration = [&]() -> cip_status {
     cip_status st = column_pass<T>(p, s, p->colmode, p->cc);
     if (st != CIP_OK) return st;
@@ -869,15 +883,23 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
     CIP_CUDA(p, cudaEventSynchronize(e1));
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
+    took.push_back(ms);
     if (ms < best) {
       best = ms;
       pick = c;
     }
   }
+  if (std::get<0>(pick) == 3)
+    for (size_t i = 0; i < cands.size(); ++i)
+      if (std::get<0>(cands[i]) != 3 && std::get<2>(cands[i]) == std::get<2>(pick) && took[i] < best_rec) {
+        best_rec = took[i];
+        std::get<3>(pick) = std::get<0>(cands[i]);
+      }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   set_colmode<T>(p, std::get<0>(pick), std::get<1>(pick));
   p->avar = std::get<2>(pick);
+  p->recmode = std::get<3>(pick) == 2 ? 2 : 1;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune[key] = pick;
   tune_cache_store(key, pick);
@@ -1090,10 +1112,9 @@ template <typename T> cip_status iterate_impl(cip_plan* p, int max_iter, double 
 }
 
 // One iteration (column pass, prior pass) enqueued with no host synchronisation and no timing
-// events, so that it can be recorded into a CUDA graph.  Its kernels share the device with other plans'
-// (batch, server): the fused column pass runs in its ring form (coldirect.cu says why; the bits are the same).
+// events, so that it can be recorded into a CUDA graph.
 template <typename T> cip_status enqueue_iteration(cip_plan* p, cudaStream_t s, int flags) {
-  cip_status cst = column_pass<T>(p, s, p->colmode == 3 ? 1 : p->colmode, p->cc);
+  cip_status cst = column_pass<T>(p, s, rec_form(p), p->cc);
   if (cst != CIP_OK) return cst;
   if (p->dl_sigma > 0) {
     cst = dict_step<T>(p, s);

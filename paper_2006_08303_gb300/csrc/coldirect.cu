@@ -10,7 +10,9 @@
 // Where the ring kernel's few stages serve few solving warps one after the other, here every bin is
 // solved at once from data that is already in shared memory: the iteration alone on the device takes
 // less time.  It issues more instructions (a copy and a load per entry), so iterations that share the
-// device with other plans' (batches, the server) keep the ring kernel.
+// device with other plans' (batches, the server) run the faster of the ring kernel and the split form
+// instead (8 TV plans of 1024^2 x 3 in a batch: split 337 us an iteration of all, ring 369; of 1024^2 x 1
+// 147 and 225).
 // One iteration, ring -> this kernel: 64^2 x 3 TV 5.71 -> 5.05 us, 256^2 x 3 8.86 -> 8.15, 512^2 x 5 24.5 ->
 // 22.7, 1024^2 x 3 50.2 (split) -> 48.7; 16 plans of 128^2 .. 512^2 in a batch 8.38 -> 9.0 ms.  With 10
 // channels at 512^2 (whose slots leave room for three rows ahead) 37.1 -> 37.8: not offered.
