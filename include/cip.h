@@ -285,8 +285,9 @@ cip_status cip_get_timing(cip_plan* plan, double* prior_pass_ms, int* prior_pass
                           int* column_pass_n);
 
 /* Test-only fault switch for the bounded device waits (no counterpart in the paper).
- * kind 1: the prior pass of CIP_PRIOR_DCT8 plans (at sizes whose u rows it stages in shared memory
- * by a bulk copy) and of CIP_PRIOR_L1 plans (which stage nothing and arm a barrier for this test) arms its copy barrier for two arrivals, gives one and issues no
+ * kind 1: the prior pass of CIP_PRIOR_DCT8, CIP_PRIOR_TV and CIP_PRIOR_TV_ISO plans (at sizes whose u
+ * rows it stages in shared memory by bulk copies: TV in complex64 up to N = 512) and of CIP_PRIOR_L1
+ * plans (which stage nothing and arm a barrier for this test) arms its copy barrier for two arrivals, gives one and issues no
  * copy, then waits at most 64 polls: the wait gives up with nothing in flight, the kernel reads u
  * from global memory instead (the iterate is unchanged) and flags the plan, so that
  * cip_get_residuals (and the residual checks of cip_iterate) return CIP_ERR_TIMEOUT until the

@@ -290,9 +290,14 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
   if constexpr (TVSTAGE) {
     // per component the row above the tile (wraps to the last row) and the tile's R rows
     if (tid == 0) {
-      mbar_init(&ubar, 1);
-      mbar_arrive_expect_tx(&ubar, (unsigned)(2 * (R + 1) * N * sizeof(T)));
-      if (!import_mode) stage_tv();
+      if (a.test_fault == 1) {  // as for the DCT tile above
+        mbar_init(&ubar, 2);
+        mbar_arrive(&ubar);
+      } else {
+        mbar_init(&ubar, 1);
+        mbar_arrive_expect_tx(&ubar, (unsigned)(2 * (R + 1) * N * sizeof(T)));
+        if (!import_mode) stage_tv();
+      }
     }
     __syncthreads();  // the barrier is initialised before anyone waits on it
   }
@@ -313,7 +318,9 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     if constexpr (USTAGE) {
       if (a.test_fault != 1) bulk_copy_g2s(us, u_in + (size_t)r0 * N, (unsigned)(R * N * sizeof(T)), &ubar);
     }
-    if constexpr (TVSTAGE) stage_tv();
+    if constexpr (TVSTAGE) {
+      if (a.test_fault != 1) stage_tv();
+    }
   }
   if (!import_mode) {
     // 1. gather the row half-spectra of the tile (two rows per complex FFT) from the column
@@ -373,7 +380,18 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     };
     constexpr bool ISO = PRIOR == PRIOR_TV_ISO;
     const C czero = mk<C>(0.0, 0.0);
-    if constexpr (TVSTAGE) mbar_wait_bounded(&ubar, 0, a.err);  // a failure is flagged: the iterate is then invalid
+    if constexpr (TVSTAGE) {
+      // a warp whose wait gave up (the plan is flagged) copies the rows itself: whoever else writes them,
+      // a late bulk copy included, writes the same values
+      u_ok = mbar_wait_bounded(&ubar, 0, a.err, a.test_fault ? 64 : (1 << 22));
+      if (__any_sync(0xffffffffu, !u_ok)) {
+        for (int i = tid & 31; i < 2 * (R + 1) * N; i += 32) {
+          const int comp = i / ((R + 1) * N), r = i - comp * (R + 1) * N;
+          us[i] = u_in[comp * plane + (size_t)grow(r / N) * N + (r & (N - 1))];
+        }
+        __syncwarp();
+      }
+    }
     // isotropic TV: the pixel's two components shrink together (group soft threshold)
     auto group = [&](T wh, T uh, T wv, T uv, T& th, T& uhn, T& ah, T& tv, T& uvn, T& av) {
       const T vh = wh + uh, vv = wv + uv;
@@ -720,10 +738,7 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
     }
   }
   if (resid) block_reduce_store<T>(part, a.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kNPart);
-  if constexpr (TVSTAGE) {
-    if (tid == 0) mbar_wait_bounded(&ubar, 0, a.err);  // as below, for a wait that gave up
-  }
-  if constexpr (USTAGE) {
+  if constexpr (USTAGE || TVSTAGE) {
     // a copy that was only late must not write this CTA's shared memory after the CTA ends
     if (tid == 0 && !u_ok && a.test_fault == 0) mbar_wait_bounded(&ubar, 0, a.err);
   }
