@@ -286,9 +286,8 @@ cip_status cip_get_timing(cip_plan* plan, double* prior_pass_ms, int* prior_pass
 
 /* Test-only fault switch for the bounded device waits (no counterpart in the paper).
  * kind 1: the prior pass of CIP_PRIOR_DCT8, CIP_PRIOR_TV and CIP_PRIOR_TV_ISO plans (at sizes whose u
- * rows it stages in shared memory by bulk copies: TV in complex64 up to N = 512) and of CIP_PRIOR_L1
- * plans (which stage nothing and arm a barrier for this test) arms its copy barrier for two arrivals, gives one and issues no
- * copy, then waits at most 64 polls: the wait gives up with nothing in flight, the kernel reads u
+ * rows it stages in shared memory by bulk copies: TV in complex64 up to N = 512) arms its copy barrier
+ * for two arrivals, gives one and issues no copy, then waits at most 64 polls: the wait gives up with nothing in flight, the kernel reads u
  * from global memory instead (the iterate is unchanged) and flags the plan, so that
  * cip_get_residuals (and the residual checks of cip_iterate) return CIP_ERR_TIMEOUT until the
  * next state reset.  kind 0: off (the default).  CIP_ERR_INVALID_ARG for other kinds. */

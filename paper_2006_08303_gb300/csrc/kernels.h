@@ -43,7 +43,7 @@ template <typename T> struct PassAArgs {
   T tau;            // lambda / rho
   T qscale;         // rho / 2 (the 1/2 of the pair extraction is folded here)
   int flags;
-  int test_fault;   // 1: the staged u copy is replaced by a barrier that never completes (test of
+  int test_fault;   // 1 (DCT and TV tiles that stage u): the staged copy is replaced by a barrier that never completes (test of
                     // the bounded wait: no copy is issued, the wait gives up after 64 polls)
   int variant;      // 1: the kernel variant with the other FFT width (complex64, N = 256 .. 1024); 2: 32
                     // elements per thread (T = I, complex64, N = 256)

@@ -74,15 +74,6 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN, V), row_minblocks<T>
   C z[E];  // element i: position tt + TT i
 
   if constexpr (KIND == PRIOR_L1) {
-    __shared__ unsigned long long fbar;
-    if (a.test_fault == 1) {  // the bounded wait of a barrier that never completes (cip_set_test_fault)
-      if (tid == 0) {
-        mbar_init(&fbar, 2);
-        mbar_arrive(&fbar);
-        mbar_wait_bounded(&fbar, 0, a.err, 64);
-      }
-      __syncthreads();
-    }
     // u (and t_prev) rows into L2 while the preceding kernel drains; an import's u is not final yet
     if (tid == 0 && !import_mode) prefetch_l2(u_in + (size_t)r0 * N, (size_t)R * N * sizeof(T));
     if (tid == 32 % NT && resid) prefetch_l2(a.tprev + (size_t)m * plane + (size_t)r0 * N, (size_t)R * N * sizeof(T));
