@@ -746,9 +746,11 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
 }
 
 std::mutex g_tune_mu;
-// (N, M, dtype, prior, forced prior-pass variant or -1) -> (column-pass form, fused tile width,
-// prior-pass variant, column-pass form of recorded iterations)
-using TuneKey = std::tuple<int, int, int, int, int>;
+// (N, M, dtype, prior, maps of a dictionary's prior pass, forced prior-pass variant or -1) -> (column-pass
+// form, fused tile width, prior-pass variant, column-pass form of recorded iterations).  Maps: M L for
+// dictionaries, whose row pass runs over them and fills the device or not; 0 for the other priors (M says it)
+// and in a line of the file that names none, which then holds for every number of filters.
+using TuneKey = std::tuple<int, int, int, int, int, int>;
 using TuneVal = std::tuple<int, int, int, int>;
 std::map<TuneKey, TuneVal> g_tune;
 bool g_tune_loaded = false;
@@ -764,18 +766,21 @@ void tune_cache_load() {
   std::ifstream in(path);
   for (std::string line; std::getline(in, line);) {
     std::istringstream f(line);
-    int n, m, dt, pr, mode, cc, av, rec;
+    int n, m, dt, pr, mode, cc, av, rec, maps;
     if (!(f >> n >> m >> dt >> pr >> mode >> cc >> av)) continue;
     if (!(f >> rec)) rec = mode == 3 ? 1 : mode;  // a line without the recorded form
-    g_tune[std::make_tuple(n, m, dt, pr, -1)] = {mode, cc, av, rec};
+    if (!(f >> maps) || pr != CIP_PRIOR_CONVDICT) maps = 0;
+    g_tune[std::make_tuple(n, m, dt, pr, maps, -1)] = {mode, cc, av, rec};
   }
 }
 void tune_cache_store(const TuneKey& key, const TuneVal& v) {
   const char* path = std::getenv("CIP_TUNE_CACHE");
-  if (!path || !*path || std::get<4>(key) >= 0) return;  // the file holds unforced decisions only
+  if (!path || !*path || std::get<5>(key) >= 0) return;  // the file holds unforced decisions only
   std::ofstream out(path, std::ios::app);
   out << std::get<0>(key) << ' ' << std::get<1>(key) << ' ' << std::get<2>(key) << ' ' << std::get<3>(key) << ' '
-      << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << ' ' << std::get<3>(v) << '\n';
+      << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << ' ' << std::get<3>(v);
+  if (std::get<4>(key) > 0) out << ' ' << std::get<4>(key);
+  out << '\n';
 }
 
 bool prior_has_variant(const cip_plan* p) {
@@ -816,7 +821,7 @@ int rec_form(const cip_plan* p) { return p->colmode == 3 ? p->recmode : p->colmo
 // Autotuner: times whole iterations (column pass, then prior pass, launched back to back as in
 // cip_iterate) for every column-pass form (fused kernel, with and without the ring; split FFT / solve / FFT) and both
 // prior-pass FFT widths where a variant exists, on this plan's buffers, and keeps the fastest,
-// cached per (N, M, dtype, prior, forced width) for the process: plans with one width (wavelet
+// cached per (N, M, dtype, prior, maps of a dictionary, forced width) for the process: plans with one width (wavelet
 // prior, complex128, N < 256, N = 2048) and plans with a forced one time their candidates once as
 // well, not at every cip_set_measurements (14 to 28 iterations and the event waits between them:
 // 2.5 ms of the 8.6 ms of a 40-iteration 512 x 512 x 10 wavelet reconstruction).  The prior pass reads u[cur] and writes the
@@ -826,7 +831,8 @@ int rec_form(const cip_plan* p) { return p->colmode == 3 ? p->recmode : p->colmo
 template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   using C = typename CT<T>::type;
   const int fav = forced_avar(p);
-  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, prior_has_variant(p) ? fav : -1);
+  const int kfav = prior_has_variant(p) ? fav : -1;
+  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, is_cd(p) ? smaps(p) : 0, kfav);
   if (low_fix(p)) {  // the low-column correction of large TV plans is part of the split form
     set_colmode<T>(p, 2, p->cc);
     if (!p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));
@@ -836,6 +842,7 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_cache_load();
     auto it = g_tune.find(key);
+    if (it == g_tune.end()) it = g_tune.find(std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, 0, kfav));
     if (it != g_tune.end()) {
       set_colmode<T>(p, std::get<0>(it->second), std::get<1>(it->second));
       p->avar = std::get<2>(it->second);
