@@ -687,7 +687,7 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mo
     // dictionary: column DFT of rho (t - u) over the L*M coefficient maps, the per-(bin, channel)
     // x- and z-update, inverse column DFT of v
     const int S = smaps(p);
-    const bool fused = p->Q == 0 && cd_fused_fits<T>(p->N, p->L);
+    const bool fused = p->Q == 0 && cd_fused_fits<T>(p->N, p->M, p->L);
     if (!fused)
       CIP_LAUNCH(p, launch_cols_fft<T>(static_cast<const C*>(p->qh), static_cast<C*>(p->colbuf),
                                        static_cast<const C*>(p->tw), p->N, S, -1, s));

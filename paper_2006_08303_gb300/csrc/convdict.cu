@@ -867,9 +867,24 @@ template <typename T> cudaError_t launch_cd_solve(const CDArgs<T>& a, cudaStream
   return cudaGetLastError();
 }
 
-template <typename T> bool cd_fused_fits(int N, int L) { return fuse_smem<T>(N, L) > 0; }
+// Where it runs.  Fewer filters than FFT teams leave warps of a CTA idle for two whole FFTs, which costs most
+// where a team's FFT is longest: complex64 at N = 1024 runs it from 8 filters (a team each) on; one channel,
+// 7 filters 62.9 us against 49.1 in three kernels, 8 filters 47.1 against 56.2, three channels 1 filter
+// 83.0 and 51.3, eight 209 and 189, but for 16 channels, where an iteration takes 629 and 670 us (below N = 1024
+// it is the faster one from one filter on: 512^2 x 8 41.7 and 47.5).
+// complex128 CTAs hold an SM each (registers), so that beyond one wave they queue while each waits for
+// its few FP64 units: 256^2 x 8 with 1 filter 236 us against 138, 9 filters 433 and 373, 512^2 x 3 9 filters 787
+// and 561; in one wave 256^2 x 1 9 filters 62.6 and 82.5; two waves with little work each 512^2 x 1 2 filters
+// 87.7 and 94.2, 4 filters 108.7 and 100.5.  Up to N = 128 it is the faster one but for 12 and more filters in
+// some waves (128^2 x 3: 1 filter 22.8 and 42.1, 32 filters 160 and 136).
+template <typename T> bool cd_fused_fits(int N, int M, int L) {
+  if (fuse_smem<T>(N, L) == 0) return false;
+  if (sizeof(T) == 4) return N < 1024 || L >= kFuseThreads / (N / fuse_elems<T>(N)) || M >= 12;
+  const int ctas = M * (N / 2 + 1), sms = 152;
+  return N <= 128 || ctas <= sms || (ctas <= 2 * sms && L <= 3);
+}
 template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s) {
-  if (a.L < 1 || a.L > 32 || !cd_fused_fits<T>(a.N, a.L)) return cudaErrorInvalidValue;
+  if (a.L < 1 || a.L > 32 || !cd_fused_fits<T>(a.N, a.M, a.L)) return cudaErrorInvalidValue;
   switch (a.N) {
     case 64: return launch_fused<T, 6>(a, s);
     case 128: return launch_fused<T, 7>(a, s);
@@ -879,8 +894,8 @@ template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream
     default: return cudaErrorInvalidValue;
   }
 }
-template bool cd_fused_fits<float>(int, int);
-template bool cd_fused_fits<double>(int, int);
+template bool cd_fused_fits<float>(int, int, int);
+template bool cd_fused_fits<double>(int, int, int);
 template cudaError_t launch_cd_fused<float>(const CDArgs<float>&, cudaStream_t);
 template cudaError_t launch_cd_fused<double>(const CDArgs<double>&, cudaStream_t);
 

@@ -96,8 +96,9 @@ template <typename T> struct CDArgs {
 };
 template <typename T> cudaError_t launch_cd_solve(const CDArgs<T>& a, cudaStream_t s);
 // the column pass around it (column DFT, solve, inverse column DFT) in one kernel, one CTA per
-// (column, channel); fits: the L column spectra of a channel fit in shared memory
-template <typename T> bool cd_fused_fits(int N, int L);
+// (column, channel); fits: it can run (the L column spectra of a channel fit in
+// shared memory) and is the faster form
+template <typename T> bool cd_fused_fits(int N, int M, int L);
 template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s);
 
 // 3D dictionary (Section IV-B, 3D case; csrc/convdict3d.cu): the same column layout for the
