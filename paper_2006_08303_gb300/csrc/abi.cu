@@ -287,7 +287,7 @@ template <typename T> cip_status alloc_state(cip_plan* p) {
     CIP_CUDA(p, cudaMemcpyAsync(p->wcos, c.data(), c.size() * sizeof(T), cudaMemcpyHostToDevice, p->ast));
     CIP_CUDA(p, cudaStreamSynchronize(p->ast));
   }
-  p->rowsA = prior_pass_kind(p) == PRIOR_L1 ? rowpass_rows(p->N) : passA_rows<T>(p->N, tile_kind(p->prior));
+  p->rowsA = prior_pass_kind(p) == PRIOR_L1 ? rowpass_rows<T>(p->N) : passA_rows<T>(p->N, tile_kind(p->prior));
   p->blocksA = (p->N / p->rowsA) * smaps(p);
   // the wavelet prior's shrinkage: a thread per pixel (all channels), at most 2048 blocks
   if (p->prior == CIP_PRIOR_WDCT) p->blocksA = std::min(p->N * p->N / 256, 2048);

@@ -168,7 +168,7 @@ cudaError_t launch_theta_store(const SetupC<T>* th64, typename CT<T>::type* th, 
 
 // The same for T = I (the l1 prior, dictionary codes) and the row transforms alone (csrc/rowpass.cu);
 // kind: PRIOR_L1, ROWS_OUT or ROWS_IN.  rows: rows per CTA; elems: FFT elements per thread.
-int rowpass_rows(int N);
+template <typename T> int rowpass_rows(int N);
 template <typename T> int rowpass_elems(int N, int variant);
 template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, cudaStream_t s);
 

@@ -21,21 +21,24 @@ namespace cip {
 
 namespace {
 
-// FFT elements per thread.  V is the plan's prior-pass variant: complex64 at N = 256 .. 1024 has 8, 16
+// FFT elements per thread.  complex128 takes 8 up to N = 256: its tiles wait for the latency of their few
+// FP64 units, and twice the threads halve the serial chain (with 8-row tiles, see row_rows: the l1 pass of
+// 64^2 42.4 -> 21.9 us, 128^2 46.3 -> 25.0, 256^2 53.7 -> 43.0).  V is the plan's prior-pass variant: complex64 at N = 256 .. 1024 has 8, 16
 // and (N = 256, where 32 merges the last two stages) 32 to choose from, timed by the autotuner.
 template <typename T> constexpr int row_elems(int N, int V) {
-  if (sizeof(T) == 8) return 16;
+  if (sizeof(T) == 8) return N <= 256 ? 8 : 16;
   if (N == 64) return 8;
   if (N == 128) return 8;
   if (N == 2048) return 32;
   const int e = N == 512 ? 16 : 8;  // the width the plan reports for V = 0 (prior_fft_default)
   return V == 0 ? e : (V == 1 ? 24 - e : 32);
 }
-// rows per CTA: 16 give whole 128-byte lines of the column layout; 8 from N = 512 on, where the tile
-// has threads enough, and at N = 128, where 16 would halve the few CTAs of small problems
-constexpr int row_rows(int N) { return N == 64 || N == 256 ? 16 : 8; }
+// rows per CTA: 16 give whole 128-byte lines of the column layout; 8 from N = 512 on, where the
+// tile has threads enough, and at N = 128, where 16 would halve the few CTAs of small problems; 8 in
+// complex128, where a row pair is 32 bytes and the time is that of the SM with the most rows
+template <typename T> constexpr int row_rows(int N) { return sizeof(T) == 4 && (N == 64 || N == 256) ? 16 : 8; }
 constexpr int row_slot(int N) { return spad(N) + (N >= 256 ? 4 : 0); }
-template <typename T> constexpr int row_threads(int N, int V) { return row_rows(N) / 2 * (N / row_elems<T>(N, V)); }
+template <typename T> constexpr int row_threads(int N, int V) { return row_rows<T>(N) / 2 * (N / row_elems<T>(N, V)); }
 template <typename T> constexpr int row_minblocks(int N, int V) {
   const int e = row_elems<T>(N, V);
   const int regs = sizeof(T) == 8 ? 168 : (e == 32 ? 128 : (e == 16 ? 80 : 56));
@@ -47,7 +50,7 @@ template <typename T, int LOGN, int KIND, int V>
 __global__ void __launch_bounds__(row_threads<T>(1 << LOGN, V), row_minblocks<T>(1 << LOGN, V))
     row_kernel(const PassAArgs<T> a) {
   using C = typename CT<T>::type;
-  constexpr int N = 1 << LOGN, H = N / 2 + 1, E = row_elems<T>(N, V), TT = N / E, R = row_rows(N), NP = R / 2;
+  constexpr int N = 1 << LOGN, H = N / 2 + 1, E = row_elems<T>(N, V), TT = N / E, R = row_rows<T>(N), NP = R / 2;
   constexpr int ZS = row_slot(N), CP = col_pitch(N), NT = row_threads<T>(N, V);
   constexpr int S8 = LOGN / 3, REM = LOGN % 3;
   constexpr bool MERGE = fft_merges<C, LOGN, E>();
@@ -207,7 +210,7 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN, V), row_minblocks<T>
 template <typename T, int LOGN, int KIND, int V> cudaError_t launch_row(const PassAArgs<T>& a, cudaStream_t s) {
   using C = typename CT<T>::type;
   constexpr int N = 1 << LOGN;
-  constexpr size_t sm = (size_t)row_rows(N) / 2 * row_slot(N) * sizeof(C);
+  constexpr size_t sm = (size_t)row_rows<T>(N) / 2 * row_slot(N) * sizeof(C);
   auto k = row_kernel<T, LOGN, KIND, V>;
   static PerDeviceOnce once;
   cudaError_t e = once([&] {
@@ -218,7 +221,7 @@ template <typename T, int LOGN, int KIND, int V> cudaError_t launch_row(const Pa
     return cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
   });
   if (e != cudaSuccess) return e;
-  return launch_pdl(k, dim3(N / row_rows(N), a.M), dim3(row_threads<T>(N, V)), sm, s, 0, a);
+  return launch_pdl(k, dim3(N / row_rows<T>(N), a.M), dim3(row_threads<T>(N, V)), sm, s, 0, a);
 }
 
 template <typename T, int KIND> cudaError_t dispatch_row(const PassAArgs<T>& a, int N, cudaStream_t s) {
@@ -260,7 +263,9 @@ template <typename T, int KIND> cudaError_t dispatch_row(const PassAArgs<T>& a, 
 
 }  // namespace
 
-int rowpass_rows(int N) { return row_rows(N); }
+template <typename T> int rowpass_rows(int N) { return row_rows<T>(N); }
+template int rowpass_rows<float>(int);
+template int rowpass_rows<double>(int);
 template <typename T> int rowpass_elems(int N, int variant) { return row_elems<T>(N, variant); }
 template int rowpass_elems<float>(int, int);
 template int rowpass_elems<double>(int, int);
