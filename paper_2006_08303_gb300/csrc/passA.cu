@@ -106,9 +106,12 @@ template <typename T> constexpr int threads_for(int N, int prior, int R, int V =
 // CTAs per SM the register budget is cut for: as many as shared memory and the
 // thread limit allow, at <= ~48 registers per thread for complex64 (so that a
 // 10-channel 512 x 512 prior pass runs as one wave) and <= ~168 for complex128
-// (whose 16-element FFT registers would otherwise spill).
-template <typename T> constexpr int minblocks_for(int nth, size_t smem, bool tv) {
-  const int by_regs = 65536 / (nth * (sizeof(T) == 4 ? (tv ? PASSA_TV_RT32 : PASSA_RT32) : 168));
+// (whose 16-element FFT registers would otherwise spill).  The 256 threads of a complex128 TV tile
+// take <= 128 from N = 128 on, two CTAs instead of one: 0 to 276 bytes of spills, but 128^2 x 8 74.5 -> 57.1 us an
+// iteration, 256^2 x 8 178 -> 160, 512^2 x 8 472 -> 447 (at N = 64, 192 bytes, 70.2 -> 73.7 for 16 channels).
+template <typename T> constexpr int minblocks_for(int nth, size_t smem, bool tv, int N) {
+  const int by_regs =
+      65536 / (nth * (sizeof(T) == 4 ? (tv ? PASSA_TV_RT32 : PASSA_RT32) : (tv && N >= 128 ? 128 : 168)));
   const int by_smem = (int)((227 * 1024) / (smem + 1024));
   const int by_thr = 2048 / nth;
   int b = by_regs < by_smem ? by_regs : by_smem;
@@ -212,7 +215,7 @@ __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(
 template <typename T, int LOGN, int PRIOR, int R, int V>
 __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
                                   minblocks_for<T>(threads_for<T>(1 << LOGN, PRIOR, R, V),
-                                                   smem_for<T>(1 << LOGN, PRIOR, R), prior_is_tv(PRIOR)))
+                                                   smem_for<T>(1 << LOGN, PRIOR, R), prior_is_tv(PRIOR), 1 << LOGN))
     passA_kernel(const PassAArgs<T> a) {
   using C = typename CT<T>::type;
   constexpr int N = 1 << LOGN;
