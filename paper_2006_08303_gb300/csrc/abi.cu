@@ -581,9 +581,29 @@ template <typename T> PassAArgs<T> passA_args(cip_plan* p, int flags) {
 
 template <typename T> PassBArgs<T> passB_args(cip_plan* p);
 
+// Whether the kernels of an iteration start programmatically.  In complex128 an SM's few FP64 units make two
+// CTAs on one SM take twice as long, and CTAs that start while the other pass still holds SMs are placed two on one:
+// where a pass has about one CTA per SM the early start costs far more than the launch latency it hides.  The
+// line: the column pass has about a CTA per SM or more, and the prior pass is small (fewer than 5 2^18 pixels in
+// all maps; beyond, many tiles per SM even out).  Iterations, early and plain: l1 512^2 x 1 150 and 100 us, x 4
+// 212 and 176, x 5 243 and 248; DCT 256^2 x 8 180 and 131, 128^2 x 8 82 and 87; wavelet 512^2 x 1 420 and 330; dictionary
+// 64^2 x 8 with 9 filters 109 and 54.  One channel of 256^2 and TV below six gain nothing (TV 256^2 x 4 85 and 87).
+// In a batch, early and plain: 4 l1 plans of 512^2 x 2 317 and 288 us an iteration of all, six
+// mixed ones 437 and 375.
+// The filter update's own kernels: 128^2 x 8 with 9 filters 442 and 360, 256^2 x 3 613 and 584, 64^2 x 3 126 and 136.
+template <typename T> Chain chain(const cip_plan* p, cudaStream_t s) {
+  if (sizeof(T) == 4 || (is_cd(p) && p->Q > 0)) return {s, true};
+  if (is_cd(p) && p->dl_sigma > 0) return {s, p->N < 128};
+  const int col = (is_cd(p) ? p->M : 1) * (p->N / 2 + 1);
+  const long long px = (long long)smaps(p) * p->N * p->N;
+  const bool tv = p->prior == CIP_PRIOR_TV || p->prior == CIP_PRIOR_TV_ISO;
+  const int few = p->prior == CIP_PRIOR_WDCT ? 64 : 128;  // the wavelet chain's eleven kernels collide earlier
+  return {s, col < few || px >= 5 << 18 || px < (tv ? 6 << 16 : (is_cd(p) ? 1 << 15 : 2 << 16))};
+}
+
 // Row transforms between the column-layout row spectra and real rows ([maps][N][N]): x = row IDFT of `spec` into `rows` (read-back, wavelet
 // chain), or spec = row DFT of scale * rows.
-template <typename T> cudaError_t rows_from_spec(cip_plan* p, const void* spec, int maps, void* rows, cudaStream_t s) {
+template <typename T> cudaError_t rows_from_spec(cip_plan* p, const void* spec, int maps, void* rows, Chain s) {
   using C = typename CT<T>::type;
   PassAArgs<T> a{};
   a.xh = static_cast<const C*>(spec);
@@ -594,7 +614,7 @@ template <typename T> cudaError_t rows_from_spec(cip_plan* p, const void* spec, 
   return launch_rowpass<T>(a, p->N, ROWS_OUT, s);
 }
 template <typename T>
-cudaError_t spec_from_rows(cip_plan* p, const void* rows, int maps, double scale, void* spec, cudaStream_t s) {
+cudaError_t spec_from_rows(cip_plan* p, const void* rows, int maps, double scale, void* spec, Chain s) {
   using C = typename CT<T>::type;
   PassAArgs<T> a{};
   a.qh = static_cast<C*>(spec);
@@ -610,7 +630,8 @@ cudaError_t spec_from_rows(cip_plan* p, const void* rows, int maps, double scale
 // (not local to a row tile) the chain x = row IDFT, J wavelet levels, channel DCT + shrinkage +
 // dual + residual partials, J inverse levels, q-hat = rho row DFT(q).  In import mode x is not
 // needed and the chain starts at the shrinkage kernel.
-template <typename T> cip_status prior_pass(cip_plan* p, const PassAArgs<T>& a, cudaStream_t s) {
+template <typename T> cip_status prior_pass(cip_plan* p, const PassAArgs<T>& a, cudaStream_t stream) {
+  const Chain s = chain<T>(p, stream);
   if (p->prior != CIP_PRIOR_WDCT) {
     CIP_LAUNCH(p, launch_passA<T>(a, p->N, prior_pass_kind(p), s));
     return CIP_OK;
@@ -681,8 +702,9 @@ template <typename T> CD3Args<T> cd3_args(cip_plan* p) {
 }
 
 // the column pass in the plan's chosen form
-template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t s, int mode, int cc) {
+template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t stream, int mode, int cc) {
   using C = typename CT<T>::type;
+  const Chain s = chain<T>(p, stream);
   if (is_cd(p)) {
     // dictionary: column DFT of rho (t - u) over the L*M coefficient maps, the per-(bin, channel)
     // x- and z-update, inverse column DFT of v
@@ -977,7 +999,8 @@ template <typename T> DLArgs<T> dl_args(cip_plan* p, bool check) {
 // sold_3D), g from Eq. g_admm, e from Eq. h_admm; theta = F g and p = sum_l theta_l z_l formed
 // again, so that the next x-update sees the updated dictionary (reading R21).  Three launches;
 // with `check` they also leave the sums of ||d - g||^2 and ||g - g_prev||^2 in dl_part.
-template <typename T> cip_status dict_step(cip_plan* p, cudaStream_t s, bool check = false) {
+template <typename T> cip_status dict_step(cip_plan* p, cudaStream_t stream, bool check = false) {
+  const Chain s = chain<T>(p, stream);
   const DLArgs<T> a = dl_args<T>(p, check);
   CIP_LAUNCH(p, launch_dl_solve<T>(a, s));
   CIP_LAUNCH(p, launch_dl_filter<T>(a, s));

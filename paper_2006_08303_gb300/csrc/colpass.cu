@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kColThreads) colfft_cols_kernel(const typename
 
 template <typename T, int LOGN, int SIGN>
 cudaError_t launch_cols(const typename CT<T>::type* src, typename CT<T>::type* dst, const typename CT<T>::type* tw,
-                        int ncols, cudaStream_t s, const typename CT<T>::type* src2, typename CT<T>::type* dst2,
+                        int ncols, Chain s, const typename CT<T>::type* src2, typename CT<T>::type* dst2,
                         int ncols2) {
   using C = typename CT<T>::type;
   constexpr int N = 1 << LOGN, TT = N / cp_elems<T>(N), TEAMS = kColThreads / TT;
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(fused_threads<T, LOGN, MMAX>(), fused_minblock
 }
 
 template <typename T, int LOGN, int MMAX>
-cudaError_t launch_fused_m(const FusedArgs<T>& a, const FusedShape<T>& f, cudaStream_t s) {
+cudaError_t launch_fused_m(const FusedArgs<T>& a, const FusedShape<T>& f, Chain s) {
   auto k = colpass_fused_kernel<T, LOGN, MMAX>;
   static PerDeviceOnce once;
   // the attribute is set to the largest size any shape of this instantiation may ask for
@@ -337,7 +337,7 @@ cudaError_t launch_fused_m(const FusedArgs<T>& a, const FusedShape<T>& f, cudaSt
 }
 
 template <typename T, int LOGN>
-cudaError_t launch_fused_n(const FusedArgs<T>& a, const FusedShape<T>& f, cudaStream_t s) {
+cudaError_t launch_fused_n(const FusedArgs<T>& a, const FusedShape<T>& f, Chain s) {
   if (a.M <= 4) return launch_fused_m<T, LOGN, 4>(a, f, s);
   if (a.M <= 8) return launch_fused_m<T, LOGN, 8>(a, f, s);
   if (a.M <= 10) return launch_fused_m<T, LOGN, 10>(a, f, s);
@@ -362,7 +362,7 @@ template <typename T> bool colpass_fused_fits(int N, int M) {
 
 template <typename T> size_t colpass_fused_smem(int N, int M) { return fused_shape<T>(N, M, optin_smem()).smem; }
 
-template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, int S, int* err, cudaStream_t s) {
+template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, int S, int* err, Chain s) {
   const FusedShape<T> f = fused_shape<T>(b.N, b.M, optin_smem());
   if (f.smem > optin_smem()) return cudaErrorInvalidConfiguration;
   if (f.nstage < 2 || f.threads > 1024) return cudaErrorInvalidConfiguration;
@@ -391,7 +391,7 @@ template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, in
 
 template <typename T>
 cudaError_t launch_cols_fft(const typename CT<T>::type* src, typename CT<T>::type* dst,
-                            const typename CT<T>::type* tw, int N, int maps, int sign, cudaStream_t s,
+                            const typename CT<T>::type* tw, int N, int maps, int sign, Chain s,
                             const typename CT<T>::type* src2, typename CT<T>::type* dst2, int ncols2) {
   const int ncols = (N / 2 + 1) * maps;
 #define CIP_COLS(L) \
@@ -413,11 +413,11 @@ template bool colpass_fused_fits<float>(int, int);
 template bool colpass_fused_fits<double>(int, int);
 template size_t colpass_fused_smem<float>(int, int);
 template size_t colpass_fused_smem<double>(int, int);
-template cudaError_t launch_colpass_fused<float>(const PassBArgs<float>&, int, int*, cudaStream_t);
-template cudaError_t launch_colpass_fused<double>(const PassBArgs<double>&, int, int*, cudaStream_t);
-template cudaError_t launch_cols_fft<float>(const float2*, float2*, const float2*, int, int, int, cudaStream_t,
+template cudaError_t launch_colpass_fused<float>(const PassBArgs<float>&, int, int*, Chain);
+template cudaError_t launch_colpass_fused<double>(const PassBArgs<double>&, int, int*, Chain);
+template cudaError_t launch_cols_fft<float>(const float2*, float2*, const float2*, int, int, int, Chain,
                                             const float2*, float2*, int);
-template cudaError_t launch_cols_fft<double>(const double2*, double2*, const double2*, int, int, int, cudaStream_t,
+template cudaError_t launch_cols_fft<double>(const double2*, double2*, const double2*, int, int, int, Chain,
                                              const double2*, double2*, int);
 
 }  // namespace cip

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kSolveThreads, solve_minblocks<T, MMAX>())
 template <typename T, int MMAX>
 cudaError_t solve_launch(typename CT<T>::type* colbuf, const typename CT<T>::type* pinv, const typename CT<T>::type* xb,
                          int N, int M, int plain, const typename CT<T>::type* lowcol, const typename CT<T>::type* tw,
-                         T rho, cudaStream_t s) {
+                         T rho, Chain s) {
   auto k = solve_split_kernel<T, MMAX>;
   constexpr size_t sm = solve_smem<T, MMAX>();
   static PerDeviceOnce once;
@@ -131,7 +131,7 @@ cudaError_t solve_launch(typename CT<T>::type* colbuf, const typename CT<T>::typ
 template <typename T>
 cudaError_t solve_m(typename CT<T>::type* colbuf, const typename CT<T>::type* pinv, const typename CT<T>::type* xb,
                     int N, int M, int plain, const typename CT<T>::type* lowcol, const typename CT<T>::type* tw,
-                    T rho, cudaStream_t s) {
+                    T rho, Chain s) {
 #define CIP_SOLVE(MM) \
   return solve_launch<T, MM>(colbuf, pinv, xb, N, M, plain, lowcol, tw, rho, s)
   if (M <= 4) CIP_SOLVE(4);
@@ -146,7 +146,7 @@ cudaError_t solve_m(typename CT<T>::type* colbuf, const typename CT<T>::type* pi
 }  // namespace
 
 template <typename T>
-cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colbuf, int N, cudaStream_t s,
+cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colbuf, int N, Chain s,
                                int* launches, const typename CT<T>::type* lowbuf, typename CT<T>::type* lowcol,
                                T rho) {
   // q-hat and x-hat use the column layout already: the column DFTs need no transposition; the
@@ -160,9 +160,9 @@ cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colb
   return e;
 }
 
-template cudaError_t launch_passB_split<float>(const PassBArgs<float>&, float2*, int, cudaStream_t, int*,
+template cudaError_t launch_passB_split<float>(const PassBArgs<float>&, float2*, int, Chain, int*,
                                                const float2*, float2*, float);
-template cudaError_t launch_passB_split<double>(const PassBArgs<double>&, double2*, int, cudaStream_t, int*,
+template cudaError_t launch_passB_split<double>(const PassBArgs<double>&, double2*, int, Chain, int*,
                                                 const double2*, double2*, double);
 
 }  // namespace cip

@@ -198,22 +198,32 @@ struct PerDeviceOnce {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Launch `kern` with programmatic stream serialisation (plus a cluster of
+// The stream of an iteration's kernels, and whether each may start programmatically before its predecessor ends.
+struct Chain {
+  cudaStream_t s;
+  bool early;
+  Chain(cudaStream_t stream, bool start_early = true) : s(stream), early(start_early) {}
+  operator cudaStream_t() const { return s; }
+};
+
+// Launch `kern` with programmatic stream serialisation where the chain starts kernels early (plus a cluster of
 // cluster_x CTAs along x when cluster_x > 0).  The kernel must call grid_dep_wait() before it touches any
 // memory that an earlier kernel of the stream writes or reads.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Chain s,
                               unsigned cluster_x, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
+  cfg.stream = s.s;
   cudaLaunchAttribute attr[2];
   unsigned n = 0;
-  attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[n].val.programmaticStreamSerializationAllowed = 1;
-  ++n;
+  if (s.early) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
   if (cluster_x > 0) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
     attr[n].val.clusterDim.x = cluster_x;

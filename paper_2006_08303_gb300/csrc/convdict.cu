@@ -202,7 +202,7 @@ template <typename T> size_t fuse_smem(int N, int L) {
   return sm <= 224 * 1024 ? sm : 0;
 }
 
-template <typename T, int LOGN> cudaError_t launch_fused(const CDArgs<T>& a, cudaStream_t s) {
+template <typename T, int LOGN> cudaError_t launch_fused(const CDArgs<T>& a, Chain s) {
   if constexpr ((1 << LOGN) / fuse_elems<T>(1 << LOGN) > 32) {
     return cudaErrorInvalidValue;
   } else {
@@ -774,7 +774,7 @@ __global__ void dl_rescale_kernel(typename CT<T>::type* __restrict__ spec, int L
   }
 }
 
-template <typename T, int M, int PM> cudaError_t dl_launch(const DLArgs<T>& a, bool spec, cudaStream_t s) {
+template <typename T, int M, int PM> cudaError_t dl_launch(const DLArgs<T>& a, bool spec, Chain s) {
   using C = typename CT<T>::type;
   const dim3 grid(a.N / kDLBlock, a.N / 2 + 1), block(kDLThreads);
   constexpr size_t sm = (size_t)(kDLBlock * (PM + M) + dl_part<M>()) * sizeof(C);
@@ -789,7 +789,7 @@ template <typename T, int M, int PM> cudaError_t dl_launch(const DLArgs<T>& a, b
   if (spec) return launch_pdl(dl_spec_kernel<T, M, PM>, grid, block, (size_t)(32 * PM + a.L * kDLBlock) * sizeof(C), s, 0, a);
   return launch_pdl(dl_solve_kernel<T, M, PM>, grid, block, sm, s, 0, a);
 }
-template <typename T, int PM> cudaError_t dl_by_m(const DLArgs<T>& a, bool spec, cudaStream_t s) {
+template <typename T, int PM> cudaError_t dl_by_m(const DLArgs<T>& a, bool spec, Chain s) {
   switch (a.M) {
 #define DL_CASE(m) \
   case m: return dl_launch<T, m, PM>(a, spec, s);
@@ -805,11 +805,11 @@ template <typename T> bool dl_args_ok(const DLArgs<T>& a) {
 
 }  // namespace
 
-template <typename T> cudaError_t launch_dl_solve(const DLArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_dl_solve(const DLArgs<T>& a, Chain s) {
   if (!dl_args_ok(a)) return cudaErrorInvalidValue;
   return a.P <= 16 ? dl_by_m<T, 16>(a, false, s) : dl_by_m<T, 32>(a, false, s);
 }
-template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, Chain s) {
   if (!dl_args_ok(a)) return cudaErrorInvalidValue;
   const int chunk = filt_chunk<T>(a.N, a.P);
   const size_t sm = 2 * (size_t)a.P * chunk * sizeof(typename CT<T>::type);
@@ -820,7 +820,7 @@ template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, cudaStrea
   if (e != cudaSuccess) return e;
   return launch_pdl(dl_filter_kernel<T>, dim3(a.L), dim3(kFiltThreads), sm, s, 0, a, chunk);
 }
-template <typename T> cudaError_t launch_dl_spec(const DLArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_dl_spec(const DLArgs<T>& a, Chain s) {
   if (!dl_args_ok(a)) return cudaErrorInvalidValue;
   return a.P <= 16 ? dl_by_m<T, 16>(a, true, s) : dl_by_m<T, 32>(a, true, s);
 }
@@ -829,12 +829,12 @@ cudaError_t launch_dl_rescale(typename CT<T>::type* spec, int L, int N, T f, cud
   dl_rescale_kernel<T><<<4 * 152, 256, 0, s>>>(spec, L, N, f);
   return cudaGetLastError();
 }
-template cudaError_t launch_dl_solve<float>(const DLArgs<float>&, cudaStream_t);
-template cudaError_t launch_dl_solve<double>(const DLArgs<double>&, cudaStream_t);
-template cudaError_t launch_dl_filter<float>(const DLArgs<float>&, cudaStream_t);
-template cudaError_t launch_dl_filter<double>(const DLArgs<double>&, cudaStream_t);
-template cudaError_t launch_dl_spec<float>(const DLArgs<float>&, cudaStream_t);
-template cudaError_t launch_dl_spec<double>(const DLArgs<double>&, cudaStream_t);
+template cudaError_t launch_dl_solve<float>(const DLArgs<float>&, Chain);
+template cudaError_t launch_dl_solve<double>(const DLArgs<double>&, Chain);
+template cudaError_t launch_dl_filter<float>(const DLArgs<float>&, Chain);
+template cudaError_t launch_dl_filter<double>(const DLArgs<double>&, Chain);
+template cudaError_t launch_dl_spec<float>(const DLArgs<float>&, Chain);
+template cudaError_t launch_dl_spec<double>(const DLArgs<double>&, Chain);
 template cudaError_t launch_dl_rescale<float>(float2*, int, int, float, cudaStream_t);
 template cudaError_t launch_dl_rescale<double>(double2*, int, int, double, cudaStream_t);
 
@@ -883,7 +883,7 @@ template <typename T> bool cd_fused_fits(int N, int M, int L) {
   const int ctas = M * (N / 2 + 1), sms = 152;
   return N <= 128 || ctas <= sms || (ctas <= 2 * sms && L <= 3);
 }
-template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, Chain s) {
   if (a.L < 1 || a.L > 32 || !cd_fused_fits<T>(a.N, a.M, a.L)) return cudaErrorInvalidValue;
   switch (a.N) {
     case 64: return launch_fused<T, 6>(a, s);
@@ -896,8 +896,8 @@ template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream
 }
 template bool cd_fused_fits<float>(int, int, int);
 template bool cd_fused_fits<double>(int, int, int);
-template cudaError_t launch_cd_fused<float>(const CDArgs<float>&, cudaStream_t);
-template cudaError_t launch_cd_fused<double>(const CDArgs<double>&, cudaStream_t);
+template cudaError_t launch_cd_fused<float>(const CDArgs<float>&, Chain);
+template cudaError_t launch_cd_fused<double>(const CDArgs<double>&, Chain);
 
 template <typename Tin>
 cudaError_t launch_embed_filters(const Tin* d, double* out, int L, int P, int N, cudaStream_t s) {

@@ -99,7 +99,7 @@ template <typename T> cudaError_t launch_cd_solve(const CDArgs<T>& a, cudaStream
 // (column, channel); fits: it can run (the L column spectra of a channel fit in
 // shared memory) and is the faster form
 template <typename T> bool cd_fused_fits(int N, int M, int L);
-template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_cd_fused(const CDArgs<T>& a, Chain s);
 
 // 3D dictionary (Section IV-B, 3D case; csrc/convdict3d.cu): the same column layout for the
 // channel-domain spectra; theta holds Theta_l(kappa, w) at plane kappa*L + l of [H][M*L][CP].
@@ -156,9 +156,9 @@ template <typename T> struct DLArgs {
   int check;       // 1: form the residual sums (an adaptation check follows this step)
   T sigma;
 };
-template <typename T> cudaError_t launch_dl_solve(const DLArgs<T>& a, cudaStream_t s);
-template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, cudaStream_t s);
-template <typename T> cudaError_t launch_dl_spec(const DLArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_dl_solve(const DLArgs<T>& a, Chain s);
+template <typename T> cudaError_t launch_dl_filter(const DLArgs<T>& a, Chain s);
+template <typename T> cudaError_t launch_dl_spec(const DLArgs<T>& a, Chain s);
 // F(g - e) <- theta - (theta - F(g - e)) f: the scaled dual times f = sigma_old / sigma_new
 template <typename T>
 cudaError_t launch_dl_rescale(typename CT<T>::type* spec, int L, int N, T f, cudaStream_t s);
@@ -170,18 +170,18 @@ cudaError_t launch_theta_store(const SetupC<T>* th64, typename CT<T>::type* th, 
 // kind: PRIOR_L1, ROWS_OUT or ROWS_IN.  rows: rows per CTA; elems: FFT elements per thread.
 template <typename T> int rowpass_rows(int N);
 template <typename T> int rowpass_elems(int N, int variant);
-template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, cudaStream_t s);
+template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, Chain s);
 
 template <typename T> int passA_rows(int N, int prior);
 template <typename T> size_t passA_smem(int N, int prior);
-template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int prior, cudaStream_t s);
+template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int prior, Chain s);
 
 // Fused column pass (csrc/colpass.cu): one CTA per half-spectrum column, factor and data term
 // streamed through a ring of TMA bulk copies.  fits: the tile and at least two ring stages fit in
 // shared memory.  `err` is set when a bounded wait gives up.
 template <typename T> bool colpass_fused_fits(int N, int M);
 template <typename T> size_t colpass_fused_smem(int N, int M);
-template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, int S, int* err, cudaStream_t s);
+template <typename T> cudaError_t launch_colpass_fused(const PassBArgs<T>& b, int S, int* err, Chain s);
 // The same for few channels without the ring (csrc/coldirect.cu): faster alone on the device.
 bool coldirect_fits(int N, int M);
 cudaError_t launch_coldirect(const PassBArgs<float>& b, int S, cudaStream_t s);
@@ -189,7 +189,7 @@ cudaError_t launch_coldirect(const PassBArgs<float>& b, int S, cudaStream_t s);
 // sign < 0 forward, > 0 inverse (unnormalised)
 template <typename T>
 cudaError_t launch_cols_fft(const typename CT<T>::type* src, typename CT<T>::type* dst,
-                            const typename CT<T>::type* tw, int N, int maps, int sign, cudaStream_t s,
+                            const typename CT<T>::type* tw, int N, int maps, int sign, Chain s,
                             const typename CT<T>::type* src2 = nullptr, typename CT<T>::type* dst2 = nullptr,
                             int ncols2 = 0);
 // split form: column FFT of qh into colbuf (same layout), per-bin solve in place, inverse column FFT
@@ -199,7 +199,7 @@ cudaError_t launch_cols_fft(const typename CT<T>::type* src, typename CT<T>::typ
 // near DC the FP32 transforms of q = D^T (t - u) carry a uniform rounding error that Psi^{-1}
 // amplifies by ~1/g, the transforms of the components of t - u do not.
 template <typename T>
-cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colbuf, int N, cudaStream_t s,
+cudaError_t launch_passB_split(const PassBArgs<T>& a, typename CT<T>::type* colbuf, int N, Chain s,
                                int* launches, const typename CT<T>::type* lowbuf = nullptr,
                                typename CT<T>::type* lowcol = nullptr, T rho = T(0));
 
@@ -259,10 +259,10 @@ bool symlet_lowpass(int p, double* h);
 // and the details from det -> the n x n band into `out`.
 template <typename T>
 cudaError_t launch_dwt2_fwd(const T* in, int in_pitch, size_t in_plane, T* det, int N, T* ll, int ll_pitch,
-                            size_t ll_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s);
+                            size_t ll_plane, int n, int M, const WaveFilt<T>& f, Chain s);
 template <typename T>
 cudaError_t launch_dwt2_inv(const T* ll, int ll_pitch, size_t ll_plane, const T* det, int N, T* out, int out_pitch,
-                            size_t out_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s);
+                            size_t out_plane, int n, int M, const WaveFilt<T>& f, Chain s);
 // Bands of side n <= wave_fuse_n run all their remaining levels in one kernel, one CTA per
 // channel, in shared memory (2 n0 (n0 + 1) values forward, 2 n0 (n0 / 2 + 1) inverse).  wave_fuse_band(N): the side
 // of the first such band of an N x N image.  Forward: band n0 from `in` -> details and the final
@@ -271,14 +271,14 @@ template <typename T> constexpr int wave_fuse_n() { return 64; }
 template <typename T> int wave_fuse_band(int N);
 template <typename T>
 cudaError_t launch_dwt2_fwd_fused(const T* in, int in_pitch, size_t in_plane, T* A, int N, int n0, int M,
-                                  const WaveFilt<T>& f, cudaStream_t s);
+                                  const WaveFilt<T>& f, Chain s);
 template <typename T>
 cudaError_t launch_dwt2_inv_fused(const T* A, int N, T* out, int out_pitch, size_t out_plane, int n0, int M,
-                                  const WaveFilt<T>& f, cudaStream_t s);
+                                  const WaveFilt<T>& f, Chain s);
 // per pixel: channel DCT (cmat [M][M], row k = frequency), shrinkage / dual update / residual
 // partials as the other prior passes (flags PA_*), q = t - u', coefficients <- C^T q in place
 template <typename T>
 cudaError_t launch_wdct_shrink(T* coef, const ChanDCT<T>& cmat, const T* u_in, T* u_out, T* tprev, const T* t_imp,
-                               double* partials, int blocks, int N, int M, T tau, int flags, cudaStream_t s);
+                               double* partials, int blocks, int N, int M, T tau, int flags, Chain s);
 
 }  // namespace cip

@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(threads_for<T>(1 << LOGN, PRIOR, R, V),
 }
 
 template <typename T, int LOGN, int PRIOR, int V>
-cudaError_t launchA(const PassAArgs<T>& a, cudaStream_t s) {
+cudaError_t launchA(const PassAArgs<T>& a, Chain s) {
   constexpr int N = 1 << LOGN;
   constexpr int R = rows_for<T>(N, PRIOR);
   constexpr int nth = threads_for<T>(N, PRIOR, R, V);
@@ -769,7 +769,7 @@ cudaError_t launchA(const PassAArgs<T>& a, cudaStream_t s) {
 }
 
 template <typename T, int PRIOR>
-cudaError_t dispatchA(const PassAArgs<T>& a, int N, cudaStream_t s) {
+cudaError_t dispatchA(const PassAArgs<T>& a, int N, Chain s) {
   if constexpr (has_variant<T>(256, PRIOR)) {
     if (a.variant == 1) {
       switch (N) {
@@ -796,7 +796,7 @@ cudaError_t dispatchA(const PassAArgs<T>& a, int N, cudaStream_t s) {
 template <typename T> int passA_rows(int N, int prior) { return rows_for<T>(N, prior); }
 template <typename T> size_t passA_smem(int N, int prior) { return smem_for<T>(N, prior, rows_for<T>(N, prior)); }
 
-template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int prior, cudaStream_t s) {
+template <typename T> cudaError_t launch_passA(const PassAArgs<T>& a, int N, int prior, Chain s) {
   switch (prior) {
     case PRIOR_TV: return dispatchA<T, PRIOR_TV>(a, N, s);
     case PRIOR_TV_ISO: return dispatchA<T, PRIOR_TV_ISO>(a, N, s);
@@ -810,7 +810,7 @@ template int passA_rows<float>(int, int);
 template int passA_rows<double>(int, int);
 template size_t passA_smem<float>(int, int);
 template size_t passA_smem<double>(int, int);
-template cudaError_t launch_passA<float>(const PassAArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_passA<double>(const PassAArgs<double>&, int, int, cudaStream_t);
+template cudaError_t launch_passA<float>(const PassAArgs<float>&, int, int, Chain);
+template cudaError_t launch_passA<double>(const PassAArgs<double>&, int, int, Chain);
 
 }  // namespace cip

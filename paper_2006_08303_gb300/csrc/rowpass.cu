@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN, V), row_minblocks<T>
   if (resid) block_reduce_store<T>(part, a.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kNPart);
 }
 
-template <typename T, int LOGN, int KIND, int V> cudaError_t launch_row(const PassAArgs<T>& a, cudaStream_t s) {
+template <typename T, int LOGN, int KIND, int V> cudaError_t launch_row(const PassAArgs<T>& a, Chain s) {
   using C = typename CT<T>::type;
   constexpr int N = 1 << LOGN;
   constexpr size_t sm = (size_t)row_rows<T>(N) / 2 * row_slot(N) * sizeof(C);
@@ -224,7 +224,7 @@ template <typename T, int LOGN, int KIND, int V> cudaError_t launch_row(const Pa
   return launch_pdl(k, dim3(N / row_rows<T>(N), a.M), dim3(row_threads<T>(N, V)), sm, s, 0, a);
 }
 
-template <typename T, int KIND> cudaError_t dispatch_row(const PassAArgs<T>& a, int N, cudaStream_t s) {
+template <typename T, int KIND> cudaError_t dispatch_row(const PassAArgs<T>& a, int N, Chain s) {
   // the row transforms alone take the variant that was fastest for them at every size (V below)
   if constexpr (sizeof(T) == 4) {
     const int v = KIND == PRIOR_L1 ? a.variant : (N == 256 ? 2 : (N == 1024 ? 1 : 0));
@@ -270,7 +270,7 @@ template <typename T> int rowpass_elems(int N, int variant) { return row_elems<T
 template int rowpass_elems<float>(int, int);
 template int rowpass_elems<double>(int, int);
 
-template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, cudaStream_t s) {
+template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, int kind, Chain s) {
   switch (kind) {
     case PRIOR_L1: return dispatch_row<T, PRIOR_L1>(a, N, s);
     case ROWS_OUT: return dispatch_row<T, ROWS_OUT>(a, N, s);
@@ -278,7 +278,7 @@ template <typename T> cudaError_t launch_rowpass(const PassAArgs<T>& a, int N, i
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_rowpass<float>(const PassAArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_rowpass<double>(const PassAArgs<double>&, int, int, cudaStream_t);
+template cudaError_t launch_rowpass<float>(const PassAArgs<float>&, int, int, Chain);
+template cudaError_t launch_rowpass<double>(const PassAArgs<double>&, int, int, Chain);
 
 }  // namespace cip

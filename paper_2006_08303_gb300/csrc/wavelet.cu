@@ -585,7 +585,7 @@ int wave_tile(int n, int M) { return n >= 64 && (n / 64) * (n / 64) * M >= 2 * 1
 
 template <typename T, int TS>
 cudaError_t fwd_level(const T* in, int in_pitch, size_t in_plane, T* det, int N, T* ll, int ll_pitch, size_t ll_plane,
-                      int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+                      int n, int M, const WaveFilt<T>& f, Chain s) {
   auto k = dwt2_fwd_kernel<T, TS>;
   constexpr size_t sm = FwdTile<T, TS>::bytes;
   static PerDeviceOnce once;
@@ -596,7 +596,7 @@ cudaError_t fwd_level(const T* in, int in_pitch, size_t in_plane, T* det, int N,
 }
 template <typename T, int TS>
 cudaError_t inv_level(const T* ll, int ll_pitch, size_t ll_plane, const T* det, int N, T* out, int out_pitch,
-                      size_t out_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+                      size_t out_plane, int n, int M, const WaveFilt<T>& f, Chain s) {
   auto k = dwt2_inv_kernel<T, TS>;
   constexpr size_t sm = InvTile<T, TS>::bytes;
   static PerDeviceOnce once;
@@ -609,7 +609,7 @@ cudaError_t inv_level(const T* ll, int ll_pitch, size_t ll_plane, const T* det, 
 
 template <typename T>
 cudaError_t launch_dwt2_fwd(const T* in, int in_pitch, size_t in_plane, T* det, int N, T* ll, int ll_pitch,
-                            size_t ll_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+                            size_t ll_plane, int n, int M, const WaveFilt<T>& f, Chain s) {
   if (n < 32 || n > N || (n & (n - 1))) return cudaErrorInvalidValue;
   return wave_tile(n, M) == 32 ? fwd_level<T, 32>(in, in_pitch, in_plane, det, N, ll, ll_pitch, ll_plane, n, M, f, s)
                                : fwd_level<T, 16>(in, in_pitch, in_plane, det, N, ll, ll_pitch, ll_plane, n, M, f, s);
@@ -617,7 +617,7 @@ cudaError_t launch_dwt2_fwd(const T* in, int in_pitch, size_t in_plane, T* det, 
 
 template <typename T>
 cudaError_t launch_dwt2_inv(const T* ll, int ll_pitch, size_t ll_plane, const T* det, int N, T* out, int out_pitch,
-                            size_t out_plane, int n, int M, const WaveFilt<T>& f, cudaStream_t s) {
+                            size_t out_plane, int n, int M, const WaveFilt<T>& f, Chain s) {
   if (n < 32 || n > N || (n & (n - 1))) return cudaErrorInvalidValue;
   return wave_tile(n, M) == 32 ? inv_level<T, 32>(ll, ll_pitch, ll_plane, det, N, out, out_pitch, out_plane, n, M, f, s)
                                : inv_level<T, 16>(ll, ll_pitch, ll_plane, det, N, out, out_pitch, out_plane, n, M, f, s);
@@ -627,7 +627,7 @@ template <typename T> int wave_fuse_band(int N) { return N < wave_fuse_n<T>() ? 
 
 template <typename T>
 cudaError_t launch_dwt2_fwd_fused(const T* in, int in_pitch, size_t in_plane, T* A, int N, int n0, int M,
-                                  const WaveFilt<T>& f, cudaStream_t s) {
+                                  const WaveFilt<T>& f, Chain s) {
   if (n0 < 32 || n0 > wave_fuse_n<T>() || n0 > N || (n0 & (n0 - 1))) return cudaErrorInvalidValue;
   const size_t sm = 2 * (size_t)n0 * (n0 + 1) * sizeof(T);
   static PerDeviceOnce once;
@@ -641,7 +641,7 @@ cudaError_t launch_dwt2_fwd_fused(const T* in, int in_pitch, size_t in_plane, T*
 
 template <typename T>
 cudaError_t launch_dwt2_inv_fused(const T* A, int N, T* out, int out_pitch, size_t out_plane, int n0, int M,
-                                  const WaveFilt<T>& f, cudaStream_t s) {
+                                  const WaveFilt<T>& f, Chain s) {
   if (n0 < 32 || n0 > wave_fuse_n<T>() || n0 > N || (n0 & (n0 - 1))) return cudaErrorInvalidValue;
   const size_t sm = 8 * (size_t)(n0 / 2) * (n0 / 2 + 1) * sizeof(T);  // C: 4 q (q + 1), V: 2 n0 (q + 1)
   static PerDeviceOnce once;
@@ -656,7 +656,7 @@ cudaError_t launch_dwt2_inv_fused(const T* A, int N, T* out, int out_pitch, size
 
 template <typename T>
 cudaError_t launch_wdct_shrink(T* coef, const ChanDCT<T>& cmat, const T* u_in, T* u_out, T* tprev, const T* t_imp,
-                               double* partials, int blocks, int N, int M, T tau, int flags, cudaStream_t s) {
+                               double* partials, int blocks, int N, int M, T tau, int flags, Chain s) {
   if (blocks < 1) return cudaErrorInvalidValue;
   switch (M) {
 #define WS_CASE(m)                                                                                              \
@@ -671,26 +671,26 @@ cudaError_t launch_wdct_shrink(T* coef, const ChanDCT<T>& cmat, const T* u_in, T
 }
 
 template cudaError_t launch_dwt2_fwd<float>(const float*, int, size_t, float*, int, float*, int, size_t, int, int,
-                                            const WaveFilt<float>&, cudaStream_t);
+                                            const WaveFilt<float>&, Chain);
 template cudaError_t launch_dwt2_fwd<double>(const double*, int, size_t, double*, int, double*, int, size_t, int, int,
-                                             const WaveFilt<double>&, cudaStream_t);
+                                             const WaveFilt<double>&, Chain);
 template cudaError_t launch_dwt2_inv<float>(const float*, int, size_t, const float*, int, float*, int, size_t, int,
-                                            int, const WaveFilt<float>&, cudaStream_t);
+                                            int, const WaveFilt<float>&, Chain);
 template cudaError_t launch_dwt2_inv<double>(const double*, int, size_t, const double*, int, double*, int, size_t,
-                                             int, int, const WaveFilt<double>&, cudaStream_t);
+                                             int, int, const WaveFilt<double>&, Chain);
 template int wave_fuse_band<float>(int);
 template int wave_fuse_band<double>(int);
 template cudaError_t launch_dwt2_fwd_fused<float>(const float*, int, size_t, float*, int, int, int,
-                                                  const WaveFilt<float>&, cudaStream_t);
+                                                  const WaveFilt<float>&, Chain);
 template cudaError_t launch_dwt2_fwd_fused<double>(const double*, int, size_t, double*, int, int, int,
-                                                   const WaveFilt<double>&, cudaStream_t);
+                                                   const WaveFilt<double>&, Chain);
 template cudaError_t launch_dwt2_inv_fused<float>(const float*, int, float*, int, size_t, int, int,
-                                                  const WaveFilt<float>&, cudaStream_t);
+                                                  const WaveFilt<float>&, Chain);
 template cudaError_t launch_dwt2_inv_fused<double>(const double*, int, double*, int, size_t, int, int,
-                                                   const WaveFilt<double>&, cudaStream_t);
+                                                   const WaveFilt<double>&, Chain);
 template cudaError_t launch_wdct_shrink<float>(float*, const ChanDCT<float>&, const float*, float*, float*, const float*,
-                                               double*, int, int, int, float, int, cudaStream_t);
+                                               double*, int, int, int, float, int, Chain);
 template cudaError_t launch_wdct_shrink<double>(double*, const ChanDCT<double>&, const double*, double*, double*,
-                                                const double*, double*, int, int, int, double, int, cudaStream_t);
+                                                const double*, double*, int, int, int, double, int, Chain);
 
 }  // namespace cip
