@@ -300,16 +300,27 @@ __device__ __forceinline__ C tw_at(const C* __restrict__ tw, int j, int N) {
 // the cancellation in b - W alpha turns that into 5e-5 of x at M = 8; four groups leave the 516 CTAs of
 // N = 256 in two waves (146 us an iteration against 134).  dl_solve + dl_filter + dl_spec before and now,
 // 256^2 x 5, L = 32, 11 x 11: 42 + 16 + 31 -> 36 + 14 + 18 us; an iteration 163 -> 136 us.
-constexpr int kDLGroups = 2, kDLThreads = kDLGroups * kDLBlock;
+// Where there are CTAs enough without the second group, one group is the faster: the second adds barriers, and
+// from M = 6 on no warps, since the registers of its threads leave half the CTAs on an SM.  Iterations, two groups
+// and one: complex64 512^2 x 8 with 9 filters 334 and 305 us, 512^2 x 6 261 and 227, 512^2 x 1 32 filters 256 and
+// 230, 256^2 x 8 93.2 and 81.5, but 256^2 x 7 32 filters 194 and 201, 512^2 x 3 428 and 439, 128^2 x 8 47.2 and 55.9;
+// complex128 512^2 x 3 1860 and 1816, 256^2 x 5 793 and 763, 128^2 x 5 254 and 302, 256^2 x 8 1186 and 1220.
+template <typename T> constexpr bool dl_one_group(int N, int M) {
+  if (sizeof(T) == 8) return N >= 512 || (N == 256 && M < 8);
+  return (N >= 512 && (M == 1 || M >= 6)) || (N == 256 && M == 8);
+}
 // resident CTAs the registers are held to: four keep the 516 CTAs of N = 256 in one wave
 template <typename T> constexpr int dl_blocks(int M, int PM) { return sizeof(T) == 4 ? (M <= 5 && PM <= 16 ? 4 : 2) : 1; }
-// filters whose operands a thread loads together (the registers of complex128 hold one)
-template <typename T> constexpr int dl_unroll() { return sizeof(T) == 4 ? 4 : 1; }
+// filters whose operands a thread loads together (the registers of complex128 hold one, or two of one group)
+template <typename T> constexpr int dl_unroll(int NG) { return sizeof(T) == 4 ? 4 : (NG == 1 ? 2 : 1); }
 // entries of the triangle of W^H W that group 0 takes beside b (M products) and W^H b (M products)
-constexpr int dl_first(int M) { return M * (M + 1) / 2 > 2 * M ? (M * (M + 1) / 2 - 2 * M) / 2 : 0; }
+constexpr int dl_first(int M, int NG) {
+  const int e = M * (M + 1) / 2;
+  return NG == 1 ? e : (e > 2 * M ? (e - 2 * M) / 2 : 0);
+}
 // elements of the region that holds the entries of group 1 and then the tile of w
-template <int M> constexpr int dl_part() {
-  constexpr int e = (M * (M + 1) / 2 - dl_first(M)) * kDLBlock, t = 32 * (kDLBlock + 1);
+template <int M, int NG> constexpr int dl_part() {
+  constexpr int e = (M * (M + 1) / 2 - dl_first(M, NG)) * kDLBlock, t = 32 * (kDLBlock + 1);
   return e > t ? e : t;
 }
 // acc[j] = sum over 32 bins k of w[j WS + k] E[k ES]: pairs at distance 16 first, then 8, 4, 2, 1 (the
@@ -339,10 +350,11 @@ __device__ __forceinline__ void dl_tree(const C* __restrict__ E, const C* __rest
     if ((t & 3) == 3) level(h1, (t & 4) == 0);
   }
 }
-template <typename T, int M, int PM>
-__global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kernel(const DLArgs<T> a) {
+template <typename T, int M, int PM, int NG>
+__global__ void __launch_bounds__(NG * kDLBlock, dl_blocks<T>(M, PM)) dl_solve_kernel(const DLArgs<T> a) {
   using C = typename CT<T>::type;
-  static_assert(kDLBlock == 64 && kDLGroups == 2, "two groups of two warps");
+  static_assert(kDLBlock == 64 && NG <= 2, "one or two groups of two warps");
+  constexpr int NT = NG * kDLBlock;
   const int N = a.N, L = a.L, P = a.P;
   const int CP = col_pitch(N), H = N / 2 + 1;
   const int grp = threadIdx.x / kDLBlock, bt = threadIdx.x - grp * kDLBlock;
@@ -355,11 +367,11 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
   C* E = reinterpret_cast<C*>(dsm);                // [kDLBlock][PM]: exp(+2 pi i k1 (a - P/2) / N)
   C* part = E + kDLBlock * PM;                     // [entries of group 1][kDLBlock] of W^H W, then
   C* wt = part;                                    // [32][kDLBlock + 1]: w of this CTA's bins
-  C* als = part + dl_part<M>();                    // [M][kDLBlock]: alpha
+  C* als = part + dl_part<M, NG>();                    // [M][kDLBlock]: alpha
   const C* zb = a.zcol + (size_t)k2 * M * L * CP + k1;  // z_{l,s} at zb[(s L + l) CP]
   const C* th = a.spec + (size_t)k2 * 2 * L * CP + k1;  // theta_l at th[l CP], F(g - e)_l at th[(L + l) CP]
   C x[M], c[M], G[M][M];
-  for (int i = tid; i < kDLBlock * PM; i += kDLThreads) {
+  for (int i = tid; i < kDLBlock * PM; i += NT) {
     const int ai = i % PM;
     E[i] = ai < P ? tw_at<+1>(a.tw, (kb * kDLBlock + i / PM) * (ai - P / 2), N) : mk<C>(0.0, 0.0);
   }
@@ -375,7 +387,7 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
   }
   // group 0: b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s, W^H b and the first E0 entries of the
   // triangle of W^H W; group 1: the others.  Each sum runs over all filters in order.
-  constexpr int E0 = dl_first(M);
+  constexpr int E0 = dl_first(M, NG);
   auto each = [&](auto f) {  // f(entry, s, t) over the triangle
 #pragma unroll
     for (int s = 0; s < M; ++s)
@@ -389,7 +401,7 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
       z[s] = mk<C>(v.x * n2, v.y * n2);
     }
   };
-  if (grp == 0) {
+  if (NG == 1 || grp == 0) {
 #pragma unroll 4
     for (int l = 0; l < L; ++l) {
       const C ge = th[(size_t)(L + l) * CP];
@@ -413,14 +425,14 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
       });
     }
   }
-  if (grp) {
+  if (NG > 1 && grp) {
     each([&](int e, int s, int t) {
       if (e >= E0) part[(e - E0) * kDLBlock + bt] = G[s][t];
     });
   }
   __syncthreads();
   C al[M];
-  if (grp == 0) {
+  if (NG == 1 || grp == 0) {
     each([&](int e, int s, int t) {
       if (e >= E0) G[s][t] = part[(e - E0) * kDLBlock + bt];
     });
@@ -476,13 +488,13 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
   const T isg = T(1) / sigma;
   C* wb = a.wcol + (size_t)k2 * L * CP + k1;
   // the operands of U filters are loaded together
-  constexpr int U = dl_unroll<T>();
+  constexpr int U = dl_unroll<T>(NG);
 #pragma unroll 1
-  for (int lb = grp; lb < L; lb += U * kDLGroups) {
+  for (int lb = grp; lb < L; lb += U * NG) {
     C z[U][M], ge[U], t[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int l = lb + u * kDLGroups;
+      const int l = lb + u * NG;
       if (l < L) {
 #pragma unroll
         for (int s = 0; s < M; ++s) z[u][s] = zb[((size_t)s * L + l) * CP];
@@ -492,7 +504,7 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int l = lb + u * kDLGroups;
+      const int l = lb + u * NG;
       if (l >= L) break;
       // b_l = sigma F(g - e)_l + sum_s conj(z_{l,s}) x_s, then d -= conj(z_s) alpha_s
       C d = mk<C>(sigma * ge[u].x, sigma * ge[u].y);
@@ -512,7 +524,7 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
   __syncthreads();
   // the support rows of the CTA's bins: thread = row a, filters l0, l0 + LSTEP, ...
   {
-    constexpr int LSTEP = kDLThreads / PM;
+    constexpr int LSTEP = NT / PM;
     const int ai = tid % PM;
     C* yp = a.ypart + ((size_t)k2 * nkb + kb) * L * P;
     auto rows = [&](auto nl) {
@@ -530,8 +542,9 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
         }
       }
     };
-    // as many at a time as few filters have (of the fixed four, L = 9 would compute 23 in vain)
-    if (L <= LSTEP) rows(std::integral_constant<int, 1>());
+    // as many at a time as few filters have (of the fixed four, L = 9 would compute 23 in vain); one in complex128,
+    // where rows computed in vain cost FP64 issue and reading E again does not (256^2 x 1, 9 filters: 339 -> 293 us)
+    if (sizeof(T) == 8 || L <= LSTEP) rows(std::integral_constant<int, 1>());
     else if (L <= 2 * LSTEP) rows(std::integral_constant<int, 2>());
     else rows(std::integral_constant<int, 4>());
   }
@@ -543,7 +556,7 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_solve_kern
   if (last) {
     __threadfence();
     const C* y0 = a.ypart + (size_t)k2 * nkb * L * P;
-    for (int i = tid; i < L * P; i += kDLThreads) {
+    for (int i = tid; i < L * P; i += NT) {
       C acc = mk<C>(0.0, 0.0);
       for (int b = 0; b < nkb; ++b) {
         const C v = __ldcg(y0 + (size_t)b * L * P + i);
@@ -678,8 +691,9 @@ __global__ void __launch_bounds__(kFiltThreads) dl_filter_kernel(const DLArgs<T>
 // primal residual |F(d - g)|^2 = |w - e-hat_old - g-hat|^2 (Parseval on the half spectrum).
 // The two groups divide the filters for g-hat, left in shared memory, and then the channels for p (each
 // p still a sum over all filters in order): 31 -> 18 us at 256^2 x 5, L = 32.
-template <typename T, int M, int PM>
-__global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kernel(const DLArgs<T> a) {
+template <typename T, int M, int PM, int NG>
+__global__ void __launch_bounds__(NG * kDLBlock, dl_blocks<T>(M, PM)) dl_spec_kernel(const DLArgs<T> a) {
+  constexpr int NT = NG * kDLBlock;
   using C = typename CT<T>::type;
   const int N = a.N, L = a.L, P = a.P, CP = col_pitch(N);
   const int tid = threadIdx.x, grp = tid / kDLBlock, bt = tid - grp * kDLBlock;
@@ -687,10 +701,10 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kerne
   extern __shared__ __align__(16) unsigned char dsm[];
   C* gk = reinterpret_cast<C*>(dsm);  // [32][PM]
   C* gs = gk + 32 * PM;               // [L][kDLBlock]: g-hat of this CTA's bins
-  __shared__ double red[kDLThreads / 32];
+  __shared__ double red[NT / 32];
   grid_dep_wait();
   grid_dep_launch();
-  for (int i = tid; i < 32 * PM; i += kDLThreads) {
+  for (int i = tid; i < 32 * PM; i += NT) {
     const int l = i / PM, ai = i - l * PM;
     gk[i] = (l < L && ai < P) ? a.gfac[((size_t)k2 * L + l) * P + ai] : mk<C>(0.0, 0.0);
   }
@@ -703,16 +717,16 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kerne
   C* th = a.spec + (size_t)k2 * 2 * L * CP + k1;
   const C* wb = a.wcol + (size_t)k2 * L * CP + k1;
   const C* zb = a.zcol + (size_t)k2 * M * L * CP + k1;
-  constexpr int U = dl_unroll<T>();
+  constexpr int U = dl_unroll<T>(NG);
 #pragma unroll 1
-  for (int lb = grp; lb < L; lb += U * kDLGroups) {
+  for (int lb = grp; lb < L; lb += U * NG) {
     C wl[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (lb + u * kDLGroups < L) wl[u] = wb[(size_t)(lb + u * kDLGroups) * CP];
+      if (lb + u * NG < L) wl[u] = wb[(size_t)(lb + u * NG) * CP];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int l = lb + u * kDLGroups;
+      const int l = lb + u * NG;
       if (l >= L) break;
       C gh = mk<C>(0.0, 0.0);
 #pragma unroll
@@ -736,8 +750,8 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kerne
     if ((tid & 31) == 0) red[tid >> 5] = v;
   }
   __syncthreads();
-  // p of channels grp, grp + kDLGroups, ...: each sum runs over all filters in order
-  constexpr int MG = (M + kDLGroups - 1) / kDLGroups;
+  // p of channels grp, grp + NG, ...: each sum runs over all filters in order
+  constexpr int MG = (M + NG - 1) / NG;
   C pm[MG];
 #pragma unroll
   for (int m = 0; m < MG; ++m) pm[m] = mk<C>(0.0, 0.0);
@@ -746,14 +760,14 @@ __global__ void __launch_bounds__(kDLThreads, dl_blocks<T>(M, PM)) dl_spec_kerne
     const C gh = gs[l * kDLBlock + bt];
 #pragma unroll
     for (int m = 0; m < MG; ++m)
-      if (grp + m * kDLGroups < M) cfma(pm[m], gh, zb[((size_t)(grp + m * kDLGroups) * L + l) * CP]);
+      if (grp + m * NG < M) cfma(pm[m], gh, zb[((size_t)(grp + m * NG) * L + l) * CP]);
   }
 #pragma unroll
   for (int m = 0; m < MG; ++m)
-    if (grp + m * kDLGroups < M) a.p_out[((size_t)k2 * M + grp + m * kDLGroups) * CP + k1] = pm[m];
+    if (grp + m * NG < M) a.p_out[((size_t)k2 * M + grp + m * NG) * CP + k1] = pm[m];
   if (a.check && tid == 0) {
     double v = 0.0;
-    for (int w = 0; w < kDLThreads / 32; ++w) v += red[w];
+    for (int w = 0; w < NT / 32; ++w) v += red[w];
     a.rpart[(size_t)k2 * gridDim.x + blockIdx.x] = v;
   }
 }
@@ -774,25 +788,28 @@ __global__ void dl_rescale_kernel(typename CT<T>::type* __restrict__ spec, int L
   }
 }
 
-template <typename T, int M, int PM> cudaError_t dl_launch(const DLArgs<T>& a, bool spec, Chain s) {
+template <typename T, int M, int PM, int NG> cudaError_t dl_launch(const DLArgs<T>& a, bool spec, Chain s) {
   using C = typename CT<T>::type;
-  const dim3 grid(a.N / kDLBlock, a.N / 2 + 1), block(kDLThreads);
-  constexpr size_t sm = (size_t)(kDLBlock * (PM + M) + dl_part<M>()) * sizeof(C);
+  const dim3 grid(a.N / kDLBlock, a.N / 2 + 1), block(NG * kDLBlock);
+  constexpr size_t sm = (size_t)(kDLBlock * (PM + M) + dl_part<M, NG>()) * sizeof(C);
   constexpr size_t spec_max = (size_t)32 * (PM + kDLBlock) * sizeof(C);
   static PerDeviceOnce once;
   cudaError_t e = once([&] {
-    cudaError_t r = cudaFuncSetAttribute(dl_solve_kernel<T, M, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t r = cudaFuncSetAttribute(dl_solve_kernel<T, M, PM, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (r != cudaSuccess) return r;
-    return cudaFuncSetAttribute(dl_spec_kernel<T, M, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spec_max);
+    return cudaFuncSetAttribute(dl_spec_kernel<T, M, PM, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spec_max);
   });
   if (e != cudaSuccess) return e;
-  if (spec) return launch_pdl(dl_spec_kernel<T, M, PM>, grid, block, (size_t)(32 * PM + a.L * kDLBlock) * sizeof(C), s, 0, a);
-  return launch_pdl(dl_solve_kernel<T, M, PM>, grid, block, sm, s, 0, a);
+  if (spec) return launch_pdl(dl_spec_kernel<T, M, PM, NG>, grid, block, (size_t)(32 * PM + a.L * kDLBlock) * sizeof(C), s, 0, a);
+  return launch_pdl(dl_solve_kernel<T, M, PM, NG>, grid, block, sm, s, 0, a);
 }
 template <typename T, int PM> cudaError_t dl_by_m(const DLArgs<T>& a, bool spec, Chain s) {
   switch (a.M) {
 #define DL_CASE(m) \
-  case m: return dl_launch<T, m, PM>(a, spec, s);
+  case m:                                                                                               \
+    if constexpr (dl_one_group<T>(256, m) || dl_one_group<T>(2048, m))                                   \
+      if (dl_one_group<T>(a.N, m)) return dl_launch<T, m, PM, 1>(a, spec, s);                            \
+    return dl_launch<T, m, PM, 2>(a, spec, s);
     DL_CASE(1) DL_CASE(2) DL_CASE(3) DL_CASE(4) DL_CASE(5) DL_CASE(6) DL_CASE(7) DL_CASE(8)
 #undef DL_CASE
     default: return cudaErrorInvalidValue;
