@@ -302,7 +302,8 @@ cip_status cip_get_launches(cip_plan* plan, unsigned long long* launches);
  * this is the autotuner's choice where it has one). */
 cip_status cip_get_prior_fft(cip_plan* plan, int* elems_per_thread);
 
-/* Launch configuration the plan uses (for reporting). */
+/* Launch configuration the plan uses (for reporting); column_pass: 1 = fused, with the ring or without (the
+ * autotuner decides between them), 2 = split. */
 cip_status cip_get_config(cip_plan* plan, int* rows_per_tile, int* col_tile, int* prior_pass_blocks,
                           int* column_pass_blocks, int* column_pass);
 

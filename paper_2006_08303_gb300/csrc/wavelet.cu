@@ -512,6 +512,11 @@ __global__ void __launch_bounds__(256) wdct_shrink_kernel(T* __restrict__ coef, 
   const bool import_mode = (flags & PA_IMPORT) != 0;
   const bool resid = (flags & PA_RESID) != 0;
   const bool store_t = (flags & PA_STORE_T) != 0;
+  // Nothing writes u_in while this grid is resident: in an iteration it is what the previous iteration's
+  // shrinkage wrote, complete before the kernel before this one could start; in an import a copy or a plainly launched
+  // kernel wrote it, complete before this grid started.  Said to the compiler, its loads move ahead of the stores
+  // of u_out: 512^2 x 10 114.2 -> 100.2 us an iteration, 1024^2 x 10 356 -> 303.
+  const T* __restrict__ ur = u_in;
   const size_t plane = (size_t)N * N;
   T part[kNPart] = {T(0), T(0), T(0), T(0), T(0)};
   for (size_t pix = (size_t)blockIdx.x * blockDim.x + threadIdx.x; pix < plane; pix += (size_t)gridDim.x * blockDim.x) {
@@ -525,7 +530,7 @@ __global__ void __launch_bounds__(256) wdct_shrink_kernel(T* __restrict__ coef, 
 #pragma unroll
         for (int m = 0; m < M; ++m) w = fma((T)cv[k * M + m], cin[m], w);
         const size_t g = (size_t)k * plane + pix;
-        const T uo = u_in[g];
+        const T uo = ur[g];
         T t, un;
         if (import_mode) {
           t = t_imp[g];
