@@ -36,7 +36,7 @@ METRIC = "ADMM voxel-iter/s"
 # the hash of the kernel sources the capture was taken from (kernel_sources_hash()).  The figure
 # is reported only while the sources still hash to that value (any change to a kernel makes it
 # null until the kernels are captured again) and only for the column pass of the captured form.
-TRAFFIC_CAPTURE = {"sources": "d5c303207c8ee882", "bytes": {"column_pass": 81.26e6, "prior_pass": 21.07e6}}
+TRAFFIC_CAPTURE = {"sources": "125c99ee1e97ecf2", "bytes": {"column_pass": 81.44e6, "prior_pass": 21.06e6}}
 KERNEL_UNITS = ("colpass.cu", "passA.cu")  # of the two captured kernels
 CAPTURED_FORM = "fused"                    # column-pass form captured (colpass_fused_kernel)
 
