@@ -13,9 +13,10 @@
 // device with other plans' (batches, the server) run the faster of the ring kernel and the split form
 // instead (8 TV plans of 1024^2 x 3 in a batch: split 337 us an iteration of all, ring 369; of 1024^2 x 1
 // 147 and 225).
-// One iteration, ring -> this kernel: 64^2 x 3 TV 5.71 -> 5.05 us, 256^2 x 3 8.86 -> 8.15, 512^2 x 5 24.5 ->
-// 22.7, 1024^2 x 3 50.2 (split) -> 48.7; 16 plans of 128^2 .. 512^2 in a batch 8.38 -> 9.0 ms.  With 10
-// channels at 512^2 (whose slots leave room for three rows ahead) 37.1 -> 37.8: not offered.
+// One TV iteration, the faster of ring and split -> this kernel: 64^2 x 3 5.97 (ring) -> 5.04 us, 256^2 x 3 8.92
+// (ring) -> 7.93, 512^2 x 5 25.7 (ring) -> 22.9, 1024^2 x 3 57.4 (split) -> 46.7, 1024^2 x 1 26.8 (split) -> 22.6; 16
+// plans of 128^2 .. 512^2 in a batch 8.38 -> 9.0 ms.  With 10 channels at 512^2 (whose slots leave room for three
+// rows ahead) 37.1 -> 37.8: not offered.
 #include "colteam.cuh"
 #include "kernels.h"
 
