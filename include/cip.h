@@ -79,11 +79,11 @@ typedef struct cip_options {
                        half-spectrum column per CTA */
   int check_every;  /* residual check period for cip_iterate with tol > 0; 0 = 10 */
   int column_pass;  /* 0 = autotuned at cip_set_measurements (fused vs split, tile width; cached per
-                       N, M, dtype and prior, for dictionaries also the number of maps M L, for the process,
+                       N, M, dtype and prior, for dictionaries also 2D or 3D and the number of maps M L, for the process,
                        and in the file named by the environment
                        variable CIP_TUNE_CACHE when set, one "N M dtype prior mode cc variant recorded maps" line per
-                       decision, read on first use; maps = M L on dictionaries' lines only (a line without it
-                       holds for every number of filters); mode 1 and 3 = fused with and without the factor's ring, 2 =
+                       decision, read on first use; maps = M L, or -M L for 3D dictionaries, on dictionaries' lines only
+                       (a line without it holds for every dictionary); mode 1 and 3 = fused with and without the factor's ring, 2 =
                        split; recorded = the mode, 1 or 2, of iterations in a batch or on the server, which a
                        line may leave out: then mode, or 1 where that is 3), 1 = fused kernel (one CTA per half-spectrum column, factor
                        streamed by TMA bulk copies; CIP_ERR_UNSUPPORTED where its tile does not fit

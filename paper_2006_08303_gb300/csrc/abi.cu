@@ -770,8 +770,10 @@ template <typename T> cip_status column_pass(cip_plan* p, cudaStream_t stream, i
 std::mutex g_tune_mu;
 // (N, M, dtype, prior, maps of a dictionary's prior pass, forced prior-pass variant or -1) -> (column-pass
 // form, fused tile width, prior-pass variant, column-pass form of recorded iterations).  Maps: M L for
-// dictionaries, whose row pass runs over them and fills the device or not; 0 for the other priors (M says it)
-// and in a line of the file that names none, which then holds for every number of filters.
+// dictionaries, whose row pass runs over them and fills the device or not, and -M L for 3D ones, whose column
+// pass overlaps it otherwise (32 maps of 256^2, widths 8 and 16: 2D 28.8 and 22.0 us an iteration, 3D 31.5 and 35.9);
+// 0 for the other priors (M says it) and in a line of the file that names none, which then holds for every
+// dictionary.
 using TuneKey = std::tuple<int, int, int, int, int, int>;
 using TuneVal = std::tuple<int, int, int, int>;
 std::map<TuneKey, TuneVal> g_tune;
@@ -801,7 +803,7 @@ void tune_cache_store(const TuneKey& key, const TuneVal& v) {
   std::ofstream out(path, std::ios::app);
   out << std::get<0>(key) << ' ' << std::get<1>(key) << ' ' << std::get<2>(key) << ' ' << std::get<3>(key) << ' '
       << std::get<0>(v) << ' ' << std::get<1>(v) << ' ' << std::get<2>(v) << ' ' << std::get<3>(v);
-  if (std::get<4>(key) > 0) out << ' ' << std::get<4>(key);
+  if (std::get<4>(key) != 0) out << ' ' << std::get<4>(key);
   out << '\n';
 }
 
@@ -854,7 +856,7 @@ template <typename T> cip_status autotune(cip_plan* p, cudaStream_t s) {
   using C = typename CT<T>::type;
   const int fav = forced_avar(p);
   const int kfav = prior_has_variant(p) ? fav : -1;
-  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, is_cd(p) ? smaps(p) : 0, kfav);
+  const TuneKey key = std::make_tuple(p->N, p->M, (int)p->dtype, p->prior, is_cd(p) ? (p->Q > 0 ? -smaps(p) : smaps(p)) : 0, kfav);
   if (low_fix(p)) {  // the low-column correction of large TV plans is part of the split form
     set_colmode<T>(p, 2, p->cc);
     if (!p->colbuf) CIP_CUDA(p, dmalloc(p, &p->colbuf, col_elems(p, p->M) * sizeof(C)));

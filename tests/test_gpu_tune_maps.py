@@ -1,4 +1,4 @@
-"""Autotuner decisions of dictionary plans are kept per number of maps M L: the row pass of one filter and of 32
+"""Autotuner decisions of dictionary plans are kept per number of maps M L and for 2D and 3D apart: the row pass of one filter and of 32
 fill the device differently, so a plan's width must not depend on which plan came first.  GPU only; the
 decisions go through the tuning file, in processes of their own."""
 import os
@@ -34,19 +34,19 @@ def run(code, cache):
 def test_each_number_of_maps_has_its_own_decision(tmp_path):
     f = tmp_path / "tune.txt"
     # N M dtype prior form tile variant recorded [maps]; widths of the variants 0, 1, 2: 8, 16, 32
-    f.write_text("256 2 0 3 1 1 0 1 4\n256 2 0 3 1 1 1 1 10\n256 2 0 3 1 1 2 1\n")
+    f.write_text("256 2 0 3 1 1 0 1 4\n256 2 0 3 1 1 1 1 10\n256 2 0 3 1 1 0 1 -10\n256 2 0 3 1 1 2 1\n")
     run("""
-assert [width(plan(L)) for L in (2, 5, 3)] == [8, 16, 32]  # the last one: a line for any number of filters
-assert width(plan(5, Q=2)) == 16
+assert [width(plan(L)) for L in (2, 5, 3)] == [8, 16, 32]  # the last one: a line for any dictionary
+assert width(plan(5, Q=2)) == 8 and width(plan(3, Q=2)) == 32  # -10: the 3D dictionary of 10 maps
 """, f)
-    assert len(f.read_text().splitlines()) == 3
+    assert len(f.read_text().splitlines()) == 4
 
 
 def test_the_autotuner_keeps_a_decision_per_number_of_maps(tmp_path):
     f = tmp_path / "tune.txt"
     run("""
-a, b, c = plan(1), plan(32), plan(1)
+a, b, c, d = plan(1), plan(32), plan(1), plan(32, Q=2)
 assert width(a) == width(c)
 """, f)
     lines = [list(map(int, s.split())) for s in f.read_text().splitlines()]
-    assert sorted(n[8] for n in lines) == [2, 64], lines
+    assert sorted(n[8] for n in lines) == [-64, 2, 64], lines
